@@ -36,8 +36,8 @@
 //   one tile holds both halves).
 // No partial sum leaves the chip and no separate kernel runs. Consumers of a
 // split pre-norm scale each token column by its RMSNorm factor first. With one
-// split (prefill) the CTA reads its own tile with plain shared loads and may
-// stage it in 128-column windows, so two CTAs share an SM.
+// split the CTA reads its own tile with plain shared loads. Prefill chunks of up
+// to 256 rows come here too; larger ones take k_gemm_pf.
 //
 // Other epilogues (SIMT path, LM head): split-K partial sums to a buffer
 // consumed by k_rope_append / k_swiglu, atomic residual add + scatter, or a
@@ -75,11 +75,9 @@ constexpr int TC_STAGES = 4;  // deepest operand ring; a launch uses min(4, k-ti
 // operand (lo) a stage holds 2 x NT token rows.
 constexpr int tc_b_bytes(int nt, bool lo) { return (lo ? 2 : 1) * nt * TC_BK * 2; }
 constexpr int tc_ring_bytes(int nt, int stages, bool lo) { return stages * (TC_BM * TC_BK * 2 + tc_b_bytes(nt, lo)); }
-constexpr int tc_red_bytes(int red_cols) { return TC_BM * red_cols * 4; }
-// red_cols: token columns of the staged fp32 tile (nt, or the window of a one-split epilogue)
-constexpr int tc_body_bytes(int nt, int stages, bool lo, int red_cols) {
-  return tc_ring_bytes(nt, stages, lo) > tc_red_bytes(red_cols) ? tc_ring_bytes(nt, stages, lo)
-                                                                : tc_red_bytes(red_cols);
+constexpr int tc_red_bytes(int nt) { return TC_BM * nt * 4; }
+constexpr int tc_body_bytes(int nt, int stages, bool lo) {
+  return tc_ring_bytes(nt, stages, lo) > tc_red_bytes(nt) ? tc_ring_bytes(nt, stages, lo) : tc_red_bytes(nt);
 }
 // TMEM columns of one CTA: the accumulator of 2 x NT columns (hi and lo halves) with a
 // two-term operand, NT otherwise, at least 32 (always a power of two).
@@ -91,9 +89,8 @@ constexpr int tc_tmem_cols(int nt, bool lo) {
 // partners could wait on each other): launches request at least this much.
 constexpr int SM_SMEM = 232448;  // shared memory per SM available to CTAs (227 KB + 1 KB per CTA)
 constexpr int tc_min_smem(int nt, bool lo) { return SM_SMEM / (512 / tc_tmem_cols(nt, lo) + 1) - 1024 + 1; }
-constexpr int tc_smem_bytes(int nt, int stages, bool lo, int red_cols = 0) {
-  const int raw = 1024 /*align slack*/ + tc_body_bytes(nt, stages, lo, red_cols > 0 ? red_cols : nt) +
-                  256 /*barriers, tmem slot*/ +
+constexpr int tc_smem_bytes(int nt, int stages, bool lo) {
+  const int raw = 1024 /*align slack*/ + tc_body_bytes(nt, stages, lo) + 256 /*barriers, tmem slot*/ +
                   nt * (16 + 4 + 16);
   return raw > tc_min_smem(nt, lo) ? raw : tc_min_smem(nt, lo);
 }
@@ -123,13 +120,12 @@ constexpr int CL_MAX = 8;  // largest cluster (split-K factor) of the cluster ep
 // Sums over the cluster of the staged values at feature f, columns c..c+3
 // (columns >= c1 give 0). All partner loads of the four columns are issued
 // before any is used.
-// With one split (prefill) the CTA's own staged tile is read with plain shared loads; it may
-// hold the window of columns starting at roff.
-__device__ __forceinline__ void cluster_sum4(const uint32_t* pb, const float* red, int roff, int S, int f, int c,
-                                             int c1, float out[4]) {
+// With one split the CTA's own staged tile is read with plain shared loads.
+__device__ __forceinline__ void cluster_sum4(const uint32_t* pb, const float* red, int S, int f, int c, int c1,
+                                             float out[4]) {
   if (S == 1) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) out[q] = (c + q < c1) ? red[(c + q - roff) * 128 + f] : 0.f;
+    for (int q = 0; q < 4; ++q) out[q] = (c + q < c1) ? red[(c + q) * 128 + f] : 0.f;
     return;
   }
   float v[CL_MAX][4];
@@ -160,13 +156,10 @@ __device__ __forceinline__ void cluster_cols(int n, int S, int& c0, int& c1) {
 
 template <int NT>
 __device__ void cluster_epilogue(const GemmArgs& a, float* red, int4* ci, const float* scale, float* ssp,
-                                 const float (&hpre)[HPRE], int m0, int n, int tok0, int cw0, int cw1) {
+                                 const float (&hpre)[HPRE], int m0, int n) {
   const int S = a.splits;
   int c0, c1;
   cluster_cols(n, S, c0, c1);
-  // columns of this pass: the CTA's share within the staged window [cw0, cw1) (the whole share
-  // unless a one-split epilogue stages in windows; the split-norm path is never windowed)
-  const int w0 = c0 > cw0 ? c0 : cw0, w1 = c1 < cw1 ? c1 : cw1;
   const int tid = threadIdx.x;
   uint32_t pb[CL_MAX];
   const uint32_t base = smem_u32(red);
@@ -177,12 +170,12 @@ __device__ void cluster_epilogue(const GemmArgs& a, float* red, int4* ci, const 
     const int col = m0 + tid;
     if (!a.xn) {
       if (col < a.N)
-        for (int c = w0; c < w1; c += 4) {
+        for (int c = c0; c < c1; c += 4) {
           float sm[4];
-          cluster_sum4(pb, red, cw0, S, tid, c, w1, sm);
+          cluster_sum4(pb, red, S, tid, c, c1, sm);
 #pragma unroll
           for (int q = 0; q < 4; ++q)
-            if (c + q < w1 && ci[c + q].w >= 0) {  // the only writer of this element
+            if (c + q < c1 && ci[c + q].w >= 0) {  // the only writer of this element
               const float g = a.alpha.mod ? a.alpha.mod[ci[c + q].x + col] : 1.f;
               atomicAdd(a.resid + (size_t)ci[c + q].w * a.ldr + col, g * sm[q]);
             }
@@ -227,7 +220,7 @@ __device__ void cluster_epilogue(const GemmArgs& a, float* red, int4* ci, const 
     if (c1 - c0 <= HPRE) {
       float sm[HPRE];
 #pragma unroll
-      for (int q = 0; q < HPRE; q += 4) cluster_sum4(pb, red, 0, S, tid, c0 + q, c1, sm + q);
+      for (int q = 0; q < HPRE; q += 4) cluster_sum4(pb, red, S, tid, c0 + q, c1, sm + q);
       float t[HPRE];
 #pragma unroll
       for (int q = 0; q < HPRE; ++q) t[q] = (c0 + q < c1) ? update(c0 + q, hpre[q], sm[q]) : 0.f;
@@ -241,7 +234,7 @@ __device__ void cluster_epilogue(const GemmArgs& a, float* red, int4* ci, const 
           hv[q] = (fin && c + q < c1) ? a.resid[(size_t)(w >= 0 ? w : ~w) * a.ldr + col] : 0.f;
         }
         float sm[4];
-        cluster_sum4(pb, red, 0, S, tid, c, c1, sm);
+        cluster_sum4(pb, red, S, tid, c, c1, sm);
         float t[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) t[q] = (c + q < c1) ? update(c + q, hv[q], sm[q]) : 0.f;
@@ -258,16 +251,16 @@ __device__ void cluster_epilogue(const GemmArgs& a, float* red, int4* ci, const 
   }
   // With a pair of rows per output (gate and up, or the two halves of a rotary pair), the
   // threads of the pair's upper row take the second half of the token columns.
-  const int cm = w0 + (w1 - w0 + 1) / 2;
+  const int cm = c0 + (c1 - c0 + 1) / 2;
   if (a.epi == EPI_CL_SWIGLU) {
     const int f = tid & 63, hs = tid >> 6;
     const int gf = (m0 >> 1) + f;  // 64 gate rows then 64 up rows per 128-row tile
-    const int ca = hs ? cm : w0, cb = hs ? w1 : cm;
+    const int ca = hs ? cm : c0, cb = hs ? c1 : cm;
     if (gf < a.md.ff)
       for (int c = ca; c < cb; c += 4) {
         float g[4], u[4];
-        cluster_sum4(pb, red, cw0, S, f, c, cb, g);
-        cluster_sum4(pb, red, cw0, S, f + 64, c, cb, u);
+        cluster_sum4(pb, red, S, f, c, cb, g);
+        cluster_sum4(pb, red, S, f + 64, c, cb, u);
 #pragma unroll
         for (int q = 0; q < 4; ++q)
           if (c + q < cb) {
@@ -275,24 +268,22 @@ __device__ void cluster_epilogue(const GemmArgs& a, float* red, int4* ci, const 
             const float gq = g[q] * f;
             const float y = gq / (1.f + expf(-gq)) * (u[q] * f);
             const bf16 yh = __float2bfloat16_rn(y);
-            const size_t at = (size_t)(tok0 + c + q) * a.md.ff + gf;
+            const size_t at = (size_t)(c + q) * a.md.ff + gf;
             reinterpret_cast<bf16*>(a.U)[at] = yh;
             if (a.U_lo) reinterpret_cast<bf16*>(a.U_lo)[at] = __float2bfloat16_rn(y - __bfloat162float(yh));
           }
       }
     return;
   }
-  // EPI_CL_QKV: column c is token k = tok0 + c of A_r
+  // EPI_CL_QKV: column c is token c of A_r
   const ModelDims& md = a.md;
   const StepDev& s = a.s;
   const int ps = md.page_size, hd = md.hd, half = hd / 2;
-  if (a.row_cslot && cw0 == 0) {
-    // prefill: sequence slot, cache slot and position of each row from the prefill plan (once, in
-    // the first window)
+  if (a.row_cslot) {
+    // prefill: sequence slot, cache slot and position of each row from the prefill plan
     for (int c = c0 + tid; c < c1; c += blockDim.x) {
-      const int row = tok0 + c;
-      const int slot = a.row_slot[row], L = a.row_cslot[row];
-      int pos = a.row_pos[row];
+      const int slot = a.row_slot[c], L = a.row_cslot[c];
+      int pos = a.row_pos[c];
       int page = s.page_table[((size_t)slot * md.M + a.r) * md.max_pages + L / ps];
       if (page < 0 || page >= md.n_pages || pos < 0 || pos >= md.max_pos) {
         atomicOr(s.err, DEVERR_INDEX);
@@ -314,15 +305,15 @@ __device__ void cluster_epilogue(const GemmArgs& a, float* red, int4* ci, const 
     const int h = fr / hd, hs = (fr % hd) >= half;
     const int i = (fr % hd) - hs * half;   // rotary pair (i, i + half) of head h
     const int tlo = tid - hs * half;       // tile row of the pair's lower element
-    const int ca = hs ? cm : w0, cb = hs ? w1 : cm;
+    const int ca = hs ? cm : c0, cb = hs ? c1 : cm;
     for (int c = ca; c < cb; c += 4) {
       float2 csn[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q)
         csn[q] = (c + q < cb) ? a.rope[(size_t)ci[c + q].z * half + i] : make_float2(1.f, 0.f);
       float x0[4], x1[4];
-      cluster_sum4(pb, red, cw0, S, tlo, c, cb, x0);
-      cluster_sum4(pb, red, cw0, S, tlo + half, c, cb, x1);
+      cluster_sum4(pb, red, S, tlo, c, cb, x0);
+      cluster_sum4(pb, red, S, tlo + half, c, cb, x1);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int cc = c + q;
@@ -333,7 +324,7 @@ __device__ void cluster_epilogue(const GemmArgs& a, float* red, int4* ci, const 
         }
         const float r0 = x0[q] * csn[q].x - x1[q] * csn[q].y, r1 = x0[q] * csn[q].y + x1[q] * csn[q].x;
         if (is_q) {
-          float* qo = a.Q + ((size_t)(tok0 + cc) * md.Hq + h) * hd;
+          float* qo = a.Q + ((size_t)cc * md.Hq + h) * hd;
           qo[i] = r0;
           qo[i + half] = r1;
         } else {
@@ -350,13 +341,13 @@ __device__ void cluster_epilogue(const GemmArgs& a, float* red, int4* ci, const 
   } else {
     const int fr = gfeat - md.q_dim - md.kv_dim;
     const int h = fr / hd, i = fr % hd;
-    for (int c = w0; c < w1; c += 4) {
+    for (int c = c0; c < c1; c += 4) {
       float x[4];
-      cluster_sum4(pb, red, cw0, S, tid, c, w1, x);
+      cluster_sum4(pb, red, S, tid, c, c1, x);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int cc = c + q;
-        if (cc < w1 && ci[cc].x >= 0) {
+        if (cc < c1 && ci[cc].x >= 0) {
           bf16* vp = pool + (size_t)ci[cc].x * md.page_elems + ((size_t)(a.j * 2 + 1) * md.Hkv + h) * ps * hd +
                      (size_t)ci[cc].y * hd;
           vp[i] = __float2bfloat16_rn(a.ss_in ? x[q] * scale[cc] : x[q]);
@@ -391,9 +382,7 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const __grid_constant__ CUtenso
   const int NS = a.stages;  // 1..TC_STAGES
   uint8_t* sA = smem;
   uint8_t* sB = smem + NS * A_BYTES;
-  // one-split epilogues may stage the tile in windows of red_window columns (smaller smem)
-  const int RW = (a.red_window > 0 && a.splits == 1 && a.red_window < NT) ? a.red_window : NT;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + tc_body_bytes(NT, NS, lo, RW));
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + tc_body_bytes(NT, NS, lo));
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * TC_STAGES + 1);
   int4* colinfo = reinterpret_cast<int4*>(reinterpret_cast<uint8_t*>(bars) + 256);  // [NT]
   float* colscale = reinterpret_cast<float*>(colinfo + NT);                          // [NT]
@@ -403,14 +392,12 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const __grid_constant__ CUtenso
   // The token count comes from the plan kernel, which completed before this
   // grid was launched (every kernel triggers its successor only after its own
   // wait), so it is read before pdl_wait(), bypassing L1.
-  const int n_all = a.n_dev ? __ldcg(a.n_dev) : a.n_host;
-  const int tok0 = blockIdx.z * NT;  // token tile of this CTA (prefill has many)
-  if (n_all <= tok0) {
+  const int n = min(NT, a.n_dev ? __ldcg(a.n_dev) : a.n_host);  // token columns
+  if (n <= 0) {
     pdl_wait();
     pdl_trigger();
     return;
   }
-  const int n = min(NT, n_all - tok0);      // token columns of this tile
   const int ncols = ((n + 15) / 16) * 16;  // MMA N: multiple of 16, <= NT
   const int m0 = blockIdx.x * TC_BM;
   const int split = blockIdx.y;
@@ -445,9 +432,8 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const __grid_constant__ CUtenso
   if (warp == 0 && lane == 0) {
     // TMA producer. Weight tiles of the first stages go out before the wait on
     // the preceding kernels (weights are never written by them); token tiles after.
-    // decode reads each weight tile once per launch (streamed, evicted first); prefill's token
-    // tiles share them
-    const uint64_t w_policy = gridDim.z == 1 ? l2_policy_evict_first() : l2_policy_evict_normal();
+    // each weight tile is read once per launch: streamed, evicted first
+    const uint64_t w_policy = l2_policy_evict_first();
     const int pre = nk < NS ? nk : NS;
     for (int i = 0; i < pre; ++i) {
       mbar_arrive_expect_tx(full(i), A_BYTES + B_BYTES);
@@ -457,8 +443,8 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const __grid_constant__ CUtenso
     pdl_trigger();
     // token tiles; a two-term operand adds its lo plane (a.blo rows down) as rows NT..2NT-1
     auto load_x = [&](int st, int kx) {
-      tma_load_2d(smem_u32(sB + st * B_BYTES), &mapX, kx, tok0, full(st));
-      if (lo) tma_load_2d(smem_u32(sB + st * B_BYTES + NT * TC_BK * 2), &mapX, kx, tok0 + a.blo, full(st));
+      tma_load_2d(smem_u32(sB + st * B_BYTES), &mapX, kx, 0, full(st));
+      if (lo) tma_load_2d(smem_u32(sB + st * B_BYTES + NT * TC_BK * 2), &mapX, kx, a.blo, full(st));
     };
     for (int i = 0; i < pre; ++i) load_x(i, (kb0 + i) * TC_BK);
     for (int i = pre; i < nk; ++i) {
@@ -479,7 +465,7 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const __grid_constant__ CUtenso
       for (int c = threadIdx.x - 64; c < n; c += 64) {
         if (a.ss_in) {
           // split norm: the column's factor from the producer's per-tile sums of squares
-          const float4* p4 = reinterpret_cast<const float4*>(a.ss_in + (size_t)(tok0 + c) * a.ldss);
+          const float4* p4 = reinterpret_cast<const float4*>(a.ss_in + (size_t)c * a.ldss);
           float t = 0.f;
 #pragma unroll 4
           for (int k = 0; k < a.ldss / 4; ++k) {
@@ -489,17 +475,17 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const __grid_constant__ CUtenso
           colscale[c] = rsqrtf(t / (float)a.K + a.norm_eps);
         }
         if (a.epi == EPI_CL_QKV && !a.row_cslot) {
-          colinfo[c] = a.s.rowinfo[a.r * a.md.max_batch + tok0 + c];
+          colinfo[c] = a.s.rowinfo[a.r * a.md.max_batch + c];
         } else if (a.epi == EPI_CL_RESID) {
           // residual row, ~row for a row masked by the no-gather ablation (residual unchanged);
           // with time/step conditioning, the offset of the row's gate vector in the table;
           // with a split norm, the row's column in the next operand and its conditioning offset
-          const int row = a.idx ? a.idx[tok0 + c] : tok0 + c;
-          const bool masked = a.act && !a.act[tok0 + c];
+          const int row = a.idx ? a.idx[c] : c;
+          const bool masked = a.act && !a.act[c];
           const int aoff = (a.alpha.mod && !masked) ? (int)(cond_row(a.alpha, row) - a.alpha.mod) : 0;
           int goff = 0, dst = -1;
           if (a.xn) {
-            dst = a.next_col ? a.next_col[row] : tok0 + c;
+            dst = a.next_col ? a.next_col[row] : c;
             if (a.gamma.mod && dst >= 0) goff = (int)(cond_row(a.gamma, row) - a.gamma.mod);
           }
           colinfo[c] = make_int4(aoff, goff, dst, masked ? ~row : row);
@@ -550,7 +536,7 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const __grid_constant__ CUtenso
 #pragma unroll
       for (int q = 0; q < HPRE; ++q)
         if (c0 + q < c1) {
-          const int row = a.idx ? a.idx[tok0 + c0 + q] : tok0 + c0 + q;
+          const int row = a.idx ? a.idx[c0 + q] : c0 + q;
           hpre[q] = a.resid[(size_t)row * a.ldr + col];
         }
     }
@@ -567,28 +553,24 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const __grid_constant__ CUtenso
     // tile layout [column][128 features]: a warp's partner reads are 128 contiguous bytes
     float* red = reinterpret_cast<float*>(smem);
     const int f = warp * 32 + lane;
-    for (int w = 0; w < ncols; w += RW) {  // one pass unless a one-split tile is staged in windows
-      const int wend = w + RW < ncols ? w + RW : ncols;
-      if (w > 0) __syncthreads();  // every thread is done with the previous window
-      for (int c0 = w; c0 < wend; c0 += 16) {
-        float v[16];
-        if (ok && nk > 0) {
-          tmem_ld_acc(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, lo ? NT : 0, v);
-        } else {
+    for (int c0 = 0; c0 < ncols; c0 += 16) {
+      float v[16];
+      if (ok && nk > 0) {
+        tmem_ld_acc(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, lo ? NT : 0, v);
+      } else {
 #pragma unroll
-          for (int i = 0; i < 16; ++i) v[i] = 0.f;
-        }
-#pragma unroll
-        for (int i = 0; i < 16; ++i) red[(c0 - w + i) * 128 + f] = v[i];
+        for (int i = 0; i < 16; ++i) v[i] = 0.f;
       }
-      tc_fence_before();
-      __syncthreads();
-      if (wend == ncols && warp == 0) tmem_dealloc(tmem, TMEM_COLS);
-      cluster_sync_all();  // every partner's tile is staged
-      cluster_epilogue<NT>(a, red, colinfo, colscale, ssp, hpre, m0, n, tok0, w, w + RW);
-      __syncwarp();
-      cluster_sync_all();  // partners have finished reading this CTA's tile
+#pragma unroll
+      for (int i = 0; i < 16; ++i) red[(c0 + i) * 128 + f] = v[i];
     }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tmem, TMEM_COLS);
+    cluster_sync_all();  // every partner's tile is staged
+    cluster_epilogue<NT>(a, red, colinfo, colscale, ssp, hpre, m0, n);
+    __syncwarp();
+    cluster_sync_all();  // partners have finished reading this CTA's tile
     return;
   }
   if (ok) {
@@ -604,7 +586,7 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const __grid_constant__ CUtenso
       if (col < a.N) {
 #pragma unroll
         for (int i = 0; i < 16; ++i)
-          if (c0 + i < n && (nk > 0 || a.epi == EPI_PARTIAL)) gemm_write(a, split, tok0 + c0 + i, col, v[i]);
+          if (c0 + i < n && (nk > 0 || a.epi == EPI_PARTIAL)) gemm_write(a, split, c0 + i, col, v[i]);
       }
     }
   }
@@ -628,17 +610,8 @@ static void launch_tc_nt(const CUtensorMap* mapW, const CUtensorMap* mapX, GemmA
   // (a failure shows at launch)
   (void)ensure_kernel_attrs((const void*)k_gemm_tc<NT, LO>, tc_smem_bytes(NT, tc_max_stages(NT, LO), LO));
   a.stages = gemm_tc_stages(a.K, a.splits, NT, LO);
-  int red_cols = NT;
-  if (a.red_window > 0 && a.splits == 1 && a.red_window < NT) {
-    // windowed one-split epilogue: with a 2-stage ring two CTAs share an SM, so one CTA's
-    // epilogue overlaps the other's main loop
-    red_cols = a.red_window;
-    if (a.stages > 2) a.stages = 2;
-  } else {
-    a.red_window = 0;
-  }
-  const int smem = tc_smem_bytes(NT, a.stages, LO, red_cols);
-  dim3 grid((a.N + TC_BM - 1) / TC_BM, a.splits, a.tok_tiles > 0 ? a.tok_tiles : 1);
+  const int smem = tc_smem_bytes(NT, a.stages, LO);
+  dim3 grid((a.N + TC_BM - 1) / TC_BM, a.splits);
   if (a.epi < EPI_CL_RESID) {
     launch_k(k_gemm_tc<NT, LO>, grid, 128, smem, st, *mapW, *mapX, a);
     return;

@@ -41,7 +41,8 @@ thread_local std::string g_create_error = "no error";
 struct DeviceMat {
   void* ptr = nullptr;
   int N = 0, K = 0;
-  CUtensorMap map;
+  CUtensorMap map;               // boxes of 128 rows
+  CUtensorMap map64, map32;      // boxes of 64 and 32 rows (narrower tiles of the prefill GEMM)
 };
 }  // namespace
 
@@ -132,7 +133,9 @@ struct tlf_ctx {
   float* d_pf_Q = nullptr;
   void* d_pf_O = nullptr;
   void* d_pf_U = nullptr;
-  CUtensorMap pf_map_X, pf_map_O, pf_map_U;
+  CUtensorMap pf_map_X, pf_map_O, pf_map_U;     // boxes of 256 rows
+  CUtensorMap pf_pair_X, pf_pair_O, pf_pair_U;  // boxes of 128 rows
+  int pf_pairs = 0;                             // SM pairs the prefill GEMM's persistent grid may fill
   int *d_pf_idx = nullptr, *d_pf_n = nullptr, *d_pf_row_slot = nullptr, *d_pf_row_cslot = nullptr,
       *d_pf_row_pos = nullptr, *d_pf_first = nullptr, *d_pf_cnt = nullptr, *d_pf_s0 = nullptr,
       *d_pf_tile_base = nullptr;
@@ -344,7 +347,8 @@ static int make_mat(tlf_ctx* ctx, DeviceMat* m, const std::vector<const uint8_t*
   if (rc) return rc;
   m->N = N;
   m->K = K;
-  if (ctx->use_tc && !make_map(&m->map, m->ptr, N, K, K, 128))
+  if (ctx->use_tc && (!make_map(&m->map, m->ptr, N, K, K, 128) || !make_map(&m->map64, m->ptr, N, K, K, 64) ||
+                      !make_map(&m->map32, m->ptr, N, K, K, 32)))
     return fail(ctx, TLF_ERR_CUDA, "cuTensorMapEncodeTiled failed for %s", what);
   return TLF_OK;
 }
@@ -1132,38 +1136,38 @@ static int ensure_prefill_buffers(tlf_ctx* ctx) {
   CK(ctx, cudaMemset(ctx->d_pf_U, 0, (size_t)C * md.ff * 2));
   if (!make_map(&ctx->pf_map_X, ctx->d_pf_X, C, d, d, 256) ||
       !make_map(&ctx->pf_map_O, ctx->d_pf_O, C, md.q_dim, md.q_dim, 256) ||
-      !make_map(&ctx->pf_map_U, ctx->d_pf_U, C, md.ff, md.ff, 256))
+      !make_map(&ctx->pf_map_U, ctx->d_pf_U, C, md.ff, md.ff, 256) ||
+      !make_map(&ctx->pf_pair_X, ctx->d_pf_X, C, d, d, 128) ||
+      !make_map(&ctx->pf_pair_O, ctx->d_pf_O, C, md.q_dim, md.q_dim, 128) ||
+      !make_map(&ctx->pf_pair_U, ctx->d_pf_U, C, md.ff, md.ff, 128))
     return fail(ctx, TLF_ERR_CUDA, "cuTensorMapEncodeTiled failed for a prefill buffer");
+  ctx->pf_pairs = gemm_pf_max_pairs(ctx->num_sms);
+  if (ctx->pf_pairs < 1) return fail(ctx, TLF_ERR_CUDA, "the prefill GEMM's clusters cannot be launched on this device");
   ctx->pf_C = C;
   ctx->pf_Smax = Smax;
   return TLF_OK;
 }
 
-// rows: the chunk's token count (an upper bound on the rows of every loop)
-static void gemm_pf(tlf_ctx* ctx, const DeviceMat& W, const CUtensorMap* xmap, GemmArgs a, int rows,
-                    cudaStream_t st) {
+// A projection of the `rows` rows of a prefill loop. Up to 256 rows are one token tile of k_gemm_tc: a short
+// prompt streams the weights, and K is split over a cluster (up to 8 CTAs, at least two k-tiles each), as in the
+// decode step, while the tiles x splits still fit one CTA per SM. More rows, or more weight tiles than SMs, fill the
+// chip with tiles of the pair GEMM: at 8192 rows it takes 254 / 109 / 62 / 144 us for the long-context model's
+// gate/up, QKV, O and down projections, against 454 / 211 / 111 / 186 us for tiles of k_gemm_tc, and 79 / 55 / 23 / 43
+// against 186 / 124 / 47 / 66 us for the mid-size model's.
+static void gemm_pf(tlf_ctx* ctx, const DeviceMat& W, const CUtensorMap* xmap, const CUtensorMap* xpair, GemmArgs a,
+                    int rows, cudaStream_t st) {
   a.N = W.N;
   a.K = W.K;
   a.err = ctx->d_err;
   a.splits = 1;
-  const int ntiles = (W.N + 127) / 128, ttiles = (rows + 255) / 256;
-  // A chunk of few token tiles (a short prompt) would stream the weights through few CTAs, one per
-  // (128-row tile, token tile): K is split over a cluster instead (up to 8 CTAs, at least two k-tiles
-  // each), as in the decode step, while the tiles x splits still fit one CTA per SM.
-  if (a.epi >= EPI_CL_RESID) {
-    const int nkb = (W.K + 63) / 64;
-    while (a.splits < 8 && (long long)ntiles * ttiles * a.splits * 2 <= ctx->num_sms && nkb >= 4 * a.splits)
-      a.splits *= 2;
-  }
-  // Stage 128 of the 256 token columns at a time (2-stage ring): two CTAs share an SM, so one
-  // CTA's epilogue overlaps the other's main loop. Only worth it when the grid has more tiles
-  // than SMs; a smaller grid keeps one CTA per SM and the deeper ring.
-  const long long tiles = (long long)ntiles * ttiles;
-  a.red_window = (a.splits == 1 && tiles > ctx->num_sms) ? 128 : 0;
   a.max_rows = ctx->pf_C;
-  // token tiles of the chunk's rows (every loop's rows are among them), not of its capacity: a short
-  // prompt would otherwise launch a grid of CTAs that only wait for the kernel before and exit
-  a.tok_tiles = ttiles;
+  const int ntiles = (W.N + 127) / 128, nkb = (W.K + 63) / 64;
+  if (rows > 256 || ntiles > ctx->num_sms) {
+    const int bn = gemm_pf_tile_n(rows, W.N, W.K, a.epi, ctx->md.hd, ctx->pf_pairs);
+    launch_gemm_pf(xpair, bn == 256 ? &W.map : bn == 128 ? &W.map64 : &W.map32, bn, a, rows, ctx->pf_pairs, st);
+    return;
+  }
+  while (a.splits < 8 && (long long)ntiles * a.splits * 2 <= ctx->num_sms && nkb >= 4 * a.splits) a.splits *= 2;
   launch_gemm_tc(&W.map, xmap, 256, a, st);
 }
 
@@ -1314,7 +1318,7 @@ static int prefill_batched(tlf_ctx* ctx, int n_seqs, const int* slot_of, const i
         a.row_slot = ctx->d_pf_row_slot + (size_t)r * C;
         a.row_cslot = ctx->d_pf_row_cslot + (size_t)r * C;
         a.row_pos = ctx->d_pf_row_pos + (size_t)r * C;
-        gemm_pf(ctx, ctx->wqkv[j], &ctx->pf_map_X, a, nr, st);
+        gemm_pf(ctx, ctx->wqkv[j], &ctx->pf_map_X, &ctx->pf_pair_X, a, nr, st);
         // attention blocks of loop r: sum over sequences of ceil(count / qblock) <= nr / qblock + S
         launch_pf_attn(md, P, sp, r, j, ctx->d_pf_Q, ctx->d_pf_O, nr / P.qblock + S + 1, st,
                        ctx->has_pool_map && ctx->pf_ws ? &ctx->map_pool : nullptr);
@@ -1325,7 +1329,7 @@ static int prefill_batched(tlf_ctx* ctx, int n_seqs, const int* slot_of, const i
         a.ldr = md.d;
         a.idx = idx_r;
         a.alpha = cond_args(ctx, ctx->d_pf_m, r, j, 0);
-        gemm_pf(ctx, ctx->wo[j], &ctx->pf_map_O, a, nr, st);
+        gemm_pf(ctx, ctx->wo[j], &ctx->pf_map_O, &ctx->pf_pair_O, a, nr, st);
         launch_norm_rows(md.dtype, ctx->d_pf_H, md.d, idx_r, n_dev, 0, nr, ctx->d_mlp_norm + (size_t)j * md.d, md.d,
                          md.eps, ctx->d_pf_X, md.d, st, cond_args(ctx, ctx->d_pf_m, r, j, 3));
         a = GemmArgs{};
@@ -1333,7 +1337,7 @@ static int prefill_batched(tlf_ctx* ctx, int n_seqs, const int* slot_of, const i
         a.epi = EPI_CL_SWIGLU;
         a.md = md;
         a.U = ctx->d_pf_U;
-        gemm_pf(ctx, ctx->wgu[j], &ctx->pf_map_X, a, nr, st);
+        gemm_pf(ctx, ctx->wgu[j], &ctx->pf_map_X, &ctx->pf_pair_X, a, nr, st);
         a = GemmArgs{};
         a.n_dev = n_dev;
         a.epi = EPI_CL_RESID;
@@ -1341,7 +1345,7 @@ static int prefill_batched(tlf_ctx* ctx, int n_seqs, const int* slot_of, const i
         a.ldr = md.d;
         a.idx = idx_r;
         a.alpha = cond_args(ctx, ctx->d_pf_m, r, j, 1);
-        gemm_pf(ctx, ctx->wd[j], &ctx->pf_map_U, a, nr, st);
+        gemm_pf(ctx, ctx->wd[j], &ctx->pf_map_U, &ctx->pf_pair_U, a, nr, st);
       }
     }
     if (last_logits && nend > 0) {

@@ -500,8 +500,6 @@ struct GemmArgs {
   const float2* rope;      // [max_pos][hd/2] (cos, sin) of position x rotary frequency
   float* Q;                // [max_rows][Hq][hd]
   void* U;                 // [max_rows][ff] bf16
-  // token tiling (prefill): gridDim.z = tok_tiles tiles of NT rows
-  int tok_tiles;
   // prefill QKV epilogue: per compact row, sequence slot, loop-r cache slot and position
   const int* row_slot;
   const int* row_cslot;
@@ -528,9 +526,6 @@ struct GemmArgs {
   int blo;                 // consumer: row offset of the token operand's lo plane (0: one plane)
   bf16* xn_lo;             // producer (split norm): lo plane of xn (NULL: none)
   void* U_lo;              // EPI_CL_SWIGLU: lo plane of U (NULL: none)
-  // One-split cluster epilogues (prefill) may stage their fp32 tile in windows of this many token
-  // columns, so the CTA needs less shared memory and two share an SM (0: the whole tile at once).
-  int red_window;
 };
 // Entries per row of the split-norm partial sums for model width d.
 inline int split_norm_ldss(int d) { return (((d + 127) / 128) + 3) / 4 * 4; }
@@ -558,6 +553,13 @@ int build_cond_table(const ModelDims& md, const float* t_w1, const float* t_b1, 
 
 void launch_gemm_simt(int dtype, const void* W, const void* X, int ldx, const GemmArgs& a, cudaStream_t st);
 void launch_gemm_tc(const CUtensorMap* mapW, const CUtensorMap* mapX, int nt_max, const GemmArgs& a,
+                    cudaStream_t st);
+// Prefill GEMM of many rows (k_gemm_pf): the pairs of SMs its persistent grid may fill (0: no such
+// launch is possible), the tile width to use for a launch, and the launch. mapX: token operand with boxes of 128
+// rows; mapW: weights with boxes of bn / 2 rows.
+int gemm_pf_max_pairs(int num_sms);
+int gemm_pf_tile_n(int rows, int N, int K, int epi, int head_dim, int max_pairs);
+void launch_gemm_pf(const CUtensorMap* mapX, const CUtensorMap* mapW, int bn, const GemmArgs& a, int rows, int max_pairs,
                     cudaStream_t st);
 // operand-ring depth of a tcgen05 GEMM whose CTAs each reduce ceil(ceil(K/64)/splits) k-tiles
 // with token tile nt (and a two-term operand when lo), and the dynamic shared memory one CTA
