@@ -323,7 +323,14 @@ __device__ void cluster_epilogue(const GemmArgs& a, float* red, int4* ci, const 
           x1[q] *= scale[cc];
         }
         const float r0 = x0[q] * csn[q].x - x1[q] * csn[q].y, r1 = x0[q] * csn[q].y + x1[q] * csn[q].x;
-        if (is_q) {
+        if (is_q && a.q_hi) {
+          const size_t at = ((size_t)cc * md.Hq + h) * hd + i;
+          const bf16 h0 = __float2bfloat16_rn(r0), h1 = __float2bfloat16_rn(r1);
+          a.q_hi[at] = h0;
+          a.q_hi[at + half] = h1;
+          a.q_lo[at] = __float2bfloat16_rn(r0 - __bfloat162float(h0));
+          a.q_lo[at + half] = __float2bfloat16_rn(r1 - __bfloat162float(h1));
+        } else if (is_q) {
           float* qo = a.Q + ((size_t)cc * md.Hq + h) * hd;
           qo[i] = r0;
           qo[i + half] = r1;

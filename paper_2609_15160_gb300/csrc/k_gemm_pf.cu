@@ -119,9 +119,9 @@ __device__ __forceinline__ void tmem_ld_32_issue(uint32_t taddr, uint32_t* r) {
       : "r"(taddr));
 }
 
-__device__ __forceinline__ uint32_t pack2(float a, float b) {
-  return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(a)) |
-         ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(b)) << 16);
+__device__ __forceinline__ uint32_t pack2(float a, float b) {  // one packed conversion
+  const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&v);
 }
 
 }  // namespace
@@ -394,7 +394,31 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
               r0[i] = is_v ? p : p * cs[i].x - q * cs[i].y;
               r1[i] = is_v ? q : p * cs[i].y + q * cs[i].x;
             }
-            if (is_q) {
+            if (is_q && a.q_hi) {
+              // 16 + 16 elements of the hi plane, then of the lo plane
+              uint32_t* sw = reinterpret_cast<uint32_t*>(srow);
+              auto split = [&](const float* v, int at) {
+#pragma unroll
+                for (int i = 0; i < 16; i += 2) {
+                  const float a0 = __bfloat162float(__float2bfloat16_rn(v[i])), a1 = __bfloat162float(__float2bfloat16_rn(v[i + 1]));
+                  sw[at + i / 2] = pack2(a0, a1);
+                  sw[16 + at + i / 2] = pack2(v[i] - a0, v[i + 1] - a1);
+                }
+              };
+              split(r0, 0);
+              split(r1, 8);
+              __syncwarp();
+              const int c = (lane & 3) * 8;
+              const int e = c < 16 ? 16 * u + c : half + 16 * u + c - 16;
+              bf16* plane = (lane & 4) ? a.q_lo : a.q_hi;
+#pragma unroll
+              for (int q = 0; q < 8; ++q) {
+                const int rr = 4 * q + (lane >> 3);
+                const int dst = __shfl_sync(0xffffffffu, drow, rr);
+                const uint4 x = *reinterpret_cast<const uint4*>(stg + rr * PG_SEG + (lane & 7) * 16);
+                if (dst >= 0) *reinterpret_cast<uint4*>(plane + (size_t)dst * md.q_dim + f + e) = x;
+              }
+            } else if (is_q) {
 #pragma unroll
               for (int i = 0; i < 16; i += 4) {
                 *reinterpret_cast<float4*>(srow + i) = make_float4(r0[i], r0[i + 1], r0[i + 2], r0[i + 3]);

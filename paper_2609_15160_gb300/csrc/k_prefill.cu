@@ -13,7 +13,9 @@
 // k_pf_plan       per loop r: compact rows A_r, each row's sequence slot, cache
 //                 slot and position, per-sequence counts, first rows and query
 //                 blocks of the attention.
-// k_pf_attn       causal attention of one block of QB queries of one sequence
+// k_pf_attn_pair  causal attention of one block of queries of one sequence against
+//                 that sequence's loop-r cache on the tensor cores (head_dim 64, 128).
+// k_pf_attn       the same for head_dim 32, one block of QB queries
 //                 against that sequence's loop-r cache, for the G query heads of
 //                 one kv head; K is staged transposed in shared memory so each
 //                 lane scores whole keys, online softmax in float32 (base 2).
@@ -296,9 +298,9 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
-__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
-  return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(a)) |
-         ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(b)) << 16);
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {  // one packed conversion
+  const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&v);
 }
 
 template <int HD, int G>
@@ -579,72 +581,127 @@ __global__ void __launch_bounds__(PFT_THREADS) k_pf_attn_tc(ModelDims md, Prefil
 }
 
 // ----------------------------------------------------------------------------
-// Warp-specialised tensor-core causal attention of a chunk (bf16, head_dim 64 or 128)
+// Tensor-core causal attention of a chunk, two query tiles a CTA (bf16, head_dim 64 or 128)
 // ----------------------------------------------------------------------------
-// Same work split as k_pf_attn_tc (one CTA per sequence, block of QT = 128/G queries and kv head;
-// the 128 MMA rows are query * G + head; cache pages of 64 slots), with the roles split across
-// warps so that no block-wide barrier sits in the page loop:
-//   warp 4      TMA producer: the block's q rows (bulk copies, staged in the empty rings), then the
-//               K and V segments of every page, straight from the paged pool through a 3-D tensor
-//               map (128-byte swizzle), into K and V rings (three deep for head_dim 128);
-//   warp 5      MMA issuer: S(p) = Q K(p)^T into one of two TMEM buffers (q as bf16 hi + lo terms,
-//               so the scores keep q's float32 precision), then O += P(p-1) V(p-1) with V taken as
-//               an MN-major operand (no transpose);
-//   warps 0-3   softmax, one thread per row: read the row of S(p) from TMEM, mask causally by cache
-//               slot, keep the running maximum (refreshed lazily: O is rescaled in TMEM only when a
-//               row's maximum grows by more than 8 in base 2) and sum in float32, and write P(p) in
-//               bf16 to one of two shared-memory buffers; at the end they normalise O and store it.
-// mbarriers connect the roles (ring full / empty, S full / free, P full / free); every wait is
-// bounded. Slots past the block's last query in its last page hold finite values (the pool is
-// zeroed when created and only ever holds finite entries), which the mask turns into P = 0.
-constexpr int PFW_THREADS = 192;
+// One CTA per (sequence, block of 2 x 128/G queries, kv head). The block is two tiles of 128 MMA rows
+// (row = query * G + head) that share every K/V block of 128 cache slots (two pages), so that the tensor
+// cores work on one tile while the other tile's softmax runs:
+//   warps 0-3, 4-7  softmax of tile 0 and 1, one thread per row: read the row of S from TMEM, mask causally by
+//                   cache slot, keep the running maximum (refreshed lazily: O is rescaled in TMEM only when a
+//                   row's maximum grows by more than 8 in base 2) and sum in float32, write P in bf16 back to
+//                   TMEM, where it is the A operand of the P V product; at the end normalise O and store it;
+//   warp 8          TMA producer: the tiles' q rows as bf16 hi and lo planes (the scores keep q's float32
+//                   precision), then K and V of every block through 3-D tensor maps into one ring;
+//   warp 9          MMA issuer: S = Qhi K^T + Qlo K^T, O += P V with V taken as an MN-major operand.
+// mbarriers connect the roles; every wait is bounded. A block past a sequence's last page loads its last
+// page twice: slots past the last query hold finite values (the pool is zeroed when created and only
+// ever holds finite entries), which the mask turns into P = 0.
+//
+// What bounds it: at head_dim 128 a block of a tile is 1536 cycles of MMAs (two S products for q's two terms, one P
+// V) against about 1024 of exponentials, so the tiles' softmaxes hide behind each other's MMAs; at head_dim 64 the
+// exponentials lead. Measured at 8192 causal rows: 310 us for 16 / 8 heads x 128 (890 useful TFLOP/s, 1330 counted
+// with both q terms, 0.70 of the measured bf16 rate; one tile of 128 rows and 64-key pages a CTA took 549 us), and 67
+// us for eight prompts of about 1000 rows, 16 heads x 64 (104 us). Scalar bf16 conversions instead of packed ones cost
+// 8 %.
+//
+// Layouts: TMEM holds S of both tiles (128 columns each) and O of both (head_dim columns each). With
+// head_dim 128 that is all 512 columns, so P overwrites its S; tcgen05 executes one thread's MMAs in
+// order, so the next S of a tile may be issued right behind the P V product that reads P. With head_dim 64
+// P has columns of its own and the next S is issued as soon as the softmax has read the one before.
+constexpr int PFA_THREADS = 320;
 
 template <int HD>
-struct PfWsShape {
-  static constexpr int ATOMS = HD / 64;                // 128-byte atom columns of a row
-  static constexpr int Q_BYTES = 128 * HD * 2;         // one of the hi / lo Q tiles [128][HD]
-  static constexpr int QCOL = 128 * 128;               // bytes of one atom column of a Q tile
-  static constexpr int KV_BYTES = 64 * HD * 2;         // a K (or V) stage: [64 keys][HD]
-  static constexpr int KVCOL = 64 * 128;               // bytes of one atom column of a stage
-  // ring depth: with head_dim 128 a K copy is issued once the S product three pages back has freed
-  // its stage, which covers the copy's latency (two stages left the MMA waiting for K); head_dim 64
-  // keeps two stages so that two CTAs (101 KB each) share an SM and cover it between them
-  static constexpr int NST = HD == 128 ? 3 : 2;
-  static constexpr int P_BYTES = 128 * 64 * 2;         // a P buffer [128][64 keys]
-  static constexpr int OFF_QHI = 0;
-  static constexpr int OFF_QLO = OFF_QHI + Q_BYTES;
-  static constexpr int OFF_K = OFF_QLO + Q_BYTES;
-  static constexpr int OFF_V = OFF_K + NST * KV_BYTES;
-  static constexpr int OFF_P = OFF_V + NST * KV_BYTES;
-  static constexpr int OFF_BAR = OFF_P + 2 * P_BYTES;
-  static constexpr int NBAR = 4 * NST + 9;
-  static_assert(128 * HD * 4 <= 2 * NST * KV_BYTES, "the float32 Q tile is staged in the K/V rings");
+struct PfaShape {
+  static constexpr int ATOMS = HD / 64;               // 128-byte atom columns of a row
+  static constexpr int COL = 128 * 128;               // bytes of one atom column of 128 rows
+  static constexpr int T_BYTES = ATOMS * COL;         // a tile of 128 rows: Q hi, Q lo, K or V
+  static constexpr int NST = HD == 128 ? 3 : 8;       // K/V ring
+  static constexpr int OFF_Q = 0;                     // tile 0 hi, lo, tile 1 hi, lo
+  static constexpr int OFF_KV = 4 * T_BYTES;
+  static constexpr int OFF_BAR = OFF_KV + NST * T_BYTES;
+  static constexpr int NBAR = 2 * NST + 2 + 8;
   static constexpr int BYTES = OFF_BAR + NBAR * 8 + 16 + 1024;  // barriers, TMEM slot, alignment slack
-  static constexpr uint32_t TMEM_COLS = 256;          // S buffers in columns 0..127, O in 128..128+HD
+  static constexpr bool SEP_P = HD == 64;
+  static constexpr uint32_t SCOL = 0, OCOL = 256, PCOL = SEP_P ? 384 : 0;
+  static constexpr uint32_t P_STEP = SEP_P ? 64 : 128;  // columns from tile 0's P to tile 1's
+  static_assert(BYTES <= 232448, "shared memory of one CTA");
 };
 
+// D(tmem) (+)= A(tmem) * B(smem desc)
+__device__ __forceinline__ void tc_mma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
+                                              uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// 32 lanes x 32-bit, 16 consecutive columns per thread, register -> TMEM; completes at tmem_st_wait().
+__device__ __forceinline__ void tmem_st_16_issue(uint32_t taddr, const uint32_t* r) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+      "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(taddr),
+      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+      "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+      : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_ld_32_issue(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,"
+      "%29,%30,%31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr));
+}
+
 template <int HD, int G>
-__global__ void __launch_bounds__(PFW_THREADS, HD == 64 ? 2 : 1) k_pf_attn_ws(ModelDims md, PrefillDev p, StepDev s, int r, int j,
-                                                             const float* __restrict__ Q, bf16* __restrict__ O,
-                                                             const __grid_constant__ CUtensorMap pool_map) {
-  using Sh = PfWsShape<HD>;
+__global__ void __launch_bounds__(PFA_THREADS, 1) k_pf_attn_pair(ModelDims md, PrefillDev p, StepDev s, int r, int j,
+                                                                 bf16* __restrict__ O,
+                                                                 const __grid_constant__ CUtensorMap q_map,
+                                                                 const __grid_constant__ CUtensorMap pool_map) {
+  using Sh = PfaShape<HD>;
   constexpr int QT = 128 / G, NST = Sh::NST;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm + Sh::OFF_BAR);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + Sh::NBAR);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   auto bar = [&](int i) { return smem_u32(&bars[i]); };
-  // K full / empty, V full / empty (NST each), then S full x2, S free x2, P full x2, P free x2
-  auto k_full = [&](int st) { return bar(st); };
-  auto k_empty = [&](int st) { return bar(NST + st); };
-  auto v_full = [&](int st) { return bar(2 * NST + st); };
-  auto v_empty = [&](int st) { return bar(3 * NST + st); };
-  auto s_full = [&](int b) { return bar(4 * NST + b); };
-  auto s_free = [&](int b) { return bar(4 * NST + 2 + b); };
-  auto p_full = [&](int b) { return bar(4 * NST + 4 + b); };
-  auto p_free = [&](int b) { return bar(4 * NST + 6 + b); };
-  const uint32_t q_full = bar(4 * NST + 8);
+  auto kv_full = [&](int st) { return bar(st); };
+  auto kv_empty = [&](int st) { return bar(NST + st); };
+  const uint32_t q_full0 = bar(2 * NST);                          // one per tile
+  auto s_full = [&](int x) { return bar(2 * NST + 2 + x); };  // S of tile x written
+  auto s_read = [&](int x) { return bar(2 * NST + 4 + x); };  // ... read by its softmax (SEP_P)
+  auto p_full = [&](int x) { return bar(2 * NST + 6 + x); };  // P of tile x written
+  auto o_done = [&](int x) { return bar(2 * NST + 8 + x); };  // its P V product done
 
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid == 0) {
+    for (int i = 0; i < NST; ++i) {
+      mbar_init(kv_full(i), 1);
+      mbar_init(kv_empty(i), 1);
+    }
+    for (int x = 0; x < 2; ++x) {
+      mbar_init(q_full0 + 8 * x, 1);
+      mbar_init(s_full(x), 1);
+      mbar_init(s_read(x), 4);
+      mbar_init(p_full(x), 4);
+      mbar_init(o_done(x), 1);
+    }
+    *abort_flag = 0;
+    fence_barrier_init();
+    prefetch_tensormap(&q_map);
+    prefetch_tensormap(&pool_map);
+  }
+  if (warp == 9) {
+    tmem_alloc(smem_u32(tmem_slot), 512);
+    tmem_relinquish();
+  }
   pdl_wait();
   pdl_trigger();
   const int S = p.S;
@@ -653,85 +710,25 @@ __global__ void __launch_bounds__(PFW_THREADS, HD == 64 ? 2 : 1) k_pf_attn_ws(Mo
   // (the last queries of a sequence) are dispatched first, so the last wave holds short ones
   const int ntiles = tbase[S];
   const int kvh = blockIdx.x % md.Hkv, tile = ntiles - 1 - (int)(blockIdx.x / md.Hkv);
-  if (tile < 0) return;
   int lo = 0, hi = S;  // sequence: largest sq with tbase[sq] <= tile
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
     if (tbase[mid] <= tile) lo = mid; else hi = mid;
   }
-  const int sq = lo, qb = tile - tbase[sq];
+  const int sq = lo, qb = tile < 0 ? 0 : tile - tbase[sq];
   const int cnt = p.cnt[r * p.Smax + sq], first = p.first[r * p.Smax + sq], s0 = p.s0[r * p.Smax + sq];
   const int slot = p.seq_slot[sq];
-  const int q0 = qb * QT, nq = min(QT, cnt - q0);
-  const int last = s0 + q0 + nq - 1;  // cache slot of the block's last query
-  const int npages = last / 64 + 1;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int* ptab = s.page_table + ((size_t)slot * md.M + r) * md.max_pages;
-
-  if (tid == 0) {
-    for (int i = 0; i < NST; ++i) {
-      mbar_init(k_full(i), 1);
-      mbar_init(k_empty(i), 1);
-      mbar_init(v_full(i), 1);
-      mbar_init(v_empty(i), 1);
-    }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(s_full(b), 1);
-      mbar_init(s_free(b), 4);
-      mbar_init(p_full(b), 4);
-      mbar_init(p_free(b), 1);
-    }
-    mbar_init(q_full, 1);
-    fence_barrier_init();
-    prefetch_tensormap(&pool_map);
-    // the block's float32 q rows, staged in the (still unused) K/V rings: the G heads of a query
-    // are contiguous, so one bulk copy per query
-    mbar_arrive_expect_tx(q_full, (uint32_t)(nq * G * HD * 4));
-    for (int qq = 0; qq < nq; ++qq)
-      bulk_g2s(smem_u32(sm + Sh::OFF_K + qq * G * HD * 4), Q + ((size_t)(first + q0 + qq) * md.Hq + kvh * G) * HD,
-               (uint32_t)(G * HD * 4), q_full);
-  }
-  if (warp == 5) {
-    tmem_alloc(smem_u32(tmem_slot), Sh::TMEM_COLS);
-    tmem_relinquish();
-  }
-  __syncthreads();  // barriers initialised
-  const bool q_ok = __all_sync(0xffffffffu, mbar_wait(q_full, 0, s.err));
-  // Q tile: row = query * G + head, as hi and lo bf16 parts (zeros past the block's queries)
-  const float* qstage = reinterpret_cast<const float*>(sm + Sh::OFF_K);
-  for (int e = tid; e < 128 * (HD / 8); e += PFW_THREADS) {
-    const int qr = e / (HD / 8), c = e % (HD / 8);
-    const int qq = qr / G;
-    float x[8];
-    if (qq < nq && q_ok) {
-      const float4* q4 = reinterpret_cast<const float4*>(qstage + (size_t)qr * HD);
-      const float4 a = q4[2 * c], b = q4[2 * c + 1];
-      x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
-    } else {
-#pragma unroll
-      for (int u = 0; u < 8; ++u) x[u] = 0.f;
-    }
-    uint32_t h[4], l[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const float a0 = __bfloat162float(__float2bfloat16_rn(x[2 * u]));
-      const float a1 = __bfloat162float(__float2bfloat16_rn(x[2 * u + 1]));
-      h[u] = pack_bf16(a0, a1);
-      l[u] = pack_bf16(x[2 * u] - a0, x[2 * u + 1] - a1);
-    }
-    const uint32_t off = (c / 8) * Sh::QCOL + sw128_off(qr, c % 8);
-    *reinterpret_cast<uint4*>(sm + Sh::OFF_QHI + off) = make_uint4(h[0], h[1], h[2], h[3]);
-    *reinterpret_cast<uint4*>(sm + Sh::OFF_QLO + off) = make_uint4(l[0], l[1], l[2], l[3]);
-  }
-  fence_proxy_async_smem();
+  const int q0 = qb * 2 * QT;
+  // queries and key blocks of the two tiles (tile 1 may have none)
+  const int nq0 = tile < 0 ? 0 : min(QT, cnt - q0), nq1 = tile < 0 ? 0 : max(0, min(QT, cnt - q0 - QT));
+  const int nb0 = nq0 > 0 ? (s0 + q0 + nq0 - 1) / 128 + 1 : 0;
+  const int nb1 = nq1 > 0 ? (s0 + q0 + QT + nq1 - 1) / 128 + 1 : 0;
+  const int nb = max(nb0, nb1);
+  const int last_page = (s0 + q0 + nq0 + nq1 - 1) / 64;
   tc_fence_before();
-  __syncthreads();
+  __syncthreads();  // barriers initialised, TMEM allocated
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  constexpr uint32_t OCOL = 128;  // first TMEM column of O
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  if (tid == 0) *abort_flag = 0;
-  __syncthreads();
   // a bounded wait; once any role has given up, the others skip their waits and wind down
   auto wait = [&](uint32_t b, uint32_t parity) {
     if (*abort_flag) return false;
@@ -742,209 +739,224 @@ __global__ void __launch_bounds__(PFW_THREADS, HD == 64 ? 2 : 1) k_pf_attn_ws(Mo
     return true;
   };
 
-  if (warp == 4) {
+  if (warp == 8) {
     // ---------------- TMA producer ----------------
     if (lane == 0) {
+      for (int x = 0; x < 2; ++x) {
+        if (x == 1 && nq1 == 0) break;
+        if (nq0 == 0) break;
+        mbar_arrive_expect_tx(q_full0 + 8 * x, 2 * Sh::T_BYTES);
+#pragma unroll
+        for (int pl = 0; pl < 2; ++pl)
+#pragma unroll
+          for (int a = 0; a < Sh::ATOMS; ++a)
+            tma_load_3d(smem_u32(sm + Sh::OFF_Q + (2 * x + pl) * Sh::T_BYTES + a * Sh::COL), &q_map, a * 64, kvh * G,
+                        first + q0 + x * QT + pl * p.C, q_full0 + 8 * x);
+      }
+      const int* ptab = s.page_table + ((size_t)slot * md.M + r) * md.max_pages;
       const int rowK = ((j * 2 + 0) * md.Hkv + kvh) * 64, rowV = ((j * 2 + 1) * md.Hkv + kvh) * 64;
-      for (int pg = 0; pg < npages; ++pg) {
-        const int st = pg % NST;
-        const uint32_t par = (uint32_t)((pg / NST) - 1) & 1u;
-        int page = ptab[pg];
-        const bool okp = page >= 0 && page < md.n_pages;
-        if (!okp) atomicOr(s.err, DEVERR_INDEX);
-        if (pg >= NST && !wait(k_empty(st), par)) break;
-        if (okp) {
-          mbar_arrive_expect_tx(k_full(st), Sh::KV_BYTES);
+      bool ok = true;
+      for (int i = 0; i < 2 * nb && ok; ++i) {  // K(0), V(0), K(1), V(1), ...
+        const int st = i % NST, kb = i >> 1;
+        if (i >= NST && !wait(kv_empty(st), (uint32_t)(i / NST - 1) & 1u)) break;
+        int pg[2] = {ptab[2 * kb], ptab[min(2 * kb + 1, last_page)]};
+        const bool okp = pg[0] >= 0 && pg[0] < md.n_pages && pg[1] >= 0 && pg[1] < md.n_pages;
+        if (!okp) {
+          atomicOr(s.err, DEVERR_INDEX);
+          mbar_arrive(kv_full(st));  // complete the phase without data
+          continue;
+        }
+        mbar_arrive_expect_tx(kv_full(st), Sh::T_BYTES);
+        uint8_t* dst = sm + Sh::OFF_KV + st * Sh::T_BYTES;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
 #pragma unroll
           for (int a = 0; a < Sh::ATOMS; ++a)
-            tma_load_3d(smem_u32(sm + Sh::OFF_K + st * Sh::KV_BYTES + a * Sh::KVCOL), &pool_map, a * 64, rowK, page,
-                        k_full(st));
-        } else {
-          mbar_arrive(k_full(st));  // complete the phase without data
-        }
-        if (pg >= NST && !wait(v_empty(st), par)) break;
-        if (okp) {
-          mbar_arrive_expect_tx(v_full(st), Sh::KV_BYTES);
-#pragma unroll
-          for (int a = 0; a < Sh::ATOMS; ++a)
-            tma_load_3d(smem_u32(sm + Sh::OFF_V + st * Sh::KV_BYTES + a * Sh::KVCOL), &pool_map, a * 64, rowV, page,
-                        v_full(st));
-        } else {
-          mbar_arrive(v_full(st));
-        }
+            tma_load_3d(smem_u32(dst + a * Sh::COL + h * (Sh::COL / 2)), &pool_map, a * 64, (i & 1) ? rowV : rowK, pg[h],
+                        kv_full(st));
       }
     }
-  } else if (warp == 5) {
+    __syncwarp();
+  } else if (warp == 9) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      constexpr uint32_t IDS = idesc_bf16_f32(128, 64), IDO = idesc_bf16_f32_bmn(128, HD);
-      // every operand descriptor is a base plus a constant step (encoded in 16-byte units), built
-      // once: this thread's instruction count per page is what paces the loop
-      const uint64_t dqh = smem_desc_sw128(smem_u32(sm + Sh::OFF_QHI));
-      const uint64_t dql = smem_desc_sw128(smem_u32(sm + Sh::OFF_QLO));
-      const uint64_t dk0 = smem_desc_sw128(smem_u32(sm + Sh::OFF_K));
-      const uint64_t dp0 = smem_desc_sw128(smem_u32(sm + Sh::OFF_P));
-      const uint64_t dv0 = smem_desc_sw128_mn(smem_u32(sm + Sh::OFF_V), Sh::KVCOL);
-      constexpr uint64_t QCOL_E = Sh::QCOL >> 4, KVCOL_E = Sh::KVCOL >> 4, KV_E = Sh::KV_BYTES >> 4,
-                         P_E = Sh::P_BYTES >> 4, V16_E = 2048 >> 4;
-      // Two streams, each issued as soon as its inputs are there: S(ns) once K(ns) has landed and the
-      // softmax has read the S buffer two pages back, and P V(npv) once P(npv) and V(npv) are in.
-      // S therefore runs ahead of the softmax instead of behind the P V product before it. One time
-      // limit covers the whole loop.
-      int ns = 0, npv = 0;
-      const uint64_t t0 = globaltimer_ns();
-      while (npv < npages) {
-        bool did = false;
-        if (ns < npages) {
-          const int b = ns & 1, st = ns % NST;
-          if (mbar_try_wait(k_full(st), (uint32_t)(ns / NST) & 1u) &&
-              (ns < 2 || mbar_try_wait(s_free(b), (uint32_t)((ns - 2) >> 1) & 1u))) {
+    if (lane == 0 && nb > 0) {
+      constexpr uint32_t IDS = idesc_bf16_f32(128, 128), IDO = idesc_bf16_f32_bmn(128, HD);
+      constexpr uint64_t T_E = Sh::T_BYTES >> 4, COL_E = Sh::COL >> 4, V16_E = 2048 >> 4;
+      const uint64_t dq = smem_desc_sw128(smem_u32(sm + Sh::OFF_Q));
+      const uint64_t dk = smem_desc_sw128(smem_u32(sm + Sh::OFF_KV));
+      const uint64_t dv = smem_desc_sw128_mn(smem_u32(sm + Sh::OFF_KV), Sh::COL);
+      auto issue_s = [&](int x, int kb) {
+        const uint64_t kd = dk + (uint64_t)((2 * kb) % NST) * T_E, qd = dq + (uint64_t)(2 * x) * T_E;
+        const uint32_t d = tmem + Sh::SCOL + 128u * (uint32_t)x;
+#pragma unroll
+        for (int pl = 0; pl < 2; ++pl)
+#pragma unroll
+          for (int kc = 0; kc < Sh::ATOMS; ++kc)
+#pragma unroll
+            for (int k = 0; k < 4; ++k)  // K = 16 per MMA: +32 bytes (encoded +2) inside the atom column
+              tc_mma_f16(d, qd + pl * T_E + kc * COL_E + 2 * k, kd + kc * COL_E + 2 * k, IDS, (pl | kc | k) ? 1u : 0u);
+        tc_commit(s_full(x));
+      };
+      auto issue_pv = [&](int x, int kb) {
+        const uint64_t vd = dv + (uint64_t)((2 * kb + 1) % NST) * T_E;
+        const uint32_t d = tmem + Sh::OCOL + (uint32_t)(HD * x), pa = tmem + Sh::PCOL + Sh::P_STEP * (uint32_t)x;
+#pragma unroll
+        for (int k = 0; k < 8; ++k)  // K = 16 keys per MMA: 8 TMEM columns of P, +2048 B (16 rows) of V
+          tc_mma_f16_ts(d, pa + 8u * k, vd + V16_E * k, IDO, (kb > 0 || k > 0) ? 1u : 0u);
+        tc_commit(o_done(x));
+      };
+      auto kfull = [&](int kb) { return wait(kv_full((2 * kb) % NST), (uint32_t)(2 * kb / NST) & 1u); };
+      auto vfull = [&](int kb) { return wait(kv_full((2 * kb + 1) % NST), (uint32_t)((2 * kb + 1) / NST) & 1u); };
+      bool ok = wait(q_full0, 0) && kfull(0);
+      if (ok) {
+        tc_fence_after();
+        issue_s(0, 0);
+        if (nb1 > 0) {
+          ok = wait(q_full0 + 8, 0);
+          tc_fence_after();
+          if (ok) issue_s(1, 0);
+        }
+        tc_commit(kv_empty(0));
+      }
+      for (int kb = 0; kb < nb && ok; ++kb) {
+        const bool next = kb + 1 < nb;
+        if (Sh::SEP_P && next) {
+          // both next S products first: each waits only for the softmax to have read the S before
+          ok = kfull(kb + 1);
+          for (int x = 0; x < 2 && ok; ++x)
+            if (kb + 1 < (x ? nb1 : nb0)) {
+              ok = wait(s_read(x), (uint32_t)kb & 1u);
+              if (!ok) break;
+              tc_fence_after();
+              issue_s(x, kb + 1);
+            }
+          if (!ok) break;
+          tc_commit(kv_empty((2 * kb + 2) % NST));
+        }
+        if (!vfull(kb)) break;
+        for (int x = 0; x < 2 && ok; ++x) {
+          if (kb < (x ? nb1 : nb0)) {
+            ok = wait(p_full(x), (uint32_t)kb & 1u);
+            if (!ok) break;
             tc_fence_after();
-            const uint64_t kb = dk0 + st * KV_E;
-            const uint32_t d = tmem + 64u * (uint32_t)b;
-#pragma unroll
-            for (int kc = 0; kc < Sh::ATOMS; ++kc)
-#pragma unroll
-              for (int k = 0; k < 4; ++k) {  // K = 16 per MMA: +32 bytes (encoded +2) inside the atom column
-                const uint64_t db = kb + kc * KVCOL_E + 2 * k;
-                tc_mma_f16(d, dqh + kc * QCOL_E + 2 * k, db, IDS, (kc | k) ? 1u : 0u);
-                tc_mma_f16(d, dql + kc * QCOL_E + 2 * k, db, IDS, 1u);
-              }
-            tc_commit(s_full(b));
-            tc_commit(k_empty(st));
-            ++ns;
-            did = true;
+            issue_pv(x, kb);
+            if (x == 1 || nb1 <= kb) tc_commit(kv_empty((2 * kb + 1) % NST));
+          }
+          if (!Sh::SEP_P && kb + 1 < (x ? nb1 : nb0)) {
+            ok = kfull(kb + 1);
+            if (!ok) break;
+            tc_fence_after();
+            issue_s(x, kb + 1);
           }
         }
-        if (npv < ns) {
-          const int bq = npv & 1, st = npv % NST;
-          if (mbar_try_wait(p_full(bq), (uint32_t)(npv >> 1) & 1u) &&
-              mbar_try_wait(v_full(st), (uint32_t)(npv / NST) & 1u)) {  // O += P(npv) V(npv)
-            tc_fence_after();
-            const uint64_t pa = dp0 + bq * P_E, vb = dv0 + st * KV_E;
-#pragma unroll
-            for (int k = 0; k < 4; ++k)  // K = 16 keys per MMA: +32 B in P's rows, +2048 B (16 rows) in V
-              tc_mma_f16(tmem + OCOL, pa + 2 * k, vb + V16_E * k, IDO, (npv > 0 || k > 0) ? 1u : 0u);
-            tc_commit(p_free(bq));
-            tc_commit(v_empty(st));
-            ++npv;
-            did = true;
-          }
-        }
-        if (!did && (*abort_flag || globaltimer_ns() - t0 > kWaitLimitNs)) {
-          atomicOr(s.err, DEVERR_WAIT);
-          *abort_flag = 1;
-          break;
-        }
+        if (!Sh::SEP_P && ok && next) tc_commit(kv_empty((2 * kb + 2) % NST));
       }
     }
+    __syncwarp();
   } else {
     // ---------------- softmax: thread = MMA row = TMEM lane ----------------
-    // The page's work per thread is short; what bounds it is the length of its dependent chains,
-    // so the row maximum and sum run as four independent partials and no per-key select is taken
-    // (ex2 of -inf is 0 once the reference maximum is finite).
-    const int row = warp * 32 + lane;
-    const uint32_t t_row = tmem + ((uint32_t)(warp * 32) << 16);
+    const int x = warp >> 2, quad = warp & 3, row = quad * 32 + lane;
+    const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
+    const uint32_t t_s = tmem + lane_off + Sh::SCOL + 128u * (uint32_t)x;
+    const uint32_t t_p = tmem + lane_off + Sh::PCOL + Sh::P_STEP * (uint32_t)x;
+    const uint32_t t_o = tmem + lane_off + Sh::OCOL + (uint32_t)(HD * x);
+    const int nbx = x ? nb1 : nb0, nqx = x ? nq1 : nq0;
     const int qi = row / G, g = row % G;
-    const bool row_ok = qi < nq;
-    const int qslot = s0 + q0 + qi;  // cache slot of this row's query
+    const bool row_ok = qi < nqx;
+    // cache slot of this row's query (-1: a row past the tile's queries, which sees no key)
+    const int qslot = row_ok ? s0 + q0 + x * QT + qi : -1;
     const float scale = 1.4426950408889634f * rsqrtf((float)HD);
-    float m_run = -INFINITY, l_run = 0.f;
+    float m_run = -INFINITY, l_run = 0.f;  // in units of the raw scores
+    const float grow_by = 8.f / scale;
     bool ok = true;
     // waits taken by the whole warp: the TMEM accesses after them are warp-collective
-    auto wait_w = [&](uint32_t bq, uint32_t parity) { return __all_sync(0xffffffffu, wait(bq, parity)); };
-    for (int pg = 0; pg < npages && ok; ++pg) {
-      const int b = pg & 1;
-      if (!wait_w(s_full(b), (uint32_t)(pg >> 1) & 1u)) { ok = false; break; }
+    auto wait_w = [&](uint32_t b, uint32_t parity) { return __all_sync(0xffffffffu, wait(b, parity)); };
+    for (int kb = 0; kb < nbx; ++kb) {
+      if (!wait_w(s_full(x), (uint32_t)kb & 1u)) { ok = false; break; }
       tc_fence_after();
-      float sc[64];
-      tmem_ld_32(t_row + 64u * (uint32_t)b, sc);
-      tmem_ld_32(t_row + 64u * (uint32_t)b + 32u, sc + 32);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(s_free(b));
-      const int kb = pg * 64;  // cache slot of column 0
-      float pm4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-      if (row_ok && kb + 63 <= qslot) {  // every key visible
+      uint32_t su[128];
 #pragma unroll
-        for (int c = 0; c < 64; ++c) {
-          sc[c] *= scale;
-          pm4[c & 3] = fmaxf(pm4[c & 3], sc[c]);
-        }
-      } else if (!row_ok || kb > qslot) {  // none visible
-#pragma unroll
-        for (int c = 0; c < 64; ++c) sc[c] = -INFINITY;
-      } else {  // the diagonal: causal by cache slot
-#pragma unroll
-        for (int c = 0; c < 64; ++c) {
-          sc[c] = kb + c <= qslot ? sc[c] * scale : -INFINITY;
-          pm4[c & 3] = fmaxf(pm4[c & 3], sc[c]);
-        }
-      }
-      const float pm = fmaxf(fmaxf(pm4[0], pm4[1]), fmaxf(pm4[2], pm4[3]));
-      // lazy maximum: O is rescaled only when a row's maximum grows by more than 8, after the
-      // P V product before has landed (warp-uniform TMEM access)
-      const bool grow = pm > m_run + 8.f;
-      const float cr = grow ? exp2f(m_run - pm) : 1.f;  // 0 when m_run was -inf
-      if (pg > 0 && __any_sync(0xffffffffu, grow)) {
-        if (!wait_w(p_free((pg - 1) & 1), (uint32_t)((pg - 1) >> 1) & 1u)) { ok = false; break; }
-        tc_fence_after();
-#pragma unroll
-        for (int c0 = 0; c0 < HD; c0 += 16) {
-          float o[16];
-          tmem_ld_16(t_row + OCOL + (uint32_t)c0, o);
-#pragma unroll
-          for (int i = 0; i < 16; ++i) o[i] *= cr;
-          tmem_st_16(t_row + OCOL + (uint32_t)c0, o);
-        }
+      for (int c = 0; c < 128; c += 32) tmem_ld_32_issue(t_s + (uint32_t)c, su + c);
+      tmem_ld_wait();
+      if (Sh::SEP_P) {
         tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(s_read(x));
+      }
+      const int vis = qslot - kb * 128;  // columns 0..vis are visible
+      float pm4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+      if (__any_sync(0xffffffffu, vis < 127)) {
+#pragma unroll
+        for (int c = 0; c < 128; ++c)
+          if (c > vis) su[c] = 0xff800000u;  // -inf
+      }
+#pragma unroll
+      for (int c = 0; c < 128; ++c) pm4[c & 3] = fmaxf(pm4[c & 3], __uint_as_float(su[c]));
+      const float pm = fmaxf(fmaxf(pm4[0], pm4[1]), fmaxf(pm4[2], pm4[3]));
+      // lazy maximum: O is rescaled only when a row's maximum grows by more than 8 in base 2, after the
+      // P V product before has landed (warp-uniform TMEM access)
+      const bool grow = pm > m_run + grow_by;
+      const float cr = grow ? exp2f((m_run - pm) * scale) : 1.f;  // 0 when m_run was -inf
+      if (kb > 0 && (Sh::SEP_P || __any_sync(0xffffffffu, grow))) {
+        if (!wait_w(o_done(x), (uint32_t)(kb - 1) & 1u)) { ok = false; break; }  // (with its own columns, P is free too)
+        tc_fence_after();
+        if (__any_sync(0xffffffffu, grow)) {
+#pragma unroll
+          for (int c0 = 0; c0 < HD; c0 += 16) {
+            float o[16];
+            tmem_ld_16(t_o + (uint32_t)c0, o);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) o[i] *= cr;
+            tmem_st_16(t_o + (uint32_t)c0, o);
+          }
+        }
       }
       if (grow) {
         l_run *= cr;
         m_run = pm;
       }
-      const float mref = m_run == -INFINITY ? 0.f : m_run;  // rows with no visible key so far
-      uint32_t pk[32];
+      const float mref = m_run == -INFINITY ? 0.f : m_run * scale;  // rows with no visible key so far: any finite value
       float ps4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-      for (int c = 0; c < 64; c += 2) {
-        const float p0 = ex2_approx(sc[c] - mref), p1 = ex2_approx(sc[c + 1] - mref);
-        ps4[(c >> 1) & 3] += p0 + p1;
-        pk[c / 2] = pack_bf16(p0, p1);
+      for (int c0 = 0; c0 < 128; c0 += 32) {
+        uint32_t pk[16];
+#pragma unroll
+        for (int c = 0; c < 32; c += 2) {
+          const float p0 = ex2_approx(fmaf(__uint_as_float(su[c0 + c]), scale, -mref));
+          const float p1 = ex2_approx(fmaf(__uint_as_float(su[c0 + c + 1]), scale, -mref));
+          ps4[(c >> 1) & 3] += p0 + p1;
+          pk[c / 2] = pack_bf16(p0, p1);
+        }
+        tmem_st_16_issue(t_p + (uint32_t)(c0 / 2), pk);
       }
       l_run += (ps4[0] + ps4[1]) + (ps4[2] + ps4[3]);
-      // P buffer b was last read by P V of page pg - 2
-      if (pg >= 2 && !wait_w(p_free(b), (uint32_t)((pg - 2) >> 1) & 1u)) { ok = false; break; }
-      uint8_t* pb = sm + Sh::OFF_P + b * Sh::P_BYTES;
-#pragma unroll
-      for (int q = 0; q < 8; ++q)
-        *reinterpret_cast<uint4*>(pb + sw128_off(row, q)) = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
-      fence_proxy_async_smem();
+      tmem_st_wait();
+      tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(p_full(b));
+      if (lane == 0) mbar_arrive(p_full(x));
     }
     // the last P V product, then O / l out
-    if (ok && wait_w(p_free((npages - 1) & 1), (uint32_t)((npages - 1) >> 1) & 1u)) {
+    if (ok && nbx > 0 && wait_w(o_done(x), (uint32_t)(nbx - 1) & 1u)) {
       tc_fence_after();
       const float inv_l = l_run > 0.f ? 1.f / l_run : 0.f;
-      bf16* orow = O + (size_t)(first + q0 + qi) * md.q_dim + (kvh * G + g) * HD;
+      bf16* orow = O + (size_t)(first + q0 + x * QT + qi) * md.q_dim + (kvh * G + g) * HD;
 #pragma unroll
-      for (int c0 = 0; c0 < HD; c0 += 16) {
-        float o[16];
-        tmem_ld_16(t_row + OCOL + (uint32_t)c0, o);
+      for (int c0 = 0; c0 < HD; c0 += 32) {
+        float o[32];
+        tmem_ld_32(t_o + (uint32_t)c0, o);
         if (row_ok) {
-          uint32_t w[8];
 #pragma unroll
-          for (int i = 0; i < 8; ++i) w[i] = pack_bf16(o[2 * i] * inv_l, o[2 * i + 1] * inv_l);
-          *reinterpret_cast<uint4*>(orow + c0) = make_uint4(w[0], w[1], w[2], w[3]);
-          *reinterpret_cast<uint4*>(orow + c0 + 8) = make_uint4(w[4], w[5], w[6], w[7]);
+          for (int i = 0; i < 32; i += 8)
+            *reinterpret_cast<uint4*>(orow + c0 + i) =
+                make_uint4(pack_bf16(o[i] * inv_l, o[i + 1] * inv_l), pack_bf16(o[i + 2] * inv_l, o[i + 3] * inv_l),
+                           pack_bf16(o[i + 4] * inv_l, o[i + 5] * inv_l), pack_bf16(o[i + 6] * inv_l, o[i + 7] * inv_l));
         }
       }
     }
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 5) tmem_dealloc(tmem, Sh::TMEM_COLS);
+  if (warp == 9) tmem_dealloc(tmem, 512);
 }
 
 __global__ void k_pf_len(ModelDims md, PrefillDev p) {
@@ -977,11 +989,11 @@ static void pf_attn_tc_launch(const ModelDims& md, const PrefillDev& p, const St
 }
 
 template <int HD, int G>
-static void pf_attn_ws_launch(const ModelDims& md, const PrefillDev& p, const StepDev& s, int r, int j,
-                              const float* Q, void* O, int tiles_bound, cudaStream_t st, const CUtensorMap* pool_map) {
-  constexpr int smem = PfWsShape<HD>::BYTES;
-  (void)ensure_kernel_attrs((const void*)k_pf_attn_ws<HD, G>, smem);  // a failure shows at launch
-  launch_k(k_pf_attn_ws<HD, G>, dim3(tiles_bound * md.Hkv), PFW_THREADS, smem, st, md, p, s, r, j, Q, (bf16*)O,
+static void pf_attn_pair_launch(const ModelDims& md, const PrefillDev& p, const StepDev& s, int r, int j, void* O,
+                                int tiles_bound, cudaStream_t st, const CUtensorMap* q_map, const CUtensorMap* pool_map) {
+  constexpr int smem = PfaShape<HD>::BYTES;
+  (void)ensure_kernel_attrs((const void*)k_pf_attn_pair<HD, G>, smem);  // a failure shows at launch
+  launch_k(k_pf_attn_pair<HD, G>, dim3(tiles_bound * md.Hkv), PFA_THREADS, smem, st, md, p, s, r, j, (bf16*)O, *q_map,
            *pool_map);
 }
 
@@ -989,20 +1001,24 @@ static void pf_attn_ws_launch(const ModelDims& md, const PrefillDev& p, const St
 // CUDA-core kernel for head_dim 32.
 static bool pf_attn_uses_tc(const ModelDims& md) { return md.hd == 64 || md.hd == 128; }
 
-int pf_attn_qblock(const ModelDims& md) { return pf_attn_uses_tc(md) ? 128 / (md.Hq / md.Hkv) : PF_QB; }
+int pf_attn_qblock(const ModelDims& md, bool pair) {
+  return pf_attn_uses_tc(md) ? (pair ? 256 : 128) / (md.Hq / md.Hkv) : PF_QB;
+}
+
+void launch_pf_attn_pair(const ModelDims& md, const PrefillDev& p, const StepDev& s, int r, int j, void* O,
+                         int tiles_bound, cudaStream_t st, const CUtensorMap* q_map, const CUtensorMap* pool_map) {
+  const int G = md.Hq / md.Hkv;
+  if (md.hd == 128 && G == 1) pf_attn_pair_launch<128, 1>(md, p, s, r, j, O, tiles_bound, st, q_map, pool_map);
+  else if (md.hd == 128 && G == 2) pf_attn_pair_launch<128, 2>(md, p, s, r, j, O, tiles_bound, st, q_map, pool_map);
+  else if (md.hd == 128) pf_attn_pair_launch<128, 4>(md, p, s, r, j, O, tiles_bound, st, q_map, pool_map);
+  else if (G == 1) pf_attn_pair_launch<64, 1>(md, p, s, r, j, O, tiles_bound, st, q_map, pool_map);
+  else if (G == 2) pf_attn_pair_launch<64, 2>(md, p, s, r, j, O, tiles_bound, st, q_map, pool_map);
+  else pf_attn_pair_launch<64, 4>(md, p, s, r, j, O, tiles_bound, st, q_map, pool_map);
+}
 
 void launch_pf_attn(const ModelDims& md, const PrefillDev& p, const StepDev& s, int r, int j, const float* Q,
-                    void* O, int tiles_bound, cudaStream_t st, const CUtensorMap* pool_map) {
+                    void* O, int tiles_bound, cudaStream_t st) {
   const int G = md.Hq / md.Hkv;
-  if (pool_map && (md.hd == 64 || md.hd == 128)) {
-    if (md.hd == 128 && G == 1) pf_attn_ws_launch<128, 1>(md, p, s, r, j, Q, O, tiles_bound, st, pool_map);
-    else if (md.hd == 128 && G == 2) pf_attn_ws_launch<128, 2>(md, p, s, r, j, Q, O, tiles_bound, st, pool_map);
-    else if (md.hd == 128 && G == 4) pf_attn_ws_launch<128, 4>(md, p, s, r, j, Q, O, tiles_bound, st, pool_map);
-    else if (md.hd == 64 && G == 1) pf_attn_ws_launch<64, 1>(md, p, s, r, j, Q, O, tiles_bound, st, pool_map);
-    else if (md.hd == 64 && G == 2) pf_attn_ws_launch<64, 2>(md, p, s, r, j, Q, O, tiles_bound, st, pool_map);
-    else pf_attn_ws_launch<64, 4>(md, p, s, r, j, Q, O, tiles_bound, st, pool_map);
-    return;
-  }
   if (md.hd == 128 && G == 1) pf_attn_tc_launch<128, 1>(md, p, s, r, j, Q, O, tiles_bound, st);
   else if (md.hd == 128 && G == 2) pf_attn_tc_launch<128, 2>(md, p, s, r, j, Q, O, tiles_bound, st);
   else if (md.hd == 128 && G == 4) pf_attn_tc_launch<128, 4>(md, p, s, r, j, Q, O, tiles_bound, st);

@@ -135,6 +135,7 @@ struct tlf_ctx {
   void* d_pf_U = nullptr;
   CUtensorMap pf_map_X, pf_map_O, pf_map_U;     // boxes of 256 rows
   CUtensorMap pf_pair_X, pf_pair_O, pf_pair_U;  // boxes of 128 rows
+  CUtensorMap pf_map_Q;                         // q planes, for the pair attention (has_pool_map)
   int pf_pairs = 0;                             // SM pairs the prefill GEMM's persistent grid may fill
   int *d_pf_idx = nullptr, *d_pf_n = nullptr, *d_pf_row_slot = nullptr, *d_pf_row_cslot = nullptr,
       *d_pf_row_pos = nullptr, *d_pf_first = nullptr, *d_pf_cnt = nullptr, *d_pf_s0 = nullptr,
@@ -309,6 +310,22 @@ static bool make_pool_map(CUtensorMap* m, const void* base, const ModelDims& md)
   cuuint64_t dims[3] = {(cuuint64_t)md.hd, (cuuint64_t)md.J * 2 * md.Hkv * md.page_size, (cuuint64_t)md.n_pages};
   cuuint64_t strides[2] = {(cuuint64_t)md.hd * 2, (cuuint64_t)md.page_elems * 2};
   cuuint32_t box[3] = {64, 64, 1};
+  cuuint32_t es[3] = {1, 1, 1};
+  CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, es,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS;
+}
+
+// 3-D bf16 tensor map over the prefill q planes ([2 C rows][Hq][hd]): box = 64 elements x the G query heads of a kv
+// head x 128 / G rows, i.e. one column of a 128-row query tile (row = query * G + head).
+static bool make_q_map(CUtensorMap* m, const void* base, const ModelDims& md, int rows) {
+  auto fn = get_encode_fn();
+  if (!fn) return false;
+  const cuuint32_t G = (cuuint32_t)(md.Hq / md.Hkv);
+  cuuint64_t dims[3] = {(cuuint64_t)md.hd, (cuuint64_t)md.Hq, (cuuint64_t)rows};
+  cuuint64_t strides[2] = {(cuuint64_t)md.hd * 2, (cuuint64_t)md.q_dim * 2};
+  cuuint32_t box[3] = {64, G, 128 / G};
   cuuint32_t es[3] = {1, 1, 1};
   CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, es,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -1141,6 +1158,8 @@ static int ensure_prefill_buffers(tlf_ctx* ctx) {
       !make_map(&ctx->pf_pair_O, ctx->d_pf_O, C, md.q_dim, md.q_dim, 128) ||
       !make_map(&ctx->pf_pair_U, ctx->d_pf_U, C, md.ff, md.ff, 128))
     return fail(ctx, TLF_ERR_CUDA, "cuTensorMapEncodeTiled failed for a prefill buffer");
+  if (ctx->has_pool_map && !make_q_map(&ctx->pf_map_Q, ctx->d_pf_Q, md, 2 * C))
+    return fail(ctx, TLF_ERR_CUDA, "cuTensorMapEncodeTiled failed for the prefill q planes");
   ctx->pf_pairs = gemm_pf_max_pairs(ctx->num_sms);
   if (ctx->pf_pairs < 1) return fail(ctx, TLF_ERR_CUDA, "the prefill GEMM's clusters cannot be launched on this device");
   ctx->pf_C = C;
@@ -1278,7 +1297,8 @@ static int prefill_batched(tlf_ctx* ctx, int n_seqs, const int* slot_of, const i
     P.cnt = ctx->d_pf_cnt;
     P.s0 = ctx->d_pf_s0;
     P.tile_base = ctx->d_pf_tile_base;
-    P.qblock = pf_attn_qblock(md);
+    const bool pair_attn = ctx->has_pool_map && ctx->pf_ws;
+    P.qblock = pf_attn_qblock(md, pair_attn);
     P.len = ctx->d_len;
     launch_pf_plan(md, P, st);
     // For a chunk of more than one 256-token tile, the rows of every loop come to the host: each
@@ -1315,13 +1335,20 @@ static int prefill_batched(tlf_ctx* ctx, int n_seqs, const int* slot_of, const i
         a.j = j;
         a.rope = ctx->d_rope;
         a.Q = ctx->d_pf_Q;
+        if (pair_attn) {
+          a.q_hi = reinterpret_cast<bf16*>(ctx->d_pf_Q);
+          a.q_lo = a.q_hi + (size_t)C * md.q_dim;
+        }
         a.row_slot = ctx->d_pf_row_slot + (size_t)r * C;
         a.row_cslot = ctx->d_pf_row_cslot + (size_t)r * C;
         a.row_pos = ctx->d_pf_row_pos + (size_t)r * C;
         gemm_pf(ctx, ctx->wqkv[j], &ctx->pf_map_X, &ctx->pf_pair_X, a, nr, st);
         // attention blocks of loop r: sum over sequences of ceil(count / qblock) <= nr / qblock + S
-        launch_pf_attn(md, P, sp, r, j, ctx->d_pf_Q, ctx->d_pf_O, nr / P.qblock + S + 1, st,
-                       ctx->has_pool_map && ctx->pf_ws ? &ctx->map_pool : nullptr);
+        const int blocks = nr / P.qblock + S + 1;
+        if (pair_attn)
+          launch_pf_attn_pair(md, P, sp, r, j, ctx->d_pf_O, blocks, st, &ctx->pf_map_Q, &ctx->map_pool);
+        else
+          launch_pf_attn(md, P, sp, r, j, ctx->d_pf_Q, ctx->d_pf_O, blocks, st);
         a = GemmArgs{};
         a.n_dev = n_dev;
         a.epi = EPI_CL_RESID;

@@ -499,6 +499,8 @@ struct GemmArgs {
   int r, j;
   const float2* rope;      // [max_pos][hd/2] (cos, sin) of position x rotary frequency
   float* Q;                // [max_rows][Hq][hd]
+  bf16* q_hi;              // prefill: q as bf16 hi and lo planes [rows][Hq][hd] instead of Q (NULL: Q)
+  bf16* q_lo;
   void* U;                 // [max_rows][ff] bf16
   // prefill QKV epilogue: per compact row, sequence slot, loop-r cache slot and position
   const int* row_slot;
@@ -616,13 +618,18 @@ struct PrefillDev {
   int* len;            // [max_seqs][M] cache lengths
 };
 void launch_pf_plan(const ModelDims& md, const PrefillDev& p, cudaStream_t st);
-// pool_map: 3-D tensor map over the KV pool, {head_dim, J * 2 * Hkv * 64 rows of a page, pages}, box
-// {64, 64, 1}, 128-byte swizzle (NULL: the kernel without tensor-map loads)
+// Causal attention of a chunk at (loop, layer), thread-staged: the tensor-core kernel for head_dim 64 and 128, the
+// CUDA-core kernel for head_dim 32. Q float32.
 void launch_pf_attn(const ModelDims& md, const PrefillDev& p, const StepDev& s, int r, int j, const float* Q,
-                    void* O, int tiles_bound, cudaStream_t st, const CUtensorMap* pool_map = nullptr);
+                    void* O, int tiles_bound, cudaStream_t st);
+// The same with pages and q loaded through tensor maps (head_dim 64 or 128). q_map: 3-D map over q's hi and lo
+// planes, {head_dim, Hq, 2 C rows}, box {64, G, 128 / G}; pool_map: 3-D map over the KV pool, {head_dim, J * 2 * Hkv *
+// 64 rows of a page, pages}, box {64, 64, 1}; 128-byte swizzle.
+void launch_pf_attn_pair(const ModelDims& md, const PrefillDev& p, const StepDev& s, int r, int j, void* O,
+                         int tiles_bound, cudaStream_t st, const CUtensorMap* q_map, const CUtensorMap* pool_map);
 void launch_pf_len(const ModelDims& md, const PrefillDev& p, cudaStream_t st);
-// Queries per block of the prefill attention kernel that launch_pf_attn picks for this model.
-int pf_attn_qblock(const ModelDims& md);
+// Queries per block of the prefill attention: of launch_pf_attn_pair, or of the kernel launch_pf_attn picks.
+int pf_attn_qblock(const ModelDims& md, bool pair);
 
 // Kernel-level attention operation (tlf_attn_decode): scratch layout and launch.
 struct AttnOpLayout {

@@ -1,6 +1,11 @@
 """Prefill kernels at the edges of their tiles, against the float64 oracle (bf16 tolerance of the parity tests)."""
+import numpy as np
 import pytest
 
+from oracle import tlf_oracle as O
+from paper_2609_15160_gb300 import synth
+
+from _parity import DepthOracle, check_cache, rel_err, tol_for
 from test_gpu_parity import _prefill_decode_compare, _small, tlf  # noqa: F401  (fixture)
 
 pytestmark = pytest.mark.gpu
@@ -22,3 +27,27 @@ def test_many_row_projections(tlf, shape, lens):  # noqa: F811
 
 def test_many_row_projections_conditioned(tlf):  # noqa: F811
     _prefill_decode_compare(tlf, _small(conditioning=True, d_model=192), [300, 90], steps=1)
+
+
+@pytest.mark.parametrize("hd,heads,kv", [(64, 4, 4), (64, 4, 2), (64, 4, 1), (128, 2, 2), (128, 4, 2), (128, 4, 1)])
+def test_pair_attention_blocks(tlf, hd, heads, kv):  # noqa: F811
+    """The two-tile prefill attention around its 128-slot key blocks and query tiles, in one chunk and in chunks whose
+    queries start inside a key block: last-token logits and every cached K/V row against the oracle."""
+    m = _small(n_heads=heads, n_kv_heads=kv, head_dim=hd, d_model=128, max_loops=2, depth_probs=(0.4, 0.6))
+    w = synth.make_weights(m)
+    om = O.OracleModel.from_config(m, w)
+    depth = DepthOracle(om)
+    rng = np.random.default_rng(hd + kv)
+    lens = [1, 127, 129, 257, 400, 640]
+    prompts = [rng.integers(0, m.vocab, size=n).astype(np.int32) for n in lens]
+    forced = [depth.forced_for(p) for p in prompts]
+    seqs = [O.OracleSequence(om) for _ in prompts]
+    want = [O.prefill_gathered(om, s, p, forced=f) for s, p, f in zip(seqs, prompts, forced)]
+    ids = list(range(1, 1 + len(lens)))
+    for chunk in (8192, 256):
+        with tlf.Context(m, w, max_seqs=len(lens), max_batch=len(lens), max_seq_len=700, prefill_chunk=chunk) as ctx:
+            lg, loops = ctx.prefill(ids, prompts, forced=forced)
+            for b, (olog, oloops) in enumerate(want):
+                np.testing.assert_array_equal(loops[b], oloops)
+                assert rel_err(lg[b], olog) < tol_for(m), (chunk, lens[b])
+                check_cache(ctx, ids[b], seqs[b], m)
