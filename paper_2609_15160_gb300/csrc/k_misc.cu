@@ -5,6 +5,7 @@
 //                time/step conditioning the gain is scaled by (1 + gamma). In
 //                split mode it writes H * gain unscaled plus the per-tile sums
 //                of squares, and the consuming GEMM applies the factor.
+// k_norm_many    the same for the many rows of a prefill loop (one plane).
 // k_rope_table   (cos, sin) of every position x rotary frequency, built once.
 // k_rope_append  sums the split-K partials of the fused QKV projection (Eq. 9),
 //                rotates q and k at the token's original position, keeps q for
@@ -90,10 +91,67 @@ __global__ void __launch_bounds__(256) k_norm_rows(const float* __restrict__ H, 
   }
 }
 
+// Gather + RMSNorm of many rows (prefill): one warp per row, C float4 per lane held in registers, so a
+// block of eight rows needs no barrier and every load of a row is in flight at once. (One 256-thread
+// block per row left most of its time to the block's two barriers: 8192 rows of d 1024 took 29 us against 11
+// here, 4.6 TB/s, and of d 2048 33 against 19 us, 5.3 TB/s.)
+template <int C>
+__global__ void __launch_bounds__(256) k_norm_many(const float* __restrict__ H, int ldh, const int* __restrict__ idx,
+                                                   const int* __restrict__ n_dev, int n_host,
+                                                   const float* __restrict__ gain, int d, float eps,
+                                                   bf16* __restrict__ X, int ldx, CondArgs cg) {
+  pdl_wait();
+  pdl_trigger();
+  const int n = n_dev ? *n_dev : n_host;
+  const int k = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (k >= n) return;
+  const int src = idx ? idx[k] : k;
+  const float4* h4 = reinterpret_cast<const float4*>(H + (size_t)src * ldh);
+  const float4* g4 = reinterpret_cast<const float4*>(gain);
+  const int d4 = d / 4;
+  float4 v[C];
+  float ss = 0.f;
+#pragma unroll
+  for (int c = 0; c < C; ++c) {
+    const int i = lane + 32 * c;
+    v[c] = i < d4 ? h4[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+#pragma unroll
+  for (int c = 0; c < C; ++c) ss += v[c].x * v[c].x + v[c].y * v[c].y + v[c].z * v[c].z + v[c].w * v[c].w;
+  const float inv = rsqrtf(warp_sum(ss) / (float)d + eps);
+  bf16* xr = X + (size_t)k * ldx;
+  // time/step conditioning: the gain is scaled by (1 + gamma) of the row's (depth, loop)
+  const float4* c4 = cg.mod ? reinterpret_cast<const float4*>(cond_row(cg, src)) : nullptr;
+#pragma unroll
+  for (int c = 0; c < C; ++c) {
+    const int i = lane + 32 * c;
+    if (i < d4) {
+      float4 g = g4[i];
+      if (c4) {
+        const float4 y = c4[i];
+        g = make_float4(g.x * (1.f + y.x), g.y * (1.f + y.y), g.z * (1.f + y.z), g.w * (1.f + y.w));
+      }
+      const __nv_bfloat162 a = __floats2bfloat162_rn(v[c].x * inv * g.x, v[c].y * inv * g.y);
+      const __nv_bfloat162 b = __floats2bfloat162_rn(v[c].z * inv * g.z, v[c].w * inv * g.w);
+      *reinterpret_cast<uint2*>(xr + 4 * i) =
+          make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+    }
+  }
+}
+
 void launch_norm_rows(int dtype, const float* H, int ldh, const int* idx, const int* n_dev, int n_host, int rows_max,
                       const float* gain, int d, float eps, void* X, int ldx, cudaStream_t st, const CondArgs& gamma,
                       float* ss_out, void* X_lo) {
   if (rows_max <= 0) return;
+  if (dtype == 1 && !ss_out && !X_lo && rows_max > 256 && d <= 2048) {
+    // many rows of one plane (prefill); a row of more than 2048 floats would not stay in one warp's registers, and
+    // few rows fill the chip better with a block each
+    const int grid = (rows_max + 7) / 8;
+    if (d <= 512) launch_k(k_norm_many<4>, grid, 256, 0, st, H, ldh, idx, n_dev, n_host, gain, d, eps, (bf16*)X, ldx, gamma);
+    else if (d <= 1024) launch_k(k_norm_many<8>, grid, 256, 0, st, H, ldh, idx, n_dev, n_host, gain, d, eps, (bf16*)X, ldx, gamma);
+    else launch_k(k_norm_many<16>, grid, 256, 0, st, H, ldh, idx, n_dev, n_host, gain, d, eps, (bf16*)X, ldx, gamma);
+    return;
+  }
   if (dtype == 1)
     launch_k(k_norm_rows<bf16>, rows_max, 256, 0, st, H, ldh, idx, n_dev, n_host, gain, d, eps, (bf16*)X, ldx, gamma,
              ss_out, split_norm_ldss(d), (bf16*)X_lo);
