@@ -75,6 +75,10 @@ struct tlf_ctx {
   bool split_norm = false;      // pre-norms split across the neighbouring GEMMs (tcgen05 path)
   bool operand_lo = false;      // X, O, U carry a lo plane (two-term GEMM operands, tcgen05 path)
   bool pf_ws = true;            // prefill attention: the warp-specialised tensor-map kernel
+  bool step_small = false;      // steps of up to 16 rows run the block in the persistent kernel
+  SmallLayer* d_layers = nullptr;  // [J] its weight pointers
+  float* d_ss8 = nullptr;       // [16][d / 8] its sums of squares
+  unsigned* d_gbar = nullptr;   // its grid barrier
   std::vector<DeviceMat> wqkv, wo, wgu, wd;
   DeviceMat emb_mat;
 
@@ -603,6 +607,18 @@ static int create_impl(tlf_ctx* ctx, const tlf_weights* w) {
     const char* e = getenv("TLF_NO_SPLIT_NORM");
     ctx->split_norm = ctx->use_tc && !(e && e[0] == '1');
   }
+  ctx->step_small = ctx->split_norm && ctx->operand_lo && c.ablation == TLF_ABLATION_NONE &&
+                    step_small_fits(md, ctx->num_sms);
+  if (ctx->step_small) {
+    std::vector<SmallLayer> ls(J);
+    for (int j = 0; j < J; ++j)
+      ls[j] = {(const bf16*)ctx->wqkv[j].ptr, (const bf16*)ctx->wo[j].ptr, (const bf16*)ctx->wgu[j].ptr,
+               (const bf16*)ctx->wd[j].ptr, ctx->d_attn_norm + (size_t)j * d, ctx->d_mlp_norm + (size_t)j * d};
+    if ((rc = upload(ctx, (void**)&ctx->d_layers, ls.data(), ls.size() * sizeof(SmallLayer), "layer pointers"))) return rc;
+    if ((rc = dev_alloc(ctx, &ctx->d_ss8, (size_t)16 * (d / 8) * 4, "norm partial sums"))) return rc;
+    if ((rc = dev_alloc(ctx, &ctx->d_gbar, 8 * 128, "grid barrier"))) return rc;
+    CK(ctx, cudaMemset(ctx->d_gbar, 0, 8 * 128));
+  }
   CK(ctx, cudaMemset(ctx->d_attn_cnt, 0, (size_t)B * md.Hkv * 4));
   if ((rc = dev_alloc(ctx, &ctx->d_logits, (size_t)B * V * 4, "logits"))) return rc;
   if ((rc = dev_alloc(ctx, &ctx->d_err, 16, "error word"))) return rc;
@@ -628,6 +644,7 @@ extern "C" void tlf_destroy(tlf_ctx* ctx) {
     auto f = [](void* p) { if (p) cudaFree(p); };
     f(ctx->d_emb); f(ctx->d_router_w); f(ctx->d_router_w1); f(ctx->d_router_b1); f(ctx->d_router_b); f(ctx->d_attn_norm); f(ctx->d_mlp_norm);
     f(ctx->d_final_norm); f(ctx->d_inv_freq); f(ctx->d_rope); f(ctx->d_rowinfo); f(ctx->d_act); f(ctx->d_col); f(ctx->d_ss); f(ctx->d_cond);
+    f(ctx->d_layers); f(ctx->d_ss8); f(ctx->d_gbar);
     for (auto* v : {&ctx->wqkv, &ctx->wo, &ctx->wgu, &ctx->wd})
       for (auto& m : *v) f(m.ptr);
     f(ctx->d_pool); f(ctx->d_pos_table); f(ctx->d_page_table); f(ctx->d_len); f(ctx->d_upload);
@@ -806,6 +823,7 @@ static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, bool prof, cudaSt
   s.rowinfo = ctx->d_rowinfo;
   s.act = ctx->d_act;
   s.col = ctx->d_col;
+  s.gbar = ctx->d_gbar;
   const PageUpdate* d_upd = reinterpret_cast<const PageUpdate*>(ctx->d_upload + 1 + 3 * B);
 
   ctx->last_launches = 0;
@@ -829,7 +847,31 @@ static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, bool prof, cudaSt
   const int lo_rows = ctx->operand_lo ? maxB : 0;
   void* x_lo = ctx->operand_lo ? static_cast<void*>(reinterpret_cast<bf16*>(ctx->d_X) + (size_t)maxB * md.d) : nullptr;
   void* u_lo = ctx->operand_lo ? static_cast<void*>(reinterpret_cast<bf16*>(ctx->d_U) + (size_t)maxB * md.ff) : nullptr;
-  for (int r = 0; r < M; ++r) {
+  // Up to 16 rows: the whole block as one persistent kernel (a profiled step keeps a launch per stage, so
+  // that each can be timed).
+  const bool small = ctx->step_small && B <= 16 && !prof;
+  if (small) {
+    launch_norm_rows(md.dtype, ctx->d_H, md.d, ctx->d_idx, ctx->d_n, 0, B, ctx->d_attn_norm, md.d, md.eps, ctx->d_X, md.d,
+                     st, cond_args(ctx, s.m, 0, 0, 2), ctx->d_ss, x_lo);
+    SmallStep a{};
+    a.md = md;
+    a.s = s;
+    a.layer = ctx->d_layers;
+    a.X = reinterpret_cast<bf16*>(ctx->d_X);
+    a.O = reinterpret_cast<bf16*>(ctx->d_O);
+    a.U = reinterpret_cast<bf16*>(ctx->d_U);
+    a.Q = ctx->d_Q;
+    a.part = ctx->d_attn_part;
+    a.ss = ctx->d_ss;
+    a.ss8 = ctx->d_ss8;
+    a.ldss = split_norm_ldss(md.d);
+    a.rope = ctx->d_rope;
+    a.cond = ctx->d_cond;
+    a.gbar = ctx->d_gbar;
+    CK(ctx, launch_step_small(a, ctx->num_sms, st));
+    ctx->last_launches += 2;
+  }
+  for (int r = 0; r < M && !small; ++r) {
     const int* n_dev = ctx->d_n + r;
     const int* idx_r = ctx->d_idx + (size_t)r * maxB;
     // rows that do not run loop r but are computed anyway (no-gather ablation) keep their residual

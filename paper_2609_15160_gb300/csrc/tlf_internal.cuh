@@ -441,6 +441,7 @@ struct StepDev {
   int* pos_table;      // [n_pages][page_size]
   void* pool;          // KV pages
   uint32_t* err;
+  unsigned* gbar;      // grid-barrier counters of the persistent step kernel, 8 x 128 bytes (zeroed by the plan kernel; NULL: none)
 };
 
 struct ModelDims {
@@ -529,6 +530,29 @@ struct GemmArgs {
   bf16* xn_lo;             // producer (split norm): lo plane of xn (NULL: none)
   void* U_lo;              // EPI_CL_SWIGLU: lo plane of U (NULL: none)
 };
+// The persistent kernel of a step of up to 16 rows (k_step.cu).
+struct SmallLayer {
+  const bf16 *wqkv, *wo, *wgu, *wd;     // packed as for the GEMMs
+  const float *attn_norm, *mlp_norm;
+};
+struct SmallStep {
+  ModelDims md;
+  StepDev s;
+  const SmallLayer* layer;  // [J], device
+  bf16 *X, *O, *U;          // two planes each, the lo plane max_batch rows down
+  float* Q;
+  float* part;              // attention partials
+  const float* ss;          // [max_batch][ldss] sums of squares of the first pre-norm (per 128 features)
+  float* ss8;               // [max_batch][d / 8] of the others (per 8 features)
+  int ldss;
+  const float2* rope;
+  const float* cond;        // conditioning table (NULL: none)
+  unsigned* gbar;
+  int w1_bytes, w2_bytes, nst;  // shared-memory layout (set by the launcher)
+};
+bool step_small_fits(const ModelDims& md, int num_sms);
+cudaError_t launch_step_small(SmallStep a, int num_sms, cudaStream_t st);
+
 // Entries per row of the split-norm partial sums for model width d.
 inline int split_norm_ldss(int d) { return (((d + 127) / 128) + 3) / 4 * 4; }
 
