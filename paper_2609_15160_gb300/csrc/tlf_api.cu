@@ -76,7 +76,7 @@ struct tlf_ctx {
   bool operand_lo = false;      // X, O, U carry a lo plane (two-term GEMM operands, tcgen05 path)
   bool pf_ws = true;            // prefill attention: the warp-specialised tensor-map kernel
   bool step_small = false;      // steps of up to 16 rows run the block in the persistent kernel
-  SmallLayer* d_layers = nullptr;  // [J] its weight pointers
+  float* d_part_small = nullptr;  // its attention partials
   float* d_ss8 = nullptr;       // [16][d / 8] its sums of squares
   unsigned* d_gbar = nullptr;   // its grid barrier
   std::vector<DeviceMat> wqkv, wo, wgu, wd;
@@ -610,11 +610,8 @@ static int create_impl(tlf_ctx* ctx, const tlf_weights* w) {
   ctx->step_small = ctx->split_norm && ctx->operand_lo && c.ablation == TLF_ABLATION_NONE &&
                     step_small_fits(md, ctx->num_sms);
   if (ctx->step_small) {
-    std::vector<SmallLayer> ls(J);
-    for (int j = 0; j < J; ++j)
-      ls[j] = {(const bf16*)ctx->wqkv[j].ptr, (const bf16*)ctx->wo[j].ptr, (const bf16*)ctx->wgu[j].ptr,
-               (const bf16*)ctx->wd[j].ptr, ctx->d_attn_norm + (size_t)j * d, ctx->d_mlp_norm + (size_t)j * d};
-    if ((rc = upload(ctx, (void**)&ctx->d_layers, ls.data(), ls.size() * sizeof(SmallLayer), "layer pointers"))) return rc;
+    if ((rc = dev_alloc(ctx, &ctx->d_part_small, step_small_part_floats(md, ctx->num_sms) * 4, "attention partials")))
+      return rc;
     if ((rc = dev_alloc(ctx, &ctx->d_ss8, (size_t)16 * (d / 8) * 4, "norm partial sums"))) return rc;
     if ((rc = dev_alloc(ctx, &ctx->d_gbar, 8 * 128, "grid barrier"))) return rc;
     CK(ctx, cudaMemset(ctx->d_gbar, 0, 8 * 128));
@@ -644,7 +641,7 @@ extern "C" void tlf_destroy(tlf_ctx* ctx) {
     auto f = [](void* p) { if (p) cudaFree(p); };
     f(ctx->d_emb); f(ctx->d_router_w); f(ctx->d_router_w1); f(ctx->d_router_b1); f(ctx->d_router_b); f(ctx->d_attn_norm); f(ctx->d_mlp_norm);
     f(ctx->d_final_norm); f(ctx->d_inv_freq); f(ctx->d_rope); f(ctx->d_rowinfo); f(ctx->d_act); f(ctx->d_col); f(ctx->d_ss); f(ctx->d_cond);
-    f(ctx->d_layers); f(ctx->d_ss8); f(ctx->d_gbar);
+    f(ctx->d_part_small); f(ctx->d_ss8); f(ctx->d_gbar);
     for (auto* v : {&ctx->wqkv, &ctx->wo, &ctx->wgu, &ctx->wd})
       for (auto& m : *v) f(m.ptr);
     f(ctx->d_pool); f(ctx->d_pos_table); f(ctx->d_page_table); f(ctx->d_len); f(ctx->d_upload);
@@ -856,12 +853,13 @@ static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, bool prof, cudaSt
     SmallStep a{};
     a.md = md;
     a.s = s;
-    a.layer = ctx->d_layers;
+    for (int j = 0; j < J; ++j)
+      a.layer[j] = {(const bf16*)ctx->wqkv[j].ptr, (const bf16*)ctx->wo[j].ptr, (const bf16*)ctx->wgu[j].ptr,
+                    (const bf16*)ctx->wd[j].ptr, ctx->d_attn_norm + (size_t)j * md.d, ctx->d_mlp_norm + (size_t)j * md.d};
     a.X = reinterpret_cast<bf16*>(ctx->d_X);
-    a.O = reinterpret_cast<bf16*>(ctx->d_O);
     a.U = reinterpret_cast<bf16*>(ctx->d_U);
     a.Q = ctx->d_Q;
-    a.part = ctx->d_attn_part;
+    a.part = ctx->d_part_small;
     a.ss = ctx->d_ss;
     a.ss8 = ctx->d_ss8;
     a.ldss = split_norm_ldss(md.d);

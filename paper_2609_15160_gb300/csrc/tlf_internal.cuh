@@ -531,6 +531,7 @@ struct GemmArgs {
   void* U_lo;              // EPI_CL_SWIGLU: lo plane of U (NULL: none)
 };
 // The persistent kernel of a step of up to 16 rows (k_step.cu).
+constexpr int SS_LAYERS = 16;  // most layers of the block it takes
 struct SmallLayer {
   const bf16 *wqkv, *wo, *wgu, *wd;     // packed as for the GEMMs
   const float *attn_norm, *mlp_norm;
@@ -538,8 +539,8 @@ struct SmallLayer {
 struct SmallStep {
   ModelDims md;
   StepDev s;
-  const SmallLayer* layer;  // [J], device
-  bf16 *X, *O, *U;          // two planes each, the lo plane max_batch rows down
+  SmallLayer layer[SS_LAYERS];  // [J], in the kernel's parameters: their pointers are read without a trip to L2
+  bf16 *X, *U;              // two planes each, the lo plane max_batch rows down
   float* Q;
   float* part;              // attention partials
   const float* ss;          // [max_batch][ldss] sums of squares of the first pre-norm (per 128 features)
@@ -551,6 +552,7 @@ struct SmallStep {
   int w1_bytes, w2_bytes, nst;  // shared-memory layout (set by the launcher)
 };
 bool step_small_fits(const ModelDims& md, int num_sms);
+size_t step_small_part_floats(const ModelDims& md, int num_sms);  // floats of SmallStep::part
 cudaError_t launch_step_small(SmallStep a, int num_sms, cudaStream_t st);
 
 // Entries per row of the split-norm partial sums for model width d.
