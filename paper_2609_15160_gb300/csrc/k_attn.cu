@@ -21,7 +21,7 @@
 // shared-memory ring with 1-D bulk TMA copies that complete on mbarriers. The
 // copies carry an L2 evict-first hint: each page is read once per launch, and the
 // hint keeps the step's small reused buffers resident in L2. The
-// eight consumer warps split every page, release the stage on a per-stage
+// eight consumer warps split every page (or four of them, taking pages in turn), release the stage on a per-stage
 // mbarrier, and keep an online-softmax state (running max, sum, output slice)
 // in float32 for the G query heads of the kv head (grouped-query attention),
 // with LPK lanes sharing a key (16 bytes each) and xor-shuffle reductions.
@@ -44,16 +44,24 @@ constexpr int ATT_PS = 64;     // keys per page (the only page size the library 
 constexpr int ATT_WARPS = 8;   // consumer warps
 constexpr int ATT_THREADS = 32 * (ATT_WARPS + 1);
 
-template <typename T, int HD>
+template <typename T, int HD, int G>
 struct AttnShape {
   static constexpr int VEC = 16 / (int)sizeof(T);   // elements per lane per key
   static constexpr int LPK = HD / VEC;              // lanes per key
   static constexpr int KPW = 32 / LPK;              // keys per warp step
-  static constexpr int KEYS_PER_WARP = ATT_PS / ATT_WARPS;
-  static constexpr int STEPS = KEYS_PER_WARP / KPW;
   static constexpr int SEG_BYTES = ATT_PS * HD * (int)sizeof(T);       // one page of K (or V) of one head
   static constexpr int STAGE_BYTES = 2 * SEG_BYTES;
   static constexpr int NST = (98304 / STAGE_BYTES) < 2 ? 2 : ((98304 / STAGE_BYTES) > 8 ? 8 : (98304 / STAGE_BYTES));
+  // Page teams: with one query head a kv head the warps' chain per page, not its instructions, is what a page costs, so
+  // two teams of four warps take the pages in turn (a ring stage then always belongs to one team, so its depth is even).
+  // With the registers of two CTAs an SM, and the merge below without a second barrier: 200 rows of 64-700 keys, 16
+  // heads x 64, 80 -> 69 us; 32 rows of 128-8192 keys 98.5 -> 95 us (5.9 TB/s).
+  static constexpr int TEAMS = G == 1 && NST % 2 == 0 ? 2 : 1;
+  // Merge buffers: with two, an item's merge needs no barrier behind it.
+  static constexpr int REDS = G == 1 ? 2 : 1;
+  static constexpr int TEAM_WARPS = ATT_WARPS / TEAMS;
+  static constexpr int KEYS_PER_WARP = ATT_PS / TEAM_WARPS;
+  static constexpr int STEPS = KEYS_PER_WARP / KPW;
   static_assert(LPK >= 1 && LPK <= 32 && (32 % LPK) == 0, "head_dim / vector width mismatch");
   static_assert(STEPS >= 1, "page too small for the warp split");
 };
@@ -61,8 +69,8 @@ struct AttnShape {
 // MASKED (the dense-cache ablation): each stage also holds the page's 64 positions, -1 = masked slot.
 template <typename T, int HD, int G, bool MASKED>
 constexpr int attn_smem_bytes() {
-  using S = AttnShape<T, HD>;
-  return 128 + S::NST * S::STAGE_BYTES + ATT_WARPS * G * (HD + 2) * 4 + (MASKED ? S::NST * ATT_PS * 4 : 0) +
+  using S = AttnShape<T, HD, G>;
+  return 128 + S::NST * S::STAGE_BYTES + S::REDS * ATT_WARPS * G * (HD + 2) * 4 + (MASKED ? S::NST * ATT_PS * 4 : 0) +
          2 * S::NST * 8 + 16;
 }
 
@@ -70,11 +78,13 @@ __device__ __forceinline__ void consumer_sync() {
   asm volatile("bar.sync 1, %0;" ::"n"(32 * ATT_WARPS) : "memory");
 }
 
+// Two CTAs an SM: the bound gives one query head the registers it can use (56 otherwise), and keeps four heads (131
+// otherwise, one CTA) at two: 36 rows of about 2950 keys, 32 / 8 heads x 128, 153 -> 141 us.
 template <typename T, int HD, int G, bool MASKED>
-__global__ void __launch_bounds__(ATT_THREADS) k_attn_decode(ModelDims md, StepDev s, int r, int j,
+__global__ void __launch_bounds__(ATT_THREADS, 2) k_attn_decode(ModelDims md, StepDev s, int r, int j,
                                                              const float* __restrict__ Q, float* __restrict__ part,
                                                              T* __restrict__ O, int* __restrict__ cnt, bool o_lo) {
-  using S = AttnShape<T, HD>;
+  using S = AttnShape<T, HD, G>;
   // output element (token k, query head hq, dim e); with o_lo also the lo plane of the
   // projection's two-term operand (bf16 of the rounding remainder, max_batch rows down)
   auto store_o = [&](int k, int hq, int e, float val) {
@@ -88,7 +98,7 @@ __global__ void __launch_bounds__(ATT_THREADS) k_attn_decode(ModelDims md, StepD
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
   uint8_t* ring = smem;                                                   // [NST][K seg | V seg]
   float* red = reinterpret_cast<float*>(ring + S::NST * S::STAGE_BYTES);  // [warps][G][HD + 2]
-  int* mring = reinterpret_cast<int*>(red + ATT_WARPS * PSZ);              // [NST][64] positions (MASKED)
+  int* mring = reinterpret_cast<int*>(red + S::REDS * ATT_WARPS * PSZ);              // [NST][64] positions (MASKED)
   uint64_t* full = reinterpret_cast<uint64_t*>(mring + (MASKED ? S::NST * ATT_PS : 0));
   uint64_t* empty = full + S::NST;
   int* flag = reinterpret_cast<int*>(empty + S::NST);
@@ -111,7 +121,7 @@ __global__ void __launch_bounds__(ATT_THREADS) k_attn_decode(ModelDims md, StepD
   if (tid == 0) {
     for (int i = 0; i < S::NST; ++i) {
       mbar_init(smem_u32(&full[i]), 1);
-      mbar_init(smem_u32(&empty[i]), ATT_WARPS);
+      mbar_init(smem_u32(&empty[i]), S::TEAM_WARPS);
     }
     *abort_flag = 0;
     fence_barrier_init();
@@ -184,6 +194,7 @@ __global__ void __launch_bounds__(ATT_THREADS) k_attn_decode(ModelDims md, StepD
 
   // ---------------- consumer warps ----------------
   const int grp = lane / S::LPK, part_lane = lane % S::LPK;
+  const int team = warp / S::TEAM_WARPS, team_warp = warp % S::TEAM_WARPS;
   const float scale = 1.4426950408889634f * rsqrtf((float)HD);
   int k, h, g;
   locate(p0, k, h, g);
@@ -204,76 +215,81 @@ __global__ void __launch_bounds__(ATT_THREADS) k_attn_decode(ModelDims md, StepD
     }
   };
   begin_item();
+  bool odd = false;  // merge buffer of the item
 
   for (int p = p0; p < p1; ++p) {
     const int i = p - p0, st = i % S::NST;
-    // a wait that runs out records the error word; the page is then computed on stale data
-    if (!*abort_flag && !mbar_wait(smem_u32(&full[st]), (i / S::NST) & 1, s.err)) *abort_flag = 1;
-    const int valid = min(ATT_PS, L - g * ATT_PS);
-    const T* sk = reinterpret_cast<const T*>(ring + st * S::STAGE_BYTES);
-    const T* sv = reinterpret_cast<const T*>(ring + st * S::STAGE_BYTES + S::SEG_BYTES);
-    const int* smask = mring + st * ATT_PS;
-    // key slot usable: inside the cache and, for a full-length cache, not masked (mu^(r) of Eq. 10)
-    auto usable = [&](int key) { return key < valid && (!MASKED || smask[key] >= 0); };
+    if (S::TEAMS == 1 || i % S::TEAMS == team) {  // this warp's team takes the page
+      // a wait that runs out records the error word; the page is then computed on stale data
+      if (!*abort_flag && !mbar_wait(smem_u32(&full[st]), (i / S::NST) & 1, s.err)) *abort_flag = 1;
+      const int valid = min(ATT_PS, L - g * ATT_PS);
+      const T* sk = reinterpret_cast<const T*>(ring + st * S::STAGE_BYTES);
+      const T* sv = reinterpret_cast<const T*>(ring + st * S::STAGE_BYTES + S::SEG_BYTES);
+      const int* smask = mring + st * ATT_PS;
+      // key slot usable: inside the cache and, for a full-length cache, not masked (mu^(r) of Eq. 10)
+      auto usable = [&](int key) { return key < valid && (!MASKED || smask[key] >= 0); };
 
-    float sc[S::STEPS][G];
+      float sc[S::STEPS][G];
 #pragma unroll
-    for (int t = 0; t < S::STEPS; ++t) {
-      const int key = warp * S::KEYS_PER_WARP + t * S::KPW + grp;
-      float kv[S::VEC];
-      const bool use = usable(key);
-      if (use) {
-        Vec16<T>::load(sk + key * HD + part_lane * S::VEC, kv);
-      } else {
+      for (int t = 0; t < S::STEPS; ++t) {
+        const int key = team_warp * S::KEYS_PER_WARP + t * S::KPW + grp;
+        float kv[S::VEC];
+        const bool use = usable(key);
+        if (use) {
+          Vec16<T>::load(sk + key * HD + part_lane * S::VEC, kv);
+        } else {
 #pragma unroll
-        for (int e = 0; e < S::VEC; ++e) kv[e] = 0.f;
+          for (int e = 0; e < S::VEC; ++e) kv[e] = 0.f;
+        }
+#pragma unroll
+        for (int gg = 0; gg < G; ++gg) {
+          float d = 0.f;
+#pragma unroll
+          for (int e = 0; e < S::VEC; ++e) d = fmaf(q[gg][e], kv[e], d);
+#pragma unroll
+          for (int o = S::LPK / 2; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+          sc[t][gg] = use ? d : -INFINITY;
+        }
       }
 #pragma unroll
       for (int gg = 0; gg < G; ++gg) {
-        float d = 0.f;
+        float pm = sc[0][gg];
 #pragma unroll
-        for (int e = 0; e < S::VEC; ++e) d = fmaf(q[gg][e], kv[e], d);
+        for (int t = 1; t < S::STEPS; ++t) pm = fmaxf(pm, sc[t][gg]);
 #pragma unroll
-        for (int o = S::LPK / 2; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-        sc[t][gg] = use ? d : -INFINITY;
-      }
-    }
+        for (int o = S::LPK; o < 32; o <<= 1) pm = fmaxf(pm, __shfl_xor_sync(0xffffffffu, pm, o));
+        if (pm > run_m[gg]) {
+          const float cr = exp2f(run_m[gg] - pm);  // 0 when run_m was -inf
+          run_l[gg] *= cr;
 #pragma unroll
-    for (int gg = 0; gg < G; ++gg) {
-      float pm = sc[0][gg];
-#pragma unroll
-      for (int t = 1; t < S::STEPS; ++t) pm = fmaxf(pm, sc[t][gg]);
-#pragma unroll
-      for (int o = S::LPK; o < 32; o <<= 1) pm = fmaxf(pm, __shfl_xor_sync(0xffffffffu, pm, o));
-      if (pm > run_m[gg]) {
-        const float cr = exp2f(run_m[gg] - pm);  // 0 when run_m was -inf
-        run_l[gg] *= cr;
-#pragma unroll
-        for (int e = 0; e < S::VEC; ++e) acc[gg][e] *= cr;
-        run_m[gg] = pm;
-      }
-    }
-#pragma unroll
-    for (int t = 0; t < S::STEPS; ++t) {
-      const int key = warp * S::KEYS_PER_WARP + t * S::KPW + grp;
-      if (usable(key)) {
-        float vv[S::VEC];
-        Vec16<T>::load(sv + key * HD + part_lane * S::VEC, vv);
-#pragma unroll
-        for (int gg = 0; gg < G; ++gg) {
-          const float pr = exp2f(sc[t][gg] - run_m[gg]);
-          run_l[gg] += pr;
-#pragma unroll
-          for (int e = 0; e < S::VEC; ++e) acc[gg][e] = fmaf(pr, vv[e], acc[gg][e]);
+          for (int e = 0; e < S::VEC; ++e) acc[gg][e] *= cr;
+          run_m[gg] = pm;
         }
       }
+#pragma unroll
+      for (int t = 0; t < S::STEPS; ++t) {
+        const int key = team_warp * S::KEYS_PER_WARP + t * S::KPW + grp;
+        if (usable(key)) {
+          float vv[S::VEC];
+          Vec16<T>::load(sv + key * HD + part_lane * S::VEC, vv);
+#pragma unroll
+          for (int gg = 0; gg < G; ++gg) {
+            const float pr = exp2f(sc[t][gg] - run_m[gg]);
+            run_l[gg] += pr;
+#pragma unroll
+            for (int e = 0; e < S::VEC; ++e) acc[gg][e] = fmaf(pr, vv[e], acc[gg][e]);
+          }
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&empty[st]));
     }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(smem_u32(&empty[st]));
 
     const bool item_end = (g + 1 == pages_of(k));
     if (item_end || p + 1 == p1) {
       // ---- this CTA's part of item (k, h) is done: merge the lane groups, then the warps ----
+      float* mred = red + (S::REDS == 2 && odd ? ATT_WARPS * PSZ : 0);
+      odd = !odd;
 #pragma unroll
       for (int gg = 0; gg < G; ++gg) {
 #pragma unroll
@@ -286,7 +302,7 @@ __global__ void __launch_bounds__(ATT_THREADS) k_attn_decode(ModelDims md, StepD
       if (grp == 0) {
 #pragma unroll
         for (int gg = 0; gg < G; ++gg) {
-          float* rw = red + (warp * G + gg) * (HD + 2);
+          float* rw = mred + (warp * G + gg) * (HD + 2);
 #pragma unroll
           for (int e = 0; e < S::VEC; ++e) rw[part_lane * S::VEC + e] = acc[gg][e];
           if (part_lane == 0) {
@@ -307,11 +323,11 @@ __global__ void __launch_bounds__(ATT_THREADS) k_attn_decode(ModelDims md, StepD
         const int gg = t / HD, e = t % HD;
         float mx = -INFINITY;
 #pragma unroll
-        for (int w = 0; w < ATT_WARPS; ++w) mx = fmaxf(mx, red[(w * G + gg) * (HD + 2) + HD]);
+        for (int w = 0; w < ATT_WARPS; ++w) mx = fmaxf(mx, mred[(w * G + gg) * (HD + 2) + HD]);
         float o = 0.f, l = 0.f;
 #pragma unroll
         for (int w = 0; w < ATT_WARPS; ++w) {
-          const float* rw = red + (w * G + gg) * (HD + 2);
+          const float* rw = mred + (w * G + gg) * (HD + 2);
           const float f = (rw[HD] == -INFINITY) ? 0.f : exp2f(rw[HD] - mx);
           o = fmaf(f, rw[e], o);
           l = fmaf(f, rw[HD + 1], l);
@@ -354,7 +370,8 @@ __global__ void __launch_bounds__(ATT_THREADS) k_attn_decode(ModelDims md, StepD
           if (tid == 0) cnt[item] = 0;  // ready for the next launch
         }
       }
-      consumer_sync();  // `red` and `flag` are reused by the next item
+      // `red` and `flag` are reused by the next item (a second buffer waits for the barrier of the item between)
+      if (S::REDS == 1 || nparts > 1) consumer_sync();
       if (p + 1 < p1) {
         g = 0;
         if (++h == Hkv) {
