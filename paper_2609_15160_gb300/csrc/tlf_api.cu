@@ -75,6 +75,7 @@ struct tlf_ctx {
   bool split_norm = false;      // pre-norms split across the neighbouring GEMMs (tcgen05 path)
   bool operand_lo = false;      // X, O, U carry a lo plane (two-term GEMM operands, tcgen05 path)
   bool pf_ws = true;            // prefill attention: the warp-specialised tensor-map kernel
+  bool step_row = false;        // float32 steps over short caches run the block one CTA per row
   bool step_small = false;      // steps of up to 16 rows run the block in the persistent kernel
   float* d_part_small = nullptr;  // its attention partials
   float* d_ss8 = nullptr;       // [16][d / 8] its sums of squares
@@ -161,7 +162,7 @@ struct tlf_ctx {
   // CUDA graphs of the step
   struct StepGraph {
     int B;
-    bool logits;
+    bool logits, rows;
     cudaGraphExec_t exec;
     int launches;
   };
@@ -607,6 +608,7 @@ static int create_impl(tlf_ctx* ctx, const tlf_weights* w) {
     const char* e = getenv("TLF_NO_SPLIT_NORM");
     ctx->split_norm = ctx->use_tc && !(e && e[0] == '1');
   }
+  ctx->step_row = c.ablation == TLF_ABLATION_NONE && step_row_fits(md);
   ctx->step_small = ctx->split_norm && ctx->operand_lo && c.ablation == TLF_ABLATION_NONE &&
                     step_small_fits(md, ctx->num_sms);
   if (ctx->step_small) {
@@ -794,7 +796,8 @@ static CondArgs cond_args(const tlf_ctx* ctx, const int* m, int r, int j, int pa
   return c;
 }
 
-static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, bool prof, cudaStream_t st) {
+// rows: the block one CTA per row (float32 models; every cache of the step holds at most RowStep::MAX_KEYS entries).
+static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, bool rows, bool prof, cudaStream_t st) {
   const ModelDims& md = ctx->md;
   const int M = md.M, J = md.J, maxB = md.max_batch;
   CK(ctx, cudaMemcpyAsync(ctx->d_upload, ctx->h_upload, ctx->upload_ints * 4, cudaMemcpyHostToDevice, st));
@@ -869,7 +872,22 @@ static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, bool prof, cudaSt
     CK(ctx, launch_step_small(a, ctx->num_sms, st));
     ctx->last_launches += 2;
   }
-  for (int r = 0; r < M && !small; ++r) {
+  if (rows) {
+    RowStep a{};
+    a.md = md;
+    a.s = s;
+    for (int j = 0; j < J; ++j)
+      a.layer[j] = {(const float*)ctx->wqkv[j].ptr, (const float*)ctx->wo[j].ptr, (const float*)ctx->wgu[j].ptr,
+                    (const float*)ctx->wd[j].ptr, ctx->d_attn_norm + (size_t)j * md.d, ctx->d_mlp_norm + (size_t)j * md.d};
+    a.rope = ctx->d_rope;
+    a.cond = ctx->d_cond;
+    a.final_norm = ctx->d_final_norm;
+    a.Xf = reinterpret_cast<float*>(ctx->d_Xf);
+    a.keys = RowStep::MAX_KEYS;
+    CK(ctx, launch_step_row(a, B, st));
+    ctx->last_launches += 1;
+  }
+  for (int r = 0; r < M && !small && !rows; ++r) {
     const int* n_dev = ctx->d_n + r;
     const int* idx_r = ctx->d_idx + (size_t)r * maxB;
     // rows that do not run loop r but are computed anyway (no-gather ablation) keep their residual
@@ -999,9 +1017,11 @@ static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, bool prof, cudaSt
       ++ctx->last_launches;  // the attention (GEMMs counted in gemm(), norms where launched)
     }
   }
-  launch_final(md, s, B, ctx->d_final_norm, ctx->d_Xf, st);
-  mark(11);
-  ++ctx->last_launches;
+  if (!rows) {
+    launch_final(md, s, B, ctx->d_final_norm, ctx->d_Xf, st);
+    mark(11);
+    ++ctx->last_launches;
+  }
   if (need_logits) {
     GemmArgs a{};
     a.n_host = B;
@@ -1022,9 +1042,9 @@ static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, bool prof, cudaSt
 
 // The step as one CUDA graph per (batch size, logits on/off), built on first
 // use after the kernels have run once directly (their attributes are set).
-static cudaGraphExec_t step_graph(tlf_ctx* ctx, int B, bool need_logits) {
+static cudaGraphExec_t step_graph(tlf_ctx* ctx, int B, bool need_logits, bool rows) {
   for (auto& g : ctx->graphs)
-    if (g.B == B && g.logits == need_logits) {
+    if (g.B == B && g.logits == need_logits && g.rows == rows) {
       ctx->last_launches = g.launches;
       return g.exec;
     }
@@ -1036,7 +1056,7 @@ static cudaGraphExec_t step_graph(tlf_ctx* ctx, int B, bool need_logits) {
     ctx->use_graphs = false;
     return nullptr;
   }
-  const int rc = enqueue_step(ctx, B, need_logits, false, ctx->cap_stream);
+  const int rc = enqueue_step(ctx, B, need_logits, rows, false, ctx->cap_stream);
   const cudaError_t e1 = cudaStreamEndCapture(ctx->cap_stream, &graph);
   if (rc != TLF_OK || e1 != cudaSuccess || cudaGraphInstantiate(&exec, graph, 0) != cudaSuccess) {
     cudaGetLastError();
@@ -1045,7 +1065,7 @@ static cudaGraphExec_t step_graph(tlf_ctx* ctx, int B, bool need_logits) {
     return nullptr;
   }
   cudaGraphDestroy(graph);
-  ctx->graphs.push_back({B, need_logits, exec, ctx->last_launches});
+  ctx->graphs.push_back({B, need_logits, rows, exec, ctx->last_launches});
   return exec;
 }
 
@@ -1063,11 +1083,13 @@ static int run_step(tlf_ctx* ctx, int B, const int* slots, const int* tokens, co
     h[1 + 2 * B + b] = slots[b];
   }
   memcpy(h + 1 + 3 * B, upd.data(), nu * sizeof(PageUpdate));
-  cudaGraphExec_t exec = prof ? nullptr : step_graph(ctx, B, need_logits);
+  bool rows = ctx->step_row && !prof;
+  for (int b = 0; b < B && rows; ++b) rows = ctx->h_len[(size_t)slots[b] * M] + 1 <= RowStep::MAX_KEYS;
+  cudaGraphExec_t exec = prof ? nullptr : step_graph(ctx, B, need_logits, rows);
   if (exec) {
     CK(ctx, cudaGraphLaunch(exec, st));
   } else {
-    const int rc = enqueue_step(ctx, B, need_logits, prof, st);
+    const int rc = enqueue_step(ctx, B, need_logits, rows, prof, st);
     if (rc) return rc;
     ctx->warmed = true;
   }

@@ -551,6 +551,26 @@ struct SmallStep {
   unsigned* gbar;
   int w1_bytes, w2_bytes, nst;  // shared-memory layout (set by the launcher)
 };
+// The block of a step of a small float32 model, one CTA per row (k_step_row.cu), final norm and cache lengths included.
+struct RowLayer {
+  const float *wqkv, *wo, *wgu, *wd;  // row-major, gate rows before up rows
+  const float *attn_norm, *mlp_norm;
+};
+struct RowStep {
+  static constexpr int MAX_KEYS = 1024;  // longest cache a row may attend to
+  ModelDims md;
+  StepDev s;
+  RowLayer layer[SS_LAYERS];
+  const float2* rope;
+  const float* cond;        // conditioning table (NULL: none)
+  const float* final_norm;
+  float* Xf;                // [B][d] the LM head's operand
+  int keys;                 // at least the longest cache of the step, the new entry included
+  int max_keys, weights_in_smem;  // set by the launcher
+};
+bool step_row_fits(const ModelDims& md);
+cudaError_t launch_step_row(RowStep a, int B, cudaStream_t st);
+
 bool step_small_fits(const ModelDims& md, int num_sms);
 size_t step_small_part_floats(const ModelDims& md, int num_sms);  // floats of SmallStep::part
 cudaError_t launch_step_small(SmallStep a, int num_sms, cudaStream_t st);
