@@ -531,8 +531,11 @@ static int create_impl(tlf_ctx* ctx, const tlf_weights* w) {
   ctx->upload_ints = (size_t)3 * B + 2 * (size_t)B * M + 16;
   if ((rc = dev_alloc(ctx, &ctx->d_upload, ctx->upload_ints * 4, "upload"))) return rc;
   CK(ctx, cudaMallocHost((void**)&ctx->h_upload, ctx->upload_ints * 4));
-  if ((rc = dev_alloc(ctx, &ctx->d_m, (size_t)B * 4, "m"))) return rc;
-  if ((rc = dev_alloc(ctx, &ctx->d_margin, (size_t)B * 4, "margin"))) return rc;
+  // loop counts, margins and the error word side by side: a step's results come to the host in one copy
+  const size_t result_bytes = (size_t)2 * B * 4 + 16;
+  if ((rc = dev_alloc(ctx, &ctx->d_m, result_bytes, "step results"))) return rc;
+  ctx->d_margin = reinterpret_cast<float*>(ctx->d_m + B);
+  ctx->d_err = reinterpret_cast<uint32_t*>(ctx->d_m + 2 * B);
   if ((rc = dev_alloc(ctx, &ctx->d_H, (size_t)B * d * 4, "H"))) return rc;
   {
     // two-term operands (hi + lo planes) for every decode GEMM of the tcgen05 path;
@@ -620,11 +623,10 @@ static int create_impl(tlf_ctx* ctx, const tlf_weights* w) {
   }
   CK(ctx, cudaMemset(ctx->d_attn_cnt, 0, (size_t)B * md.Hkv * 4));
   if ((rc = dev_alloc(ctx, &ctx->d_logits, (size_t)B * V * 4, "logits"))) return rc;
-  if ((rc = dev_alloc(ctx, &ctx->d_err, 16, "error word"))) return rc;
-  CK(ctx, cudaMemset(ctx->d_err, 0, 16));
-  CK(ctx, cudaMallocHost((void**)&ctx->h_m, (size_t)B * 4));
-  CK(ctx, cudaMallocHost((void**)&ctx->h_margin, (size_t)B * 4));
-  CK(ctx, cudaMallocHost((void**)&ctx->h_err, 16));
+  CK(ctx, cudaMemset(ctx->d_m, 0, result_bytes));
+  CK(ctx, cudaMallocHost((void**)&ctx->h_m, result_bytes));
+  ctx->h_margin = reinterpret_cast<float*>(ctx->h_m + B);
+  ctx->h_err = reinterpret_cast<uint32_t*>(ctx->h_m + 2 * B);
   CK(ctx, cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking));
   {
     const char* e = getenv("TLF_NO_GRAPH");
@@ -647,13 +649,11 @@ extern "C" void tlf_destroy(tlf_ctx* ctx) {
     for (auto* v : {&ctx->wqkv, &ctx->wo, &ctx->wgu, &ctx->wd})
       for (auto& m : *v) f(m.ptr);
     f(ctx->d_pool); f(ctx->d_pos_table); f(ctx->d_page_table); f(ctx->d_len); f(ctx->d_upload);
-    f(ctx->d_m); f(ctx->d_margin); f(ctx->d_H); f(ctx->d_X); f(ctx->d_O); f(ctx->d_U); f(ctx->d_Xf);
+    f(ctx->d_m); f(ctx->d_H); f(ctx->d_X); f(ctx->d_O); f(ctx->d_U); f(ctx->d_Xf);
     f(ctx->d_part); f(ctx->d_Q); f(ctx->d_idx); f(ctx->d_n); f(ctx->d_item_base); f(ctx->d_nch); f(ctx->d_chunk);
-    f(ctx->d_attn_part); f(ctx->d_attn_cnt); f(ctx->d_logits); f(ctx->d_err);
+    f(ctx->d_attn_part); f(ctx->d_attn_cnt); f(ctx->d_logits);
     if (ctx->h_upload) cudaFreeHost(ctx->h_upload);
     if (ctx->h_m) cudaFreeHost(ctx->h_m);
-    if (ctx->h_margin) cudaFreeHost(ctx->h_margin);
-    if (ctx->h_err) cudaFreeHost(ctx->h_err);
     for (auto e : ctx->events) if (e) cudaEventDestroy(e);
     for (auto& g : ctx->graphs) cudaGraphExecDestroy(g.exec);
     f(ctx->d_pf_in); f(ctx->d_pf_m); f(ctx->d_pf_margin); f(ctx->d_pf_H); f(ctx->d_pf_X); f(ctx->d_pf_Q);
@@ -1034,9 +1034,7 @@ static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, bool rows, bool p
     mark(12);
   }
   CK(ctx, cudaGetLastError());
-  CK(ctx, cudaMemcpyAsync(ctx->h_m, ctx->d_m, (size_t)B * 4, cudaMemcpyDeviceToHost, st));
-  CK(ctx, cudaMemcpyAsync(ctx->h_margin, ctx->d_margin, (size_t)B * 4, cudaMemcpyDeviceToHost, st));
-  CK(ctx, cudaMemcpyAsync(ctx->h_err, ctx->d_err, 4, cudaMemcpyDeviceToHost, st));
+  CK(ctx, cudaMemcpyAsync(ctx->h_m, ctx->d_m, (size_t)2 * maxB * 4 + 4, cudaMemcpyDeviceToHost, st));
   return TLF_OK;
 }
 
@@ -1069,8 +1067,9 @@ static cudaGraphExec_t step_graph(tlf_ctx* ctx, int B, bool need_logits, bool ro
   return exec;
 }
 
+// logits: where the step's logits go behind it (NULL: they stay in d_logits).
 static int run_step(tlf_ctx* ctx, int B, const int* slots, const int* tokens, const int* forced,
-                    const std::vector<PageUpdate>& upd, bool need_logits, cudaStream_t st) {
+                    const std::vector<PageUpdate>& upd, bool need_logits, cudaStream_t st, float* logits = nullptr) {
   const ModelDims& md = ctx->md;
   const int M = md.M, J = md.J;
   const bool prof = ctx->profiling;
@@ -1093,6 +1092,9 @@ static int run_step(tlf_ctx* ctx, int B, const int* slots, const int* tokens, co
     if (rc) return rc;
     ctx->warmed = true;
   }
+  if (logits)  // queued behind the step, so one wait covers both
+    CK(ctx, cudaMemcpyAsync(logits, ctx->d_logits, (size_t)B * md.V * 4,
+                            is_device_ptr(logits) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st));
   CK(ctx, cudaStreamSynchronize(st));
   if (*ctx->h_err) {
     const uint32_t e = *ctx->h_err;
@@ -1163,17 +1165,11 @@ extern "C" int tlf_decode_step(tlf_ctx* ctx, int32_t batch, const uint64_t* seq_
   if (rc) return rc;
   cudaStream_t st = (cudaStream_t)stream;
   const bool want = logits != nullptr;
-  rc = run_step(ctx, batch, slots.data(), tokens, forced, upd, want, st);
+  rc = run_step(ctx, batch, slots.data(), tokens, forced, upd, want, st, logits);
   if (rc) return rc;
   advance_lengths(ctx, batch, slots.data());
   for (int b = 0; b < batch; ++b) loops[b] = ctx->h_m[b];
   if (router_margin) memcpy(router_margin, ctx->h_margin, (size_t)batch * 4);
-  if (want) {
-    const size_t bytes = (size_t)batch * ctx->md.V * 4;
-    if (is_device_ptr(logits)) CK(ctx, cudaMemcpyAsync(logits, ctx->d_logits, bytes, cudaMemcpyDeviceToDevice, st));
-    else CK(ctx, cudaMemcpyAsync(logits, ctx->d_logits, bytes, cudaMemcpyDeviceToHost, st));
-    CK(ctx, cudaStreamSynchronize(st));
-  }
   return TLF_OK;
 }
 
