@@ -11,9 +11,10 @@
 //   hint, because each tile is read once per launch.
 // - Warp 1 lane 0 issues tcgen05.mma (M=128, K=16) accumulating in TMEM and
 //   releases each stage with tcgen05.commit.
-// - All four warps then read the accumulator with tcgen05.ld (warp w owns TMEM
-//   lanes 32w..32w+31 = output features) and run the epilogue. Split-K over
-//   gridDim.y keeps enough CTAs in flight to stream the weights at HBM speed.
+// - All warps then read the accumulator with tcgen05.ld (warp w owns TMEM lanes
+//   32 (w % 4).. + 31 = output features) and run the epilogue, each group of four
+//   warps on its share of the token columns. Split-K over gridDim.y keeps enough
+//   CTAs in flight to stream the weights at HBM speed.
 // Two-term operands (decode): the token operand arrives as bf16 hi and lo
 // planes, loaded as one B tile of 2 x NT rows; the MMA runs with N = 2 x NT
 // (two MMAs of N = 256 for a 256-token tile, whose halves fill TMEM) and the
@@ -66,6 +67,12 @@ __device__ __forceinline__ void gemm_write(const GemmArgs& a, int split, int row
 // ----------------------------------------------------------------------------
 constexpr int TC_BM = 128;
 constexpr int TC_BK = 64;  // 64 bf16 = one 128-byte swizzle row
+// Threads of a CTA. The epilogue of a wide token tile is bound by its chain of loads and stores per column, one thread
+// per feature, so groups of 128 threads share the columns. Measured with the mid-size model, 4 warps against these
+// counts: a decode step of 200 rows 2960 -> 2640 us, of 100 rows 1710 -> 1630 us; a prompt of 256 tokens
+// 2270 -> 1810 us. With 8 warps for 256 tokens these take 2720 and 1890 us; 16 for a two-plane tile of 128 take 1810 us
+// at 100 rows, as many registers leave no room for a second CTA. Narrower tiles have too few columns to share.
+constexpr int tc_threads(int nt, bool lo) { return nt >= (lo ? 256 : 64) ? 512 : nt >= (lo ? 64 : 32) ? 256 : 128; }
 constexpr int TC_STAGES = 4;  // deepest operand ring; a launch uses min(4, k-tiles per CTA) stages
 
 // Dynamic shared memory of one CTA: the operand ring (reused after the main loop
@@ -154,13 +161,24 @@ __device__ __forceinline__ void cluster_cols(int n, int S, int& c0, int& c1) {
   c1 = min(n, c0 + per);
 }
 
-template <int NT>
+// The columns among [c0, c1) of this thread's group of 128 threads.
+template <int NT, bool LO>
+__device__ __forceinline__ void group_cols(int c0, int c1, int& g0, int& g1) {
+  constexpr int GROUPS = tc_threads(NT, LO) / 128;
+  const int per = (max(0, c1 - c0) + GROUPS - 1) / GROUPS;
+  g0 = c0 + (int)(threadIdx.x >> 7) * per;
+  g1 = min(c1, g0 + per);
+}
+
+template <int NT, bool LO>
 __device__ void cluster_epilogue(const GemmArgs& a, float* red, int4* ci, const float* scale, float* ssp,
                                  const float (&hpre)[HPRE], int m0, int n) {
   const int S = a.splits;
-  int c0, c1;
+  int c0, c1;  // the CTA's columns
   cluster_cols(n, S, c0, c1);
-  const int tid = threadIdx.x;
+  int g0, g1;  // this thread group's columns among them
+  group_cols<NT, LO>(c0, c1, g0, g1);
+  const int tid = threadIdx.x & 127;  // feature of the tile
   uint32_t pb[CL_MAX];
   const uint32_t base = smem_u32(red);
 #pragma unroll
@@ -170,12 +188,12 @@ __device__ void cluster_epilogue(const GemmArgs& a, float* red, int4* ci, const 
     const int col = m0 + tid;
     if (!a.xn) {
       if (col < a.N)
-        for (int c = c0; c < c1; c += 4) {
+        for (int c = g0; c < g1; c += 4) {
           float sm[4];
-          cluster_sum4(pb, red, S, tid, c, c1, sm);
+          cluster_sum4(pb, red, S, tid, c, g1, sm);
 #pragma unroll
           for (int q = 0; q < 4; ++q)
-            if (c + q < c1 && ci[c + q].w >= 0) {  // the only writer of this element
+            if (c + q < g1 && ci[c + q].w >= 0) {  // the only writer of this element
               const float g = a.alpha.mod ? a.alpha.mod[ci[c + q].x + col] : 1.f;
               atomicAdd(a.resid + (size_t)ci[c + q].w * a.ldr + col, g * sm[q]);
             }
@@ -215,34 +233,34 @@ __device__ void cluster_epilogue(const GemmArgs& a, float* red, int4* ci, const 
       if (lane == 0)
 #pragma unroll
         for (int q = 0; q < Q; ++q)
-          if (c + q < c1 && ci[c + q].z >= 0) ssp[warp * NT + c + q] = t[q];
+          if (c + q < g1 && ci[c + q].z >= 0) ssp[warp * NT + c + q] = t[q];
     };
-    if (c1 - c0 <= HPRE) {
+    if (g1 - g0 <= HPRE) {
       float sm[HPRE];
 #pragma unroll
-      for (int q = 0; q < HPRE; q += 4) cluster_sum4(pb, red, S, tid, c0 + q, c1, sm + q);
+      for (int q = 0; q < HPRE; q += 4) cluster_sum4(pb, red, S, tid, g0 + q, g1, sm + q);
       float t[HPRE];
 #pragma unroll
-      for (int q = 0; q < HPRE; ++q) t[q] = (c0 + q < c1) ? update(c0 + q, hpre[q], sm[q]) : 0.f;
-      sums(c0, t, std::integral_constant<int, HPRE>{});
+      for (int q = 0; q < HPRE; ++q) t[q] = (g0 + q < g1) ? update(g0 + q, hpre[q], sm[q]) : 0.f;
+      sums(g0, t, std::integral_constant<int, HPRE>{});
     } else {
-      for (int c = c0; c < c1; c += 4) {
+      for (int c = g0; c < g1; c += 4) {
         float hv[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          const int w = (c + q < c1) ? ci[c + q].w : -1;
-          hv[q] = (fin && c + q < c1) ? a.resid[(size_t)(w >= 0 ? w : ~w) * a.ldr + col] : 0.f;
+          const int w = (c + q < g1) ? ci[c + q].w : -1;
+          hv[q] = (fin && c + q < g1) ? a.resid[(size_t)(w >= 0 ? w : ~w) * a.ldr + col] : 0.f;
         }
         float sm[4];
-        cluster_sum4(pb, red, S, tid, c, c1, sm);
+        cluster_sum4(pb, red, S, tid, c, g1, sm);
         float t[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) t[q] = (c + q < c1) ? update(c + q, hv[q], sm[q]) : 0.f;
+        for (int q = 0; q < 4; ++q) t[q] = (c + q < g1) ? update(c + q, hv[q], sm[q]) : 0.f;
         sums(c, t, std::integral_constant<int, 4>{});
       }
     }
     __syncthreads();
-    for (int c = c0 + tid; c < c1; c += blockDim.x) {
+    for (int c = c0 + (int)threadIdx.x; c < c1; c += blockDim.x) {
       const int dst = ci[c].z;
       if (dst >= 0)
         a.ss_out[(size_t)dst * a.ldss + m0 / TC_BM] = ssp[c] + ssp[NT + c] + ssp[2 * NT + c] + ssp[3 * NT + c];
@@ -251,11 +269,11 @@ __device__ void cluster_epilogue(const GemmArgs& a, float* red, int4* ci, const 
   }
   // With a pair of rows per output (gate and up, or the two halves of a rotary pair), the
   // threads of the pair's upper row take the second half of the token columns.
-  const int cm = c0 + (c1 - c0 + 1) / 2;
+  const int cm = g0 + (g1 - g0 + 1) / 2;
   if (a.epi == EPI_CL_SWIGLU) {
     const int f = tid & 63, hs = tid >> 6;
     const int gf = (m0 >> 1) + f;  // 64 gate rows then 64 up rows per 128-row tile
-    const int ca = hs ? cm : c0, cb = hs ? c1 : cm;
+    const int ca = hs ? cm : g0, cb = hs ? g1 : cm;
     if (gf < a.md.ff)
       for (int c = ca; c < cb; c += 4) {
         float g[4], u[4];
@@ -281,7 +299,7 @@ __device__ void cluster_epilogue(const GemmArgs& a, float* red, int4* ci, const 
   const int ps = md.page_size, hd = md.hd, half = hd / 2;
   if (a.row_cslot) {
     // prefill: sequence slot, cache slot and position of each row from the prefill plan
-    for (int c = c0 + tid; c < c1; c += blockDim.x) {
+    for (int c = c0 + (int)threadIdx.x; c < c1; c += blockDim.x) {
       const int slot = a.row_slot[c], L = a.row_cslot[c];
       int pos = a.row_pos[c];
       int page = s.page_table[((size_t)slot * md.M + a.r) * md.max_pages + L / ps];
@@ -305,7 +323,7 @@ __device__ void cluster_epilogue(const GemmArgs& a, float* red, int4* ci, const 
     const int h = fr / hd, hs = (fr % hd) >= half;
     const int i = (fr % hd) - hs * half;   // rotary pair (i, i + half) of head h
     const int tlo = tid - hs * half;       // tile row of the pair's lower element
-    const int ca = hs ? cm : c0, cb = hs ? c1 : cm;
+    const int ca = hs ? cm : g0, cb = hs ? g1 : cm;
     for (int c = ca; c < cb; c += 4) {
       float2 csn[4];
 #pragma unroll
@@ -348,13 +366,13 @@ __device__ void cluster_epilogue(const GemmArgs& a, float* red, int4* ci, const 
   } else {
     const int fr = gfeat - md.q_dim - md.kv_dim;
     const int h = fr / hd, i = fr % hd;
-    for (int c = c0; c < c1; c += 4) {
+    for (int c = g0; c < g1; c += 4) {
       float x[4];
-      cluster_sum4(pb, red, S, tid, c, c1, x);
+      cluster_sum4(pb, red, S, tid, c, g1, x);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int cc = c + q;
-        if (cc < c1 && ci[cc].x >= 0) {
+        if (cc < g1 && ci[cc].x >= 0) {
           bf16* vp = pool + (size_t)ci[cc].x * md.page_elems + ((size_t)(a.j * 2 + 1) * md.Hkv + h) * ps * hd +
                      (size_t)ci[cc].y * hd;
           vp[i] = __float2bfloat16_rn(a.ss_in ? x[q] * scale[cc] : x[q]);
@@ -378,7 +396,7 @@ __device__ __forceinline__ void tmem_ld_acc(uint32_t taddr, int lo_off, float* v
 // LO: the token operand is two-term (hi + lo planes); a compile-time choice, so the one-plane
 // instantiations (prefill, the LM head) carry none of its code.
 template <int NT, bool LO>
-__global__ void __launch_bounds__(128) k_gemm_tc(const __grid_constant__ CUtensorMap mapW,
+__global__ void __launch_bounds__(tc_threads(NT, LO)) k_gemm_tc(const __grid_constant__ CUtensorMap mapW,
                                                  const __grid_constant__ CUtensorMap mapX, GemmArgs a) {
   constexpr int A_BYTES = TC_BM * TC_BK * 2;
   constexpr bool lo = LO;
@@ -469,7 +487,7 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const __grid_constant__ CUtenso
     if (warp >= 2) {
       // idle during the main loop: fetch what the epilogue needs per token column
       // (outputs of the plan kernel and of the preceding GEMM, read after the wait)
-      for (int c = threadIdx.x - 64; c < n; c += 64) {
+      for (int c = threadIdx.x - 64; c < n; c += tc_threads(NT, LO) - 64) {
         if (a.ss_in) {
           // split norm: the column's factor from the producer's per-tile sums of squares
           const float4* p4 = reinterpret_cast<const float4*>(a.ss_in + (size_t)c * a.ldss);
@@ -536,20 +554,24 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const __grid_constant__ CUtenso
 #pragma unroll
   for (int q = 0; q < HPRE; ++q) hpre[q] = 0.f;
   if (a.epi == EPI_CL_RESID && a.xn) {
-    int c0, c1;
+    int c0, c1, g0, g1;
     cluster_cols(n, a.splits, c0, c1);
-    const int col = m0 + threadIdx.x;
-    if (c1 - c0 <= HPRE && col < a.N) {
+    group_cols<NT, LO>(c0, c1, g0, g1);
+    const int col = m0 + (threadIdx.x & 127);
+    if (g1 - g0 <= HPRE && col < a.N) {
 #pragma unroll
       for (int q = 0; q < HPRE; ++q)
-        if (c0 + q < c1) {
-          const int row = a.idx ? a.idx[c0 + q] : c0 + q;
+        if (g0 + q < g1) {
+          const int row = a.idx ? a.idx[g0 + q] : g0 + q;
           hpre[q] = a.resid[(size_t)row * a.ldr + col];
         }
     }
   }
 
-  // Epilogue: warp w holds output features m0 + 32w + lane; columns are token rows.
+  // Epilogue: warp w holds output features m0 + 32 (w % 4) + lane; columns are token rows, 16 at a time by the groups of
+  // four warps in turn.
+  constexpr int GROUPS = tc_threads(NT, LO) / 128;
+  const int quad = warp & 3, group = warp >> 2;
   bool ok = true;
   if (nk > 0) ok = mbar_wait(done, 0, a.err);
   ok = __all_sync(0xffffffffu, ok);  // tcgen05.ld is warp-collective
@@ -559,11 +581,11 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const __grid_constant__ CUtenso
     // then reduce across the cluster. Every CTA reaches both cluster barriers.
     // tile layout [column][128 features]: a warp's partner reads are 128 contiguous bytes
     float* red = reinterpret_cast<float*>(smem);
-    const int f = warp * 32 + lane;
-    for (int c0 = 0; c0 < ncols; c0 += 16) {
+    const int f = quad * 32 + lane;
+    for (int c0 = 16 * group; c0 < ncols; c0 += 16 * GROUPS) {
       float v[16];
       if (ok && nk > 0) {
-        tmem_ld_acc(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, lo ? NT : 0, v);
+        tmem_ld_acc(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)c0, lo ? NT : 0, v);
       } else {
 #pragma unroll
         for (int i = 0; i < 16; ++i) v[i] = 0.f;
@@ -575,17 +597,17 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const __grid_constant__ CUtenso
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, TMEM_COLS);
     cluster_sync_all();  // every partner's tile is staged
-    cluster_epilogue<NT>(a, red, colinfo, colscale, ssp, hpre, m0, n);
+    cluster_epilogue<NT, LO>(a, red, colinfo, colscale, ssp, hpre, m0, n);
     __syncwarp();
     cluster_sync_all();  // partners have finished reading this CTA's tile
     return;
   }
   if (ok) {
-    const int col = m0 + warp * 32 + lane;
-    for (int c0 = 0; c0 < ncols; c0 += 16) {
+    const int col = m0 + quad * 32 + lane;
+    for (int c0 = 16 * group; c0 < ncols; c0 += 16 * GROUPS) {
       float v[16];
       if (nk > 0) {
-        tmem_ld_acc(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, lo ? NT : 0, v);
+        tmem_ld_acc(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)c0, lo ? NT : 0, v);
       } else {
 #pragma unroll
         for (int i = 0; i < 16; ++i) v[i] = 0.f;
@@ -620,7 +642,7 @@ static void launch_tc_nt(const CUtensorMap* mapW, const CUtensorMap* mapX, GemmA
   const int smem = tc_smem_bytes(NT, a.stages, LO);
   dim3 grid((a.N + TC_BM - 1) / TC_BM, a.splits);
   if (a.epi < EPI_CL_RESID) {
-    launch_k(k_gemm_tc<NT, LO>, grid, 128, smem, st, *mapW, *mapX, a);
+    launch_k(k_gemm_tc<NT, LO>, grid, tc_threads(NT, LO), smem, st, *mapW, *mapX, a);
     return;
   }
   // cluster epilogue: the splits of one tile form a (1, splits, 1) cluster
@@ -628,7 +650,7 @@ static void launch_tc_nt(const CUtensorMap* mapW, const CUtensorMap* mapX, GemmA
     (void)ensure_kernel_attrs((const void*)k_gemm_tc<NT, LO>, tc_smem_bytes(NT, tc_max_stages(NT, LO), LO), true);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
-  cfg.blockDim = dim3(128);
+  cfg.blockDim = dim3(tc_threads(NT, LO));
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];

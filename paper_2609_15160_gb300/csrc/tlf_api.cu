@@ -138,8 +138,7 @@ struct tlf_ctx {
   float* d_pf_Q = nullptr;
   void* d_pf_O = nullptr;
   void* d_pf_U = nullptr;
-  CUtensorMap pf_map_X, pf_map_O, pf_map_U;     // boxes of 256 rows
-  CUtensorMap pf_pair_X, pf_pair_O, pf_pair_U;  // boxes of 128 rows
+  CUtensorMap pf_map_X[5], pf_map_O[5], pf_map_U[5];  // boxes of 16, 32, 64, 128 and 256 rows
   CUtensorMap pf_map_Q;                         // q planes, for the pair attention (has_pool_map)
   int pf_pairs = 0;                             // SM pairs the prefill GEMM's persistent grid may fill
   int *d_pf_idx = nullptr, *d_pf_n = nullptr, *d_pf_row_slot = nullptr, *d_pf_row_cslot = nullptr,
@@ -1209,12 +1208,12 @@ static int ensure_prefill_buffers(tlf_ctx* ctx) {
   CK(ctx, cudaMemset(ctx->d_pf_X, 0, (size_t)C * d * 2));
   CK(ctx, cudaMemset(ctx->d_pf_O, 0, (size_t)C * md.q_dim * 2));
   CK(ctx, cudaMemset(ctx->d_pf_U, 0, (size_t)C * md.ff * 2));
-  if (!make_map(&ctx->pf_map_X, ctx->d_pf_X, C, d, d, 256) ||
-      !make_map(&ctx->pf_map_O, ctx->d_pf_O, C, md.q_dim, md.q_dim, 256) ||
-      !make_map(&ctx->pf_map_U, ctx->d_pf_U, C, md.ff, md.ff, 256) ||
-      !make_map(&ctx->pf_pair_X, ctx->d_pf_X, C, d, d, 128) ||
-      !make_map(&ctx->pf_pair_O, ctx->d_pf_O, C, md.q_dim, md.q_dim, 128) ||
-      !make_map(&ctx->pf_pair_U, ctx->d_pf_U, C, md.ff, md.ff, 128))
+  bool maps = true;
+  for (int i = 0; i < 5; ++i)
+    maps = maps && make_map(&ctx->pf_map_X[i], ctx->d_pf_X, C, d, d, 16 << i) &&
+           make_map(&ctx->pf_map_O[i], ctx->d_pf_O, C, md.q_dim, md.q_dim, 16 << i) &&
+           make_map(&ctx->pf_map_U[i], ctx->d_pf_U, C, md.ff, md.ff, 16 << i);
+  if (!maps)
     return fail(ctx, TLF_ERR_CUDA, "cuTensorMapEncodeTiled failed for a prefill buffer");
   if (ctx->has_pool_map && !make_q_map(&ctx->pf_map_Q, ctx->d_pf_Q, md, 2 * C))
     return fail(ctx, TLF_ERR_CUDA, "cuTensorMapEncodeTiled failed for the prefill q planes");
@@ -1231,8 +1230,8 @@ static int ensure_prefill_buffers(tlf_ctx* ctx) {
 // chip with tiles of the pair GEMM: at 8192 rows it takes 254 / 109 / 62 / 144 us for the long-context model's
 // gate/up, QKV, O and down projections, against 454 / 211 / 111 / 186 us for tiles of k_gemm_tc, and 79 / 55 / 23 / 43
 // against 186 / 124 / 47 / 66 us for the mid-size model's.
-static void gemm_pf(tlf_ctx* ctx, const DeviceMat& W, const CUtensorMap* xmap, const CUtensorMap* xpair, GemmArgs a,
-                    int rows, cudaStream_t st) {
+static void gemm_pf(tlf_ctx* ctx, const DeviceMat& W, const CUtensorMap* xmaps, GemmArgs a, int rows,
+                    cudaStream_t st) {
   a.N = W.N;
   a.K = W.K;
   a.err = ctx->d_err;
@@ -1241,11 +1240,16 @@ static void gemm_pf(tlf_ctx* ctx, const DeviceMat& W, const CUtensorMap* xmap, c
   const int ntiles = (W.N + 127) / 128, nkb = (W.K + 63) / 64;
   if (rows > 256 || ntiles > ctx->num_sms) {
     const int bn = gemm_pf_tile_n(rows, W.N, W.K, a.epi, ctx->md.hd, ctx->pf_pairs);
-    launch_gemm_pf(xpair, bn == 256 ? &W.map : bn == 128 ? &W.map64 : &W.map32, bn, a, rows, ctx->pf_pairs, st);
+    launch_gemm_pf(&xmaps[3], bn == 256 ? &W.map : bn == 128 ? &W.map64 : &W.map32, bn, a, rows, ctx->pf_pairs, st);
     return;
   }
   while (a.splits < 8 && (long long)ntiles * a.splits * 2 <= ctx->num_sms && nkb >= 4 * a.splits) a.splits *= 2;
-  launch_gemm_tc(&W.map, xmap, 256, a, st);
+  // The smallest token tile that holds the rows: less shared memory and TMEM let a kernel start beside its predecessor.
+  // The mid-size model's prompts of 4 / 64 / 117 / 256 tokens take 1184 / 1430 / 1570 / 1808 us against 1267 / 1480 /
+  // 1510 / 1807 us with 256-token tiles.
+  int i = 0;
+  while (i < 4 && rows > 16 << i) ++i;
+  launch_gemm_tc(&W.map, &xmaps[i], 16 << i, a, st);
 }
 
 // Prompts of the (already created) sequences slot_of[0..n), chunk by chunk: every chunk is routed,
@@ -1400,7 +1404,7 @@ static int prefill_batched(tlf_ctx* ctx, int n_seqs, const int* slot_of, const i
         a.row_slot = ctx->d_pf_row_slot + (size_t)r * C;
         a.row_cslot = ctx->d_pf_row_cslot + (size_t)r * C;
         a.row_pos = ctx->d_pf_row_pos + (size_t)r * C;
-        gemm_pf(ctx, ctx->wqkv[j], &ctx->pf_map_X, &ctx->pf_pair_X, a, nr, st);
+        gemm_pf(ctx, ctx->wqkv[j], ctx->pf_map_X, a, nr, st);
         // attention blocks of loop r: sum over sequences of ceil(count / qblock) <= nr / qblock + S
         const int blocks = nr / P.qblock + S + 1;
         if (pair_attn)
@@ -1414,7 +1418,7 @@ static int prefill_batched(tlf_ctx* ctx, int n_seqs, const int* slot_of, const i
         a.ldr = md.d;
         a.idx = idx_r;
         a.alpha = cond_args(ctx, ctx->d_pf_m, r, j, 0);
-        gemm_pf(ctx, ctx->wo[j], &ctx->pf_map_O, &ctx->pf_pair_O, a, nr, st);
+        gemm_pf(ctx, ctx->wo[j], ctx->pf_map_O, a, nr, st);
         launch_norm_rows(md.dtype, ctx->d_pf_H, md.d, idx_r, n_dev, 0, nr, ctx->d_mlp_norm + (size_t)j * md.d, md.d,
                          md.eps, ctx->d_pf_X, md.d, st, cond_args(ctx, ctx->d_pf_m, r, j, 3));
         a = GemmArgs{};
@@ -1422,7 +1426,7 @@ static int prefill_batched(tlf_ctx* ctx, int n_seqs, const int* slot_of, const i
         a.epi = EPI_CL_SWIGLU;
         a.md = md;
         a.U = ctx->d_pf_U;
-        gemm_pf(ctx, ctx->wgu[j], &ctx->pf_map_X, &ctx->pf_pair_X, a, nr, st);
+        gemm_pf(ctx, ctx->wgu[j], ctx->pf_map_X, a, nr, st);
         a = GemmArgs{};
         a.n_dev = n_dev;
         a.epi = EPI_CL_RESID;
@@ -1430,7 +1434,7 @@ static int prefill_batched(tlf_ctx* ctx, int n_seqs, const int* slot_of, const i
         a.ldr = md.d;
         a.idx = idx_r;
         a.alpha = cond_args(ctx, ctx->d_pf_m, r, j, 1);
-        gemm_pf(ctx, ctx->wd[j], &ctx->pf_map_U, &ctx->pf_pair_U, a, nr, st);
+        gemm_pf(ctx, ctx->wd[j], ctx->pf_map_U, a, nr, st);
       }
     }
     if (last_logits && nend > 0) {

@@ -29,6 +29,13 @@ def test_many_row_projections_conditioned(tlf):  # noqa: F811
     _prefill_decode_compare(tlf, _small(conditioning=True, d_model=192), [300, 90], steps=1)
 
 
+@pytest.mark.parametrize("shape", SHAPES, ids=str)
+@pytest.mark.parametrize("n", [1, 16, 17, 32, 33, 64, 65, 128, 129, 256])
+def test_few_row_projections(tlf, shape, n):  # noqa: F811
+    """A chunk of up to 256 rows: every token tile at its first and last size, with the CTA sizes that go with it."""
+    _prefill_decode_compare(tlf, _small(**SHAPES[shape]), [n], steps=1)
+
+
 @pytest.mark.parametrize("hd,heads,kv", [(64, 4, 4), (64, 4, 2), (64, 4, 1), (128, 2, 2), (128, 4, 2), (128, 4, 1)])
 def test_pair_attention_blocks(tlf, hd, heads, kv):  # noqa: F811
     """The two-tile prefill attention around its 128-slot key blocks and query tiles, in one chunk and in chunks whose
