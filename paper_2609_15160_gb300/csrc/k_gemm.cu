@@ -43,6 +43,7 @@
 // Other epilogues (SIMT path, LM head): split-K partial sums to a buffer
 // consumed by k_rope_append / k_swiglu, atomic residual add + scatter, or a
 // plain float32 store (logits).
+#include <algorithm>
 #include <type_traits>
 
 #include "tlf_internal.cuh"
@@ -102,7 +103,7 @@ constexpr int tc_smem_bytes(int nt, int stages, bool lo) {
   return raw > tc_min_smem(nt, lo) ? raw : tc_min_smem(nt, lo);
 }
 // Deepest operand ring of a token tile: a 256-token two-term stage holds 80 KB, so two fit.
-constexpr int tc_max_stages(int nt, bool lo) { return (lo && nt >= 256) ? 2 : TC_STAGES; }
+constexpr int tc_max_stages(int nt, bool lo) { return (lo && nt >= 256) ? 2 : (!lo && nt == 128) ? 3 : TC_STAGES; }
 constexpr bool tmem_fits(int nt, bool lo) {
   return (SM_SMEM / (tc_smem_bytes(nt, 1, lo) + 1024)) * tc_tmem_cols(nt, lo) <= 512 &&
          tc_smem_bytes(nt, tc_max_stages(nt, lo), lo) <= SM_SMEM - 1024;
@@ -624,21 +625,21 @@ __global__ void __launch_bounds__(tc_threads(NT, LO)) k_gemm_tc(const __grid_con
   if (warp == 0) tmem_dealloc(tmem, TMEM_COLS);
 }
 
-int gemm_tc_stages(int K, int splits, int nt, bool lo) {
+int gemm_tc_stages(int K, int splits, int nt, bool lo, int cap) {
   const int nkb = (K + TC_BK - 1) / TC_BK;
   const int per_cta = (nkb + splits - 1) / splits;
-  const int cap = tc_max_stages(nt, lo);
+  const int deepest = tc_max_stages(nt, lo);
+  if (cap <= 0 || cap > deepest) cap = deepest;
   return per_cta < 1 ? 1 : (per_cta > cap ? cap : per_cta);
 }
 
-int gemm_tc_smem_bytes(int nt, int stages, bool lo) { return tc_smem_bytes(nt, stages, lo); }
-
+int gemm_tc_per_sm(int nt, int stages, bool lo) { return std::min(16, SM_SMEM / (tc_smem_bytes(nt, stages, lo) + 1024)); }
 
 template <int NT, bool LO>
 static void launch_tc_nt(const CUtensorMap* mapW, const CUtensorMap* mapX, GemmArgs a, cudaStream_t st) {
   // (a failure shows at launch)
   (void)ensure_kernel_attrs((const void*)k_gemm_tc<NT, LO>, tc_smem_bytes(NT, tc_max_stages(NT, LO), LO));
-  a.stages = gemm_tc_stages(a.K, a.splits, NT, LO);
+  a.stages = gemm_tc_stages(a.K, a.splits, NT, LO, a.stages);
   const int smem = tc_smem_bytes(NT, a.stages, LO);
   dim3 grid((a.N + TC_BM - 1) / TC_BM, a.splits);
   if (a.epi < EPI_CL_RESID) {

@@ -125,6 +125,7 @@ struct tlf_ctx {
   float* h_margin = nullptr;
   uint32_t* h_err = nullptr;
   int s_qkv = 1, s_o = 1, s_gu = 1, s_d = 1, split_cap = 8;
+  int ring = 0;  // most stages of the decode projections' operand rings (0: as deep as fits)
 
   // batched prefill (bf16 models): chunk workspaces, allocated on first use
   int pf_C = 0, pf_Smax = 0;
@@ -374,6 +375,9 @@ static int make_mat(tlf_ctx* ctx, DeviceMat* m, const std::vector<const uint8_t*
   return TLF_OK;
 }
 
+// k-tiles a CTA from which a tcgen05 projection takes two CTAs an SM
+constexpr int GEMM_LONG_K = 8;
+
 static int choose_splits(int tiles, int nkb, int target_ctas, int cap) {
   int s = (target_ctas + tiles - 1) / tiles;
   s = std::max(1, std::min(s, std::min(nkb, cap)));
@@ -560,22 +564,33 @@ static int create_impl(tlf_ctx* ctx, const tlf_weights* w) {
   }
   // split-K factors. tcgen05 path: the largest cluster size (<= 8, the portable
   // limit) whose grid still fits in one wave, counting how many CTAs of the
-  // resulting ring depth share an SM (10 % margin for cluster placement).
+  // resulting ring depth share an SM (10 % margin for cluster placement). A projection
+  // that leaves a CTA eight k-tiles or more that way takes the depth at which two CTAs
+  // share an SM, and then all of them do, so that each kernel starts beside its
+  // predecessor: the long-context model's step of 48 / 64 / 100 / 128 rows takes 726 / 767 /
+  // 945 / 1017 us against 964 / 993 / 1120 / 1190 us at full depth (its gate/up tiles fill 86
+  // of 152 SMs then). Shorter k ranges stay at full depth: the mid-size model's step of
+  // 100 / 128 rows takes 1632 / 1759 us against 1682 / 1816 us.
   if (ctx->use_tc) {
-    auto pick = [&](int tiles, int K) {
-      const int nkb = (K + 63) / 64;
-      for (int S = std::min(8, nkb); S > 1; --S) {
-        const int bytes =
-            gemm_tc_smem_bytes(ctx->nt_max, gemm_tc_stages(K, S, ctx->nt_max, ctx->operand_lo), ctx->operand_lo);
-        const int per_sm = std::min(16, 232448 / (bytes + 1024));
-        if (10LL * tiles * S <= 9LL * per_sm * ctx->num_sms) return S;
-      }
+    const int nt = ctx->nt_max;
+    const bool lo = ctx->operand_lo;
+    auto pick = [&](int tiles, int K, int ring) {
+      for (int S = std::min(8, (K + 63) / 64); S > 1; --S)
+        if (10LL * tiles * S <= 9LL * gemm_tc_per_sm(nt, gemm_tc_stages(K, S, nt, lo, ring), lo) * ctx->num_sms) return S;
       return 1;
     };
-    ctx->s_qkv = pick((md.qkv_dim + 127) / 128, d);
-    ctx->s_o = pick((d + 127) / 128, md.q_dim);
-    ctx->s_gu = pick(ctx->wgu[0].N / 128, d);
-    ctx->s_d = pick((d + 127) / 128, ff);
+    struct { int tiles, K; int* splits; } proj[4] = {{(md.qkv_dim + 127) / 128, d, &ctx->s_qkv},
+                                                     {(d + 127) / 128, md.q_dim, &ctx->s_o},
+                                                     {ctx->wgu[0].N / 128, d, &ctx->s_gu},
+                                                     {(d + 127) / 128, ff, &ctx->s_d}};
+    int two = gemm_tc_stages(1 << 20, 1, nt, lo, 0);  // deepest ring with two CTAs an SM
+    while (two > 1 && gemm_tc_per_sm(nt, two, lo) < 2) --two;
+    for (auto& p : proj) {
+      *p.splits = pick(p.tiles, p.K, 0);
+      if ((p.K + 63) / 64 < GEMM_LONG_K * *p.splits || gemm_tc_per_sm(nt, two, lo) < 2) continue;
+      *p.splits = pick(p.tiles, p.K, two);
+      ctx->ring = two;
+    }
   } else {
     const int target = 2 * ctx->num_sms;
     ctx->s_qkv = choose_splits((md.qkv_dim + 63) / 64, (d + 31) / 32, target, ctx->split_cap);
@@ -906,6 +921,7 @@ static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, bool rows, bool p
       a.n_dev = n_dev;
       a.max_rows = maxB;
       a.splits = ctx->s_qkv;
+      a.stages = ctx->ring;
       a.blo = lo_rows;
       if (split) {
         a.ss_in = ctx->d_ss;
@@ -945,6 +961,7 @@ static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, bool rows, bool p
       a.act = act_r;
       a.alpha = cond_args(ctx, s.m, r, j, 0);
       a.splits = ctx->s_o;
+      a.stages = ctx->ring;
       a.blo = lo_rows;
       if (split) {  // the MLP pre-norm of this layer, same rows
         a.xn = reinterpret_cast<bf16*>(ctx->d_X);
@@ -966,6 +983,7 @@ static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, bool rows, bool p
       a.n_dev = n_dev;
       a.max_rows = maxB;
       a.splits = ctx->s_gu;
+      a.stages = ctx->ring;
       a.blo = lo_rows;
       if (split) {
         a.ss_in = ctx->d_ss;
@@ -998,6 +1016,7 @@ static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, bool rows, bool p
       a.act = act_r;
       a.alpha = cond_args(ctx, s.m, r, j, 1);
       a.splits = ctx->s_d;
+      a.stages = ctx->ring;
       a.blo = lo_rows;
       if (split && (j + 1 < J || r + 1 < M)) {
         // the attention pre-norm of the next layer, or of layer 0 of loop r + 1 for the rows
@@ -1243,12 +1262,16 @@ static void gemm_pf(tlf_ctx* ctx, const DeviceMat& W, const CUtensorMap* xmaps, 
     launch_gemm_pf(&xmaps[3], bn == 256 ? &W.map : bn == 128 ? &W.map64 : &W.map32, bn, a, rows, ctx->pf_pairs, st);
     return;
   }
-  while (a.splits < 8 && (long long)ntiles * a.splits * 2 <= ctx->num_sms && nkb >= 4 * a.splits) a.splits *= 2;
   // The smallest token tile that holds the rows: less shared memory and TMEM let a kernel start beside its predecessor.
-  // The mid-size model's prompts of 4 / 64 / 117 / 256 tokens take 1184 / 1430 / 1570 / 1808 us against 1267 / 1480 /
-  // 1510 / 1807 us with 256-token tiles.
+  // Tiles of up to 128 rows also let two CTAs share an SM; K is split further for them while a CTA has eight k-tiles or
+  // more. The mid-size model's prompts of 4 / 64 / 117 tokens take 1162 / 1430 / 1532 us against 1267 / 1480 / 1550 us
+  // with tiles of 256 and one CTA an SM, the long-context model's 697 / 800 / 905 us against 905 / 1050 / 1180 us.
   int i = 0;
   while (i < 4 && rows > 16 << i) ++i;
+  const int per_sm = gemm_tc_per_sm(16 << i, gemm_tc_stages(W.K, 1, 16 << i, false, 0), false) > 1 ? 2 : 1;
+  while (a.splits < 8 && nkb >= 4 * a.splits &&
+         (long long)ntiles * a.splits * 2 <= (nkb >= GEMM_LONG_K * a.splits ? per_sm : 1) * ctx->num_sms)
+    a.splits *= 2;
   launch_gemm_tc(&W.map, &xmaps[i], 16 << i, a, st);
 }
 

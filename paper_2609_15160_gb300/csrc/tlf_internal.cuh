@@ -481,7 +481,7 @@ struct GemmArgs {
   int N;             // output features (rows of W)
   int K;             // reduction length
   int splits;        // split-K factor (gridDim.y; the cluster size for EPI_CL_*)
-  int stages;        // depth of the tcgen05 kernel's operand ring (set by the launcher)
+  int stages;        // tcgen05 kernel: most stages of its operand ring (0: as deep as fits), then its depth
   const int* act;    // RESID epilogues: rows with act[row] == 0 keep their residual (NULL: none)
   CondArgs alpha;    // RESID epilogues: the update is gated by alpha (conditioning; mod NULL: none)
   const int* n_dev;  // token rows n (device scalar), or NULL to use n_host
@@ -612,8 +612,9 @@ void launch_gemm_pf(const CUtensorMap* mapX, const CUtensorMap* mapW, int bn, co
 // operand-ring depth of a tcgen05 GEMM whose CTAs each reduce ceil(ceil(K/64)/splits) k-tiles
 // with token tile nt (and a two-term operand when lo), and the dynamic shared memory one CTA
 // then needs
-int gemm_tc_stages(int K, int splits, int nt, bool lo);
-int gemm_tc_smem_bytes(int nt, int stages, bool lo = false);
+// Depth of the tcgen05 kernel's operand ring (at most cap stages; 0: as deep as fits), and how many of its CTAs share an SM.
+int gemm_tc_stages(int K, int splits, int nt, bool lo, int cap);
+int gemm_tc_per_sm(int nt, int stages, bool lo);
 
 void launch_rope_table(const ModelDims& md, const double* inv_freq, float2* table, cudaStream_t st);
 void launch_rope_append(const ModelDims& md, const StepDev& s, int r, int j, const float* part, int splits,

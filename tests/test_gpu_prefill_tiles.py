@@ -36,6 +36,14 @@ def test_few_row_projections(tlf, shape, n):  # noqa: F811
     _prefill_decode_compare(tlf, _small(**SHAPES[shape]), [n], steps=1)
 
 
+@pytest.mark.parametrize("rows", [33, 64, 65, 128])
+def test_long_k_projections(tlf, rows):  # noqa: F811
+    """Projections with eight k-tiles a CTA and more (78 gate/up tiles over 8 k-tiles, 78 k-tiles down): two CTAs share an
+    SM, in the prompts' chunk and in the decode step."""
+    m = _small(d_model=512, ffn_hidden=4992, n_layers=1, max_loops=2, depth_probs=(0.5, 0.5))
+    _prefill_decode_compare(tlf, m, [1] * rows, steps=1)
+
+
 @pytest.mark.parametrize("hd,heads,kv", [(64, 4, 4), (64, 4, 2), (64, 4, 1), (128, 2, 2), (128, 4, 2), (128, 4, 1)])
 def test_pair_attention_blocks(tlf, hd, heads, kv):  # noqa: F811
     """The two-tile prefill attention around its 128-slot key blocks and query tiles, in one chunk and in chunks whose
