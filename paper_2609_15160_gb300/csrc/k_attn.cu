@@ -27,7 +27,8 @@
 // with LPK lanes sharing a key (16 bytes each) and xor-shuffle reductions.
 // Scores are in base 2 (q pre-scaled by log2(e)/sqrt(hd)).
 //
-// When a CTA finishes its part of an item it merges its warps. An item that
+// When a CTA finishes its part of an item it merges its warps (with one query head
+// a kv head, a merging warp does while the consumers go on). An item that
 // lies inside one CTA's range is written out directly. Otherwise each
 // contributing CTA stores a partial (max, sum, output) and takes a ticket with
 // an atomic counter, and the CTA that takes the last ticket merges the
@@ -42,7 +43,6 @@ namespace tlf {
 
 constexpr int ATT_PS = 64;     // keys per page (the only page size the library accepts)
 constexpr int ATT_WARPS = 8;   // consumer warps
-constexpr int ATT_THREADS = 32 * (ATT_WARPS + 1);
 
 template <typename T, int HD, int G>
 struct AttnShape {
@@ -54,11 +54,17 @@ struct AttnShape {
   static constexpr int NST = (98304 / STAGE_BYTES) < 2 ? 2 : ((98304 / STAGE_BYTES) > 8 ? 8 : (98304 / STAGE_BYTES));
   // Page teams: with one query head a kv head the warps' chain per page, not its instructions, is what a page costs, so
   // two teams of four warps take the pages in turn (a ring stage then always belongs to one team, so its depth is even).
-  // With the registers of two CTAs an SM, and the merge below without a second barrier: 200 rows of 64-700 keys, 16
-  // heads x 64, 80 -> 69 us; 32 rows of 128-8192 keys 98.5 -> 95 us (5.9 TB/s).
+  // With the registers of two CTAs an SM: 200 rows of 64-700 keys, 16 heads x 64, 80 -> 69 us; 32 rows of 128-8192 keys
+  // 98.5 -> 95 us.
   static constexpr int TEAMS = G == 1 && NST % 2 == 0 ? 2 : 1;
-  // Merge buffers: with two, an item's merge needs no barrier behind it.
-  static constexpr int REDS = G == 1 ? 2 : 1;
+  // A warp of its own merges the parts of all items of a CTA but the last, out of REDS buffers, while the consumer warps
+  // go on without a barrier: the 200 rows above 69 -> 62 us (5.1 TB/s), the 32 rows 95 -> 93 us (6.0 TB/s), 64 rows of
+  // 500-1500 keys, 8 heads x 128, 50 us. The last item is the launch's tail, where all warps merge faster (one CTA an
+  // item, 8 rows of 300-700 keys: 14.4 us, 15.5 with the one warp). With more query heads a kv head the tenth warp's
+  // registers cost more than the barriers: 100 rows of 30-500 keys, 16 / 8 heads x 128, 40 -> 51 us.
+  static constexpr bool MERGER = G == 1;
+  static constexpr int REDS = MERGER ? 4 : 1;
+  static constexpr int THREADS = 32 * (ATT_WARPS + 1 + (MERGER ? 1 : 0));
   static constexpr int TEAM_WARPS = ATT_WARPS / TEAMS;
   static constexpr int KEYS_PER_WARP = ATT_PS / TEAM_WARPS;
   static constexpr int STEPS = KEYS_PER_WARP / KPW;
@@ -71,7 +77,7 @@ template <typename T, int HD, int G, bool MASKED>
 constexpr int attn_smem_bytes() {
   using S = AttnShape<T, HD, G>;
   return 128 + S::NST * S::STAGE_BYTES + S::REDS * ATT_WARPS * G * (HD + 2) * 4 + (MASKED ? S::NST * ATT_PS * 4 : 0) +
-         2 * S::NST * 8 + 16;
+         2 * (S::NST + S::REDS) * 8 + 16;
 }
 
 __device__ __forceinline__ void consumer_sync() {
@@ -81,7 +87,7 @@ __device__ __forceinline__ void consumer_sync() {
 // Two CTAs an SM: the bound gives one query head the registers it can use (56 otherwise), and keeps four heads (131
 // otherwise, one CTA) at two: 36 rows of about 2950 keys, 32 / 8 heads x 128, 153 -> 141 us.
 template <typename T, int HD, int G, bool MASKED>
-__global__ void __launch_bounds__(ATT_THREADS, 2) k_attn_decode(ModelDims md, StepDev s, int r, int j,
+__global__ void __launch_bounds__(AttnShape<T, HD, G>::THREADS, 2) k_attn_decode(ModelDims md, StepDev s, int r, int j,
                                                              const float* __restrict__ Q, float* __restrict__ part,
                                                              T* __restrict__ O, int* __restrict__ cnt, bool o_lo) {
   using S = AttnShape<T, HD, G>;
@@ -101,8 +107,10 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) k_attn_decode(ModelDims md, St
   int* mring = reinterpret_cast<int*>(red + S::REDS * ATT_WARPS * PSZ);              // [NST][64] positions (MASKED)
   uint64_t* full = reinterpret_cast<uint64_t*>(mring + (MASKED ? S::NST * ATT_PS : 0));
   uint64_t* empty = full + S::NST;
-  int* flag = reinterpret_cast<int*>(empty + S::NST);
-  volatile int* abort_flag = flag + 1;  // set when a bounded wait runs out: later waits are skipped
+  uint64_t* red_full = empty + S::NST;       // [REDS] an item's parts of all warps are in its buffer (MERGER)
+  uint64_t* red_empty = red_full + S::REDS;  // [REDS] and merged
+  int* flags = reinterpret_cast<int*>(red_empty + S::REDS);  // last contributor: consumers, merging warp
+  volatile int* abort_flag = flags + 2;  // set when a bounded wait runs out: later waits are skipped
 
   pdl_wait();
   pdl_trigger();
@@ -123,6 +131,10 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) k_attn_decode(ModelDims md, St
       mbar_init(smem_u32(&full[i]), 1);
       mbar_init(smem_u32(&empty[i]), S::TEAM_WARPS);
     }
+    for (int i = 0; i < S::REDS; ++i) {
+      mbar_init(smem_u32(&red_full[i]), ATT_WARPS);
+      mbar_init(smem_u32(&red_empty[i]), 1);
+    }
     *abort_flag = 0;
     fence_barrier_init();
   }
@@ -142,6 +154,70 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) k_attn_decode(ModelDims md, St
     const int off = p - pbase[k], np = pages_of(k);
     h = off / np;
     g = off % np;
+  };
+
+  // Merge of the CTA's part of item (k, h), by NT threads (t0 is this one's index) that `sync` synchronises: written out,
+  // or stored as a partial, which the last contributor merges with the others'.
+  auto finish_item = [&](const float* mred, int* flag, int k, int h, int t0, auto nt, auto sync) {
+    constexpr int NT = decltype(nt)::value;
+    const int np = pages_of(k);
+    const int item = k * Hkv + h;
+    const int first = pbase[k] + h * np;
+    const int c_first = first / per, c_last = (first + np - 1) / per;
+    float* my = part + (size_t)(item + blockIdx.x) * PSZ;
+    const int nparts = c_last - c_first + 1;
+    // merged state of this CTA's warps: thread t owns (head gg, dim e)
+    for (int t = t0; t < G * HD; t += NT) {
+      const int gg = t / HD, e = t % HD;
+      float mx = -INFINITY;
+#pragma unroll
+      for (int w = 0; w < ATT_WARPS; ++w) mx = fmaxf(mx, mred[(w * G + gg) * (HD + 2) + HD]);
+      float o = 0.f, l = 0.f;
+#pragma unroll
+      for (int w = 0; w < ATT_WARPS; ++w) {
+        const float* rw = mred + (w * G + gg) * (HD + 2);
+        const float f = (rw[HD] == -INFINITY) ? 0.f : exp2f(rw[HD] - mx);
+        o = fmaf(f, rw[e], o);
+        l = fmaf(f, rw[HD + 1], l);
+      }
+      if (nparts == 1) {
+        store_o(k, h * G + gg, e, o / l);
+      } else {
+        my[gg * (HD + 2) + e] = o;
+        if (e == 0) {
+          my[gg * (HD + 2) + HD] = mx;
+          my[gg * (HD + 2) + HD + 1] = l;
+        }
+      }
+    }
+    if (nparts > 1) {
+      __threadfence();
+      sync();
+      if (t0 == 0) {
+        const int ticket = atomicAdd(cnt + item, 1);
+        *flag = (ticket == nparts - 1);
+      }
+      sync();
+      if (*flag) {
+        // last contributor: merge the partials of CTAs c_first..c_last
+        __threadfence();
+        for (int t = t0; t < G * HD; t += NT) {
+          const int gg = t / HD, e = t % HD;
+          float mx = -INFINITY;
+          for (int c = c_first; c <= c_last; ++c)
+            mx = fmaxf(mx, __ldcg(part + (size_t)(item + c) * PSZ + gg * (HD + 2) + HD));
+          float o = 0.f, l = 0.f;
+          for (int c = c_first; c <= c_last; ++c) {
+            const float* pp = part + (size_t)(item + c) * PSZ + gg * (HD + 2);
+            const float f = exp2f(__ldcg(pp + HD) - mx);
+            o = fmaf(f, __ldcg(pp + e), o);
+            l = fmaf(f, __ldcg(pp + HD + 1), l);
+          }
+          store_o(k, h * G + gg, e, o / l);
+        }
+        if (t0 == 0) cnt[item] = 0;  // ready for the next launch
+      }
+    }
   };
 
   if (warp == ATT_WARPS) {
@@ -192,6 +268,27 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) k_attn_decode(ModelDims md, St
     return;
   }
 
+  if (S::MERGER && warp == ATT_WARPS + 1) {
+    // ---------------- merging warp ----------------
+    int k, h, g;
+    locate(p0, k, h, g);
+    for (int p = p0, it = 0; (p += pages_of(k) - g) < p1; ++it) {  // the items before the CTA's last
+      const int b = it % S::REDS;
+      if (!*abort_flag && !mbar_wait(smem_u32(&red_full[b]), (it / S::REDS) & 1, s.err)) *abort_flag = 1;
+      finish_item(red + b * ATT_WARPS * PSZ, flags + 1, k, h, lane, std::integral_constant<int, 32>{}, [] { __syncwarp(); });
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&red_empty[b]));
+      g = 0;
+      if (++h == Hkv) {
+        h = 0;
+        do {
+          ++k;
+        } while (k < n_r && nkeys[k] == 0);
+      }
+    }
+    return;
+  }
+
   // ---------------- consumer warps ----------------
   const int grp = lane / S::LPK, part_lane = lane % S::LPK;
   const int team = warp / S::TEAM_WARPS, team_warp = warp % S::TEAM_WARPS;
@@ -215,7 +312,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) k_attn_decode(ModelDims md, St
     }
   };
   begin_item();
-  bool odd = false;  // merge buffer of the item
+  int it = 0;  // items so far
 
   for (int p = p0; p < p1; ++p) {
     const int i = p - p0, st = i % S::NST;
@@ -288,8 +385,8 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) k_attn_decode(ModelDims md, St
     const bool item_end = (g + 1 == pages_of(k));
     if (item_end || p + 1 == p1) {
       // ---- this CTA's part of item (k, h) is done: merge the lane groups, then the warps ----
-      float* mred = red + (S::REDS == 2 && odd ? ATT_WARPS * PSZ : 0);
-      odd = !odd;
+      const int b = it % S::REDS;
+      float* mred = red + b * ATT_WARPS * PSZ;
 #pragma unroll
       for (int gg = 0; gg < G; ++gg) {
 #pragma unroll
@@ -299,6 +396,10 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) k_attn_decode(ModelDims md, St
           for (int e = 0; e < S::VEC; ++e) acc[gg][e] += __shfl_xor_sync(0xffffffffu, acc[gg][e], o);
         }
       }
+      if (S::MERGER && it >= S::REDS && !*abort_flag &&
+          !mbar_wait(smem_u32(&red_empty[b]), ((it / S::REDS) - 1) & 1, s.err))
+        *abort_flag = 1;
+      ++it;
       if (grp == 0) {
 #pragma unroll
         for (int gg = 0; gg < G; ++gg) {
@@ -311,67 +412,14 @@ __global__ void __launch_bounds__(ATT_THREADS, 2) k_attn_decode(ModelDims md, St
           }
         }
       }
-      consumer_sync();
-      const int np = pages_of(k);
-      const int item = k * Hkv + h;
-      const int first = pbase[k] + h * np;
-      const int c_first = first / per, c_last = (first + np - 1) / per;
-      float* my = part + (size_t)(item + blockIdx.x) * PSZ;
-      const int nparts = c_last - c_first + 1;
-      // merged state of this CTA's warps: thread t owns (head gg, dim e)
-      for (int t = tid; t < G * HD; t += 32 * ATT_WARPS) {
-        const int gg = t / HD, e = t % HD;
-        float mx = -INFINITY;
-#pragma unroll
-        for (int w = 0; w < ATT_WARPS; ++w) mx = fmaxf(mx, mred[(w * G + gg) * (HD + 2) + HD]);
-        float o = 0.f, l = 0.f;
-#pragma unroll
-        for (int w = 0; w < ATT_WARPS; ++w) {
-          const float* rw = mred + (w * G + gg) * (HD + 2);
-          const float f = (rw[HD] == -INFINITY) ? 0.f : exp2f(rw[HD] - mx);
-          o = fmaf(f, rw[e], o);
-          l = fmaf(f, rw[HD + 1], l);
-        }
-        if (nparts == 1) {
-          store_o(k, h * G + gg, e, o / l);
-        } else {
-          my[gg * (HD + 2) + e] = o;
-          if (e == 0) {
-            my[gg * (HD + 2) + HD] = mx;
-            my[gg * (HD + 2) + HD + 1] = l;
-          }
-        }
-      }
-      if (nparts > 1) {
-        __threadfence();
+      if (S::MERGER && p + 1 < p1) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&red_full[b]));
+      } else {
         consumer_sync();
-        if (tid == 0) {
-          const int ticket = atomicAdd(cnt + item, 1);
-          *flag = (ticket == nparts - 1);
-        }
-        consumer_sync();
-        if (*flag) {
-          // last contributor: merge the partials of CTAs c_first..c_last
-          __threadfence();
-          for (int t = tid; t < G * HD; t += 32 * ATT_WARPS) {
-            const int gg = t / HD, e = t % HD;
-            float mx = -INFINITY;
-            for (int c = c_first; c <= c_last; ++c)
-              mx = fmaxf(mx, __ldcg(part + (size_t)(item + c) * PSZ + gg * (HD + 2) + HD));
-            float o = 0.f, l = 0.f;
-            for (int c = c_first; c <= c_last; ++c) {
-              const float* pp = part + (size_t)(item + c) * PSZ + gg * (HD + 2);
-              const float f = exp2f(__ldcg(pp + HD) - mx);
-              o = fmaf(f, __ldcg(pp + e), o);
-              l = fmaf(f, __ldcg(pp + HD + 1), l);
-            }
-            store_o(k, h * G + gg, e, o / l);
-          }
-          if (tid == 0) cnt[item] = 0;  // ready for the next launch
-        }
+        finish_item(mred, flags, k, h, tid, std::integral_constant<int, 32 * ATT_WARPS>{}, consumer_sync);
+        if (!S::MERGER) consumer_sync();  // `red` and the flag are reused by the next item
       }
-      // `red` and `flag` are reused by the next item (a second buffer waits for the barrier of the item between)
-      if (S::REDS == 1 || nparts > 1) consumer_sync();
       if (p + 1 < p1) {
         g = 0;
         if (++h == Hkv) {
@@ -393,7 +441,7 @@ static void attn_launch_v(const ModelDims& md, const StepDev& s, int r, int j, c
                           int* cnt, int grid, cudaStream_t st, bool o_lo) {
   constexpr int smem = attn_smem_bytes<T, HD, G, MASKED>();
   (void)ensure_kernel_attrs((const void*)k_attn_decode<T, HD, G, MASKED>, smem);  // a failure shows at launch
-  launch_k(k_attn_decode<T, HD, G, MASKED>, grid, ATT_THREADS, smem, st, md, s, r, j, Q, part, (T*)O, cnt, o_lo);
+  launch_k(k_attn_decode<T, HD, G, MASKED>, grid, AttnShape<T, HD, G>::THREADS, smem, st, md, s, r, j, Q, part, (T*)O, cnt, o_lo);
 }
 
 template <typename T, int HD, int G>
