@@ -353,6 +353,7 @@ def measure(T, wl, args, rank: int, ws: int, local: int, steps: int, warmup: int
         barrier()
         step_ms = [st_ev[i].elapsed_time(en_ev[i]) for i in range(steps)]
         total_ms = float(sum(step_ms))
+    launches = steps * ctx.last_step_profile()[2]  # every timed step launches the same kernels
 
     # --- end-to-end pass: host tokens in, host logits out ---
     barrier()
@@ -376,14 +377,13 @@ def measure(T, wl, args, rank: int, ws: int, local: int, steps: int, warmup: int
 
     # --- kernel-level pass: attention kernel time and algorithmic KV bytes ---
     ctx.set_profiling(True)
-    att_ms, att_bytes, launches, att_launches = 0.0, 0.0, 0, 0
+    att_ms, att_bytes, att_launches = 0.0, 0.0, 0
     kernel_ms = {}
     for s in range(steps):
         ctx.decode_step(ids, toks[2 * n_steps + s], forced=forced, logits=logits_dev, stream=stream)
-        ms, by, nl = ctx.last_step_profile()
+        ms, by, _ = ctx.last_step_profile()
         att_ms += ms
         att_bytes += by
-        launches += nl
         att_launches += m.n_layers * m.max_loops
         if breakdown:
             for kname, kms in ctx.last_step_kernel_times().items():

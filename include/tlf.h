@@ -358,7 +358,8 @@ int tlf_last_active_sets(tlf_ctx* ctx, int32_t* counts, int32_t* idx);
 /* Kernel-level timing of the last decode step, filled when
  * tlf_set_profiling(ctx, 1) is on: milliseconds spent in the recursion-wise
  * attention kernels, the KV bytes they read (K and V of every visited entry
- * once per kv head), and the number of kernels launched. */
+ * once per kv head), and the number of kernels launched. A profiled step runs
+ * the shared block as one launch per stage, whatever its size. */
 int tlf_set_profiling(tlf_ctx* ctx, int32_t on);
 int tlf_last_step_profile(const tlf_ctx* ctx, float* attn_ms, double* attn_kv_bytes,
                           int32_t* kernel_launches);

@@ -17,7 +17,9 @@
 //     scatter (Eq. 7) -> gather+RMSNorm -> gate/up GEMM -> SwiGLU -> down GEMM +
 //     residual scatter
 //   -> final RMSNorm + cache-length update -> tied LM head.
-// Kernels of a loop with no active token exit on the device-side count.
+// Kernels of a loop with no active token exit on the device-side count. The loops run as one
+// persistent kernel for up to 16 bf16 rows, as one CTA per row for small float32 models, and as a
+// launch per stage otherwise.
 #include <cudaTypedefs.h>
 
 #include <algorithm>
