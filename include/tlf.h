@@ -189,8 +189,9 @@ int64_t tlf_page_bytes(const tlf_config* cfg);
  *                        replaying a captured CUDA graph (read here)
  *   TLF_NO_PDL=1         plain stream order instead of programmatic
  *                        dependent launch (read when the library loads)
- *   TLF_NO_SPLIT_NORM=1  every decode pre-norm as a kernel of its own instead
- *                        of split across the neighbouring GEMMs (read here)
+ *   TLF_NO_SPLIT_NORM=1  every pre-norm of decode steps and short prompts as a
+ *                        kernel of its own instead of split across the
+ *                        neighbouring GEMMs (read here)
  *   TLF_NO_OPERAND_LO=1  one bf16 plane for the decode GEMMs' activation
  *                        operands instead of hi + lo (two-term) planes (read
  *                        here)

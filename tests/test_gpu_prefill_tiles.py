@@ -44,6 +44,15 @@ def test_long_k_projections(tlf, rows):  # noqa: F811
     _prefill_decode_compare(tlf, m, [1] * rows, steps=1)
 
 
+@pytest.mark.parametrize("d,n,cond", [(1024, 200, False), (1024, 200, True), (1088, 32, False), (1088, 33, False),
+                                      (192, 255, True)])
+def test_split_norms_of_short_prompts(tlf, d, n, cond):  # noqa: F811
+    """Pre-norms split between the projections of a one-tile loop, on both sides of the rule, with and without
+    conditioning, over more loops and layers than one; feature tiles that end inside 128."""
+    m = _small(d_model=d, n_layers=3, max_loops=2, depth_probs=(0.5, 0.5), conditioning=cond)
+    _prefill_decode_compare(tlf, m, [n], steps=1)
+
+
 @pytest.mark.parametrize("hd,heads,kv", [(64, 4, 4), (64, 4, 2), (64, 4, 1), (128, 2, 2), (128, 4, 2), (128, 4, 1)])
 def test_pair_attention_blocks(tlf, hd, heads, kv):  # noqa: F811
     """The two-tile prefill attention around its 128-slot key blocks and query tiles, in one chunk and in chunks whose
