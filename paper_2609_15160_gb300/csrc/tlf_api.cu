@@ -58,6 +58,8 @@ struct tlf_ctx {
   bool use_tc = false;
   int nt_max = 0;
 
+  std::vector<void*> device;    // every device allocation of the context, in order (dev_alloc)
+
   // weights
   void* d_emb = nullptr;
   void* d_router_w = nullptr;
@@ -346,8 +348,15 @@ static int dev_alloc(tlf_ctx* ctx, T** p, size_t bytes, const char* what) {
   void* q = nullptr;
   cudaError_t e = cudaMalloc(&q, bytes < 16 ? 16 : bytes);
   if (e != cudaSuccess) return fail(ctx, TLF_ERR_CUDA, "cudaMalloc(%s, %zu bytes): %s", what, bytes, cudaGetErrorString(e));
+  ctx->device.push_back(q);
   *p = static_cast<T*>(q);
   return TLF_OK;
+}
+
+// Frees what was allocated since the context held `keep` allocations.
+static void dev_free_from(tlf_ctx* ctx, size_t keep) {
+  for (size_t i = keep; i < ctx->device.size(); ++i) cudaFree(ctx->device[i]);
+  ctx->device.resize(keep);
 }
 
 static int upload(tlf_ctx* ctx, void** dst, const void* src, size_t bytes, const char* what) {
@@ -500,20 +509,19 @@ static int create_impl(tlf_ctx* ctx, const tlf_weights* w) {
                             w->cond_dt_b1, w->cond_dt_w2, w->cond_dt_b2, w->mod_w, w->mod_b};
     const size_t cnt[10] = {d * F, (size_t)d, dd, (size_t)d, d * F, (size_t)d, dd, (size_t)d, J4 * d, J4};
     float* dev[10] = {};
-    rc = 0;
+    const size_t P = (size_t)M * (M + 1) / 2;
+    rc = dev_alloc(ctx, &ctx->d_cond, (size_t)J * P * 4 * d * 4, "conditioning table");
+    const size_t keep = ctx->device.size();
     for (int i = 0; i < 10 && rc == 0; ++i) {
       if (!src[i]) rc = fail(ctx, TLF_ERR_BAD_WEIGHTS, "a conditioning weight pointer is NULL");
       else rc = upload(ctx, (void**)&dev[i], src[i], cnt[i] * 4, "conditioning weights");
     }
-    const size_t P = (size_t)M * (M + 1) / 2;
-    if (rc == 0) rc = dev_alloc(ctx, &ctx->d_cond, (size_t)J * P * 4 * d * 4, "conditioning table");
     if (rc == 0) {
       const int e = build_cond_table(md, dev[0], dev[1], dev[2], dev[3], dev[4], dev[5], dev[6], dev[7], dev[8],
                                      dev[9], ctx->d_cond, 0);
       if (e) rc = fail(ctx, TLF_ERR_CUDA, "conditioning table: %s", cudaGetErrorString((cudaError_t)e));
     }
-    for (float* p : dev)
-      if (p) cudaFree(p);
+    dev_free_from(ctx, keep);
     if (rc) return rc;
   }
 
@@ -659,23 +667,11 @@ extern "C" void tlf_destroy(tlf_ctx* ctx) {
   if (!ctx) return;
   if (!ctx->host_only) {
     cudaDeviceSynchronize();
-    auto f = [](void* p) { if (p) cudaFree(p); };
-    f(ctx->d_emb); f(ctx->d_router_w); f(ctx->d_router_w1); f(ctx->d_router_b1); f(ctx->d_router_b); f(ctx->d_attn_norm); f(ctx->d_mlp_norm);
-    f(ctx->d_final_norm); f(ctx->d_inv_freq); f(ctx->d_rope); f(ctx->d_rowinfo); f(ctx->d_act); f(ctx->d_col); f(ctx->d_ss); f(ctx->d_cond);
-    f(ctx->d_part_small); f(ctx->d_ss8); f(ctx->d_gbar);
-    for (auto* v : {&ctx->wqkv, &ctx->wo, &ctx->wgu, &ctx->wd})
-      for (auto& m : *v) f(m.ptr);
-    f(ctx->d_pool); f(ctx->d_pos_table); f(ctx->d_page_table); f(ctx->d_len); f(ctx->d_upload);
-    f(ctx->d_m); f(ctx->d_H); f(ctx->d_X); f(ctx->d_O); f(ctx->d_U); f(ctx->d_Xf);
-    f(ctx->d_part); f(ctx->d_Q); f(ctx->d_idx); f(ctx->d_n); f(ctx->d_item_base); f(ctx->d_nch); f(ctx->d_chunk);
-    f(ctx->d_attn_part); f(ctx->d_attn_cnt); f(ctx->d_logits);
+    dev_free_from(ctx, 0);
     if (ctx->h_upload) cudaFreeHost(ctx->h_upload);
     if (ctx->h_m) cudaFreeHost(ctx->h_m);
     for (auto e : ctx->events) if (e) cudaEventDestroy(e);
     for (auto& g : ctx->graphs) cudaGraphExecDestroy(g.exec);
-    f(ctx->d_pf_in); f(ctx->d_pf_m); f(ctx->d_pf_margin); f(ctx->d_pf_H); f(ctx->d_pf_X); f(ctx->d_pf_Q);
-    f(ctx->d_pf_O); f(ctx->d_pf_U); f(ctx->d_pf_idx); f(ctx->d_pf_n); f(ctx->d_pf_row_slot); f(ctx->d_pf_row_cslot);
-    f(ctx->d_pf_row_pos); f(ctx->d_pf_first); f(ctx->d_pf_cnt); f(ctx->d_pf_s0); f(ctx->d_pf_tile_base);
     if (ctx->h_pf_in) cudaFreeHost(ctx->h_pf_in);
     if (ctx->h_pf_m) cudaFreeHost(ctx->h_pf_m);
     if (ctx->h_pf_nr) cudaFreeHost(ctx->h_pf_nr);
@@ -1200,6 +1196,8 @@ extern "C" int tlf_decode_step(tlf_ctx* ctx, int32_t batch, const uint64_t* seq_
 static int ensure_prefill_buffers(tlf_ctx* ctx) {
   if (ctx->pf_C) return TLF_OK;
   const ModelDims& md = ctx->md;
+  ctx->pf_pairs = gemm_pf_max_pairs(ctx->num_sms);
+  if (ctx->pf_pairs < 1) return fail(ctx, TLF_ERR_CUDA, "the prefill GEMM's clusters cannot be launched on this device");
   int C = ctx->cfg.prefill_chunk > 0 ? ctx->cfg.prefill_chunk : 8192;
   C = (C + 255) / 256 * 256;
   const int Smax = std::min(1024, std::min(C, ctx->cfg.max_seqs));
@@ -1242,8 +1240,6 @@ static int ensure_prefill_buffers(tlf_ctx* ctx) {
     return fail(ctx, TLF_ERR_CUDA, "cuTensorMapEncodeTiled failed for a prefill buffer");
   if (ctx->has_pool_map && !make_q_map(&ctx->pf_map_Q, ctx->d_pf_Q, md, 2 * C))
     return fail(ctx, TLF_ERR_CUDA, "cuTensorMapEncodeTiled failed for the prefill q planes");
-  ctx->pf_pairs = gemm_pf_max_pairs(ctx->num_sms);
-  if (ctx->pf_pairs < 1) return fail(ctx, TLF_ERR_CUDA, "the prefill GEMM's clusters cannot be launched on this device");
   ctx->pf_C = C;
   ctx->pf_Smax = Smax;
   return TLF_OK;
