@@ -1084,9 +1084,11 @@ static cudaGraphExec_t step_graph(tlf_ctx* ctx, int B, bool need_logits, bool ro
   return exec;
 }
 
-// logits: where the step's logits go behind it (NULL: they stay in d_logits).
+// logits: where the step's logits go behind it (NULL: they stay in d_logits). A copy that CUDA refuses is reported in
+// *copied: the step itself has run, and its caller advances the cache lengths as the device did.
 static int run_step(tlf_ctx* ctx, int B, const int* slots, const int* tokens, const int* forced,
-                    const std::vector<PageUpdate>& upd, bool need_logits, cudaStream_t st, float* logits = nullptr) {
+                    const std::vector<PageUpdate>& upd, bool need_logits, cudaStream_t st, float* logits = nullptr,
+                    cudaError_t* copied = nullptr) {
   const ModelDims& md = ctx->md;
   const int M = md.M, J = md.J;
   const bool prof = ctx->profiling;
@@ -1110,8 +1112,8 @@ static int run_step(tlf_ctx* ctx, int B, const int* slots, const int* tokens, co
     ctx->warmed = true;
   }
   if (logits)  // queued behind the step, so one wait covers both
-    CK(ctx, cudaMemcpyAsync(logits, ctx->d_logits, (size_t)B * md.V * 4,
-                            is_device_ptr(logits) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st));
+    *copied = cudaMemcpyAsync(logits, ctx->d_logits, (size_t)B * md.V * 4,
+                              is_device_ptr(logits) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st);
   CK(ctx, cudaStreamSynchronize(st));
   if (*ctx->h_err) {
     const uint32_t e = *ctx->h_err;
@@ -1182,11 +1184,16 @@ extern "C" int tlf_decode_step(tlf_ctx* ctx, int32_t batch, const uint64_t* seq_
   if (rc) return rc;
   cudaStream_t st = (cudaStream_t)stream;
   const bool want = logits != nullptr;
-  rc = run_step(ctx, batch, slots.data(), tokens, forced, upd, want, st, logits);
+  cudaError_t copied = cudaSuccess;
+  rc = run_step(ctx, batch, slots.data(), tokens, forced, upd, want, st, logits, &copied);
   if (rc) return rc;
   advance_lengths(ctx, batch, slots.data());
   for (int b = 0; b < batch; ++b) loops[b] = ctx->h_m[b];
   if (router_margin) memcpy(router_margin, ctx->h_margin, (size_t)batch * 4);
+  if (copied != cudaSuccess) {
+    cudaGetLastError();
+    return fail(ctx, TLF_ERR_CUDA, "logits copy: %s", cudaGetErrorString(copied));
+  }
   return TLF_OK;
 }
 

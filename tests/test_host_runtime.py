@@ -50,3 +50,56 @@ def test_a_context_gives_back_all_its_device_memory(lib, dtype):
         ctx.prefill([1, 2], [np.arange(70, dtype=np.int32), np.arange(5, dtype=np.int32)])
         ctx.decode_step([1, 2], [3, 4])
     assert lib.fake_live() == before
+
+
+class _DeviceBuffer:
+    """A buffer that the fake runtime takes for device memory."""
+
+    def __init__(self, lib, nbytes):
+        self.lib, self.ptr = lib, lib.fake_device_buffer(nbytes)
+
+    def data_ptr(self):
+        return self.ptr
+
+    def free(self):
+        self.lib.fake_free(self.ptr)
+
+
+@pytest.fixture
+def loops(lib):
+    """loops(batch, n): from now on every step's results say n loops for each row (nothing computes them here)."""
+    hooks = []
+
+    def set_loops(batch, n):
+        size = 2 * batch * 4 + 4  # loop counts, margins, error word
+
+        def fill(dst, src, nbytes):
+            if nbytes == size:
+                C.memmove(dst, (C.c_int32 * batch)(*[n] * batch), 4 * batch)
+        hooks.append(C.CFUNCTYPE(None, C.c_void_p, C.c_void_p, C.c_size_t)(fill))
+        lib.fake_on_copy(hooks[-1])
+    yield set_loops
+    lib.fake_on_copy(None)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_a_refused_logits_copy_leaves_host_and_device_at_the_same_lengths(lib, loops, dtype):
+    """The step has run by then: the call waits for it and advances the lengths, as the device has, before it fails."""
+    m = _model(dtype)
+    with _context(m) as ctx:
+        loops(4, 2)
+        ctx.load_cache(1, synth.make_cache_positions(m, 10, 3))
+        want = [ctx.cache_len(1, r) for r in (1, 2, 3)]
+        out = _DeviceBuffer(lib, 4 * m.vocab)
+        lib.fake_refuse_copy(out.ptr)
+        for step in range(3):  # directly, captured, replayed
+            syncs = lib.fake_syncs()
+            with pytest.raises(tlf.TlfError) as e:
+                ctx.decode_step([1], [5], logits=out)
+            assert e.value.name == "CUDA" and "logits copy" in str(e.value)
+            assert lib.fake_syncs() > syncs
+            want = [want[0] + 1, want[1] + 1, want[2]]
+            assert [ctx.cache_len(1, r) for r in (1, 2, 3)] == want
+        lib.fake_refuse_copy(None)
+        ctx.decode_step([1], [5], logits=out)
+        out.free()
