@@ -246,8 +246,15 @@ int tlf_prefill(tlf_ctx* ctx, int32_t n_seqs, const uint64_t* seq_ids, const int
  *   router_margin  host float32 [batch] or NULL: the router's decision margin
  *                  (see tlf_exit_rule); a token is a near-tie when it is small
  * The call synchronises `stream` before returning (loop counts are host
- * outputs). Errors: INVALID_ARG, UNKNOWN_SEQ, CAPACITY, SEQ_TOO_LONG,
- * OUT_OF_PAGES, CUDA, DEVICE. */
+ * outputs). For bf16 models whose shapes fit, a step of up to 16 rows is one
+ * cooperative kernel that needs every SM of the device, with almost all of its
+ * shared memory, at the same time: other work on the GPU delays it for as long
+ * as it holds any SM, and makes it fail with DEVICE if it keeps one from it for
+ * more than 4 s. Where CUDA refuses such a launch (a stream limited to some of
+ * the SMs), the context runs its steps as separate kernels from then on.
+ * After CUDA or DEVICE, logits may hold values of the failed step.
+ * Errors: INVALID_ARG, UNKNOWN_SEQ, CAPACITY, SEQ_TOO_LONG, OUT_OF_PAGES,
+ * CUDA, DEVICE. */
 int tlf_decode_step(tlf_ctx* ctx, int32_t batch, const uint64_t* seq_ids, const int32_t* tokens,
                     const int32_t* forced, float* logits, int32_t* loops, float* router_margin,
                     void* stream);

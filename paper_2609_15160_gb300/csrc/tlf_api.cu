@@ -861,8 +861,9 @@ static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, bool rows, bool p
   void* x_lo = ctx->operand_lo ? static_cast<void*>(reinterpret_cast<bf16*>(ctx->d_X) + (size_t)maxB * md.d) : nullptr;
   void* u_lo = ctx->operand_lo ? static_cast<void*>(reinterpret_cast<bf16*>(ctx->d_U) + (size_t)maxB * md.ff) : nullptr;
   // Up to 16 rows: the whole block as one persistent kernel (a profiled step keeps a launch per stage, so
-  // that each can be timed).
-  const bool small = ctx->step_small && B <= 16 && !prof;
+  // that each can be timed; so does a context whose cooperative launch was refused, as for a stream that may use fewer
+  // SMs than the device has).
+  bool small = ctx->step_small && B <= SS_ROWS && !prof;
   if (small) {
     launch_norm_rows(md.dtype, ctx->d_H, md.d, ctx->d_idx, ctx->d_n, 0, B, ctx->d_attn_norm, md.d, md.eps, ctx->d_X, md.d,
                      st, cond_args(ctx, s.m, 0, 0, 2), ctx->d_ss, x_lo);
@@ -882,8 +883,13 @@ static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, bool rows, bool p
     a.rope = ctx->d_rope;
     a.cond = ctx->d_cond;
     a.gbar = ctx->d_gbar;
-    CK(ctx, launch_step_small(a, ctx->num_sms, st));
-    ctx->last_launches += 2;
+    small = launch_step_small(a, ctx->num_sms, st) == cudaSuccess;
+    if (small) {
+      ctx->last_launches += 2;
+    } else {
+      cudaGetLastError();
+      ctx->step_small = false;
+    }
   }
   if (rows) {
     RowStep a{};
@@ -1071,12 +1077,14 @@ static cudaGraphExec_t step_graph(tlf_ctx* ctx, int B, bool need_logits, bool ro
     ctx->use_graphs = false;
     return nullptr;
   }
+  const bool small = ctx->step_small;
   const int rc = enqueue_step(ctx, B, need_logits, rows, false, ctx->cap_stream);
   const cudaError_t e1 = cudaStreamEndCapture(ctx->cap_stream, &graph);
   if (rc != TLF_OK || e1 != cudaSuccess || cudaGraphInstantiate(&exec, graph, 0) != cudaSuccess) {
     cudaGetLastError();
     if (graph) cudaGraphDestroy(graph);
-    ctx->use_graphs = false;  // run the kernels directly from now on
+    // run the kernels directly from now on (or, where the persistent kernel was refused, capture the next step without it)
+    if (small == ctx->step_small) ctx->use_graphs = false;
     return nullptr;
   }
   cudaGraphDestroy(graph);
@@ -1105,8 +1113,22 @@ static int run_step(tlf_ctx* ctx, int B, const int* slots, const int* tokens, co
   for (int b = 0; b < B && rows; ++b) rows = ctx->h_len[(size_t)slots[b] * M] + 1 <= RowStep::MAX_KEYS;
   cudaGraphExec_t exec = prof ? nullptr : step_graph(ctx, B, need_logits, rows);
   if (exec) {
-    CK(ctx, cudaGraphLaunch(exec, st));
-  } else {
+    const cudaError_t e = cudaGraphLaunch(exec, st);
+    if (e != cudaSuccess && ctx->step_small && B <= SS_ROWS) {
+      // the graph holds the persistent kernel: this and later steps run without it
+      cudaGetLastError();
+      ctx->step_small = false;
+      for (size_t i = ctx->graphs.size(); i-- > 0;)
+        if (ctx->graphs[i].B <= SS_ROWS) {
+          cudaGraphExecDestroy(ctx->graphs[i].exec);
+          ctx->graphs.erase(ctx->graphs.begin() + i);
+        }
+      exec = nullptr;
+    } else {
+      CK(ctx, e);
+    }
+  }
+  if (!exec) {
     const int rc = enqueue_step(ctx, B, need_logits, rows, prof, st);
     if (rc) return rc;
     ctx->warmed = true;

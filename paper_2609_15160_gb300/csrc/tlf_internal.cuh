@@ -531,6 +531,7 @@ struct GemmArgs {
   void* U_lo;              // EPI_CL_SWIGLU: lo plane of U (NULL: none)
 };
 // The persistent kernel of a step of up to 16 rows (k_step.cu).
+constexpr int SS_ROWS = 16;    // most rows of a step it takes
 constexpr int SS_LAYERS = 16;  // most layers of the block it takes
 struct SmallLayer {
   const bf16 *wqkv, *wo, *wgu, *wd;     // packed as for the GEMMs

@@ -103,3 +103,40 @@ def test_a_refused_logits_copy_leaves_host_and_device_at_the_same_lengths(lib, l
         lib.fake_refuse_copy(None)
         ctx.decode_step([1], [5], logits=out)
         out.free()
+
+
+@pytest.mark.parametrize("refused", ["first launch", "capture", "replay"])
+def test_a_refused_cooperative_launch_falls_back_to_a_launch_per_stage(lib, loops, refused):
+    """Steps of up to 16 rows want every SM at once; where CUDA says no, the step and all later ones run as kernels of
+    their own, and are still captured and replayed."""
+    m = _model()
+    with _context(m) as ctx:
+        loops(4, 1)
+        ctx.load_cache(1, synth.make_cache_positions(m, 10, 3))
+
+        def step():
+            """(persistent kernels, projections, replayed graphs) of one step, and the launches it reports"""
+            names = (b"k_step_small", b"k_gemm_tc")
+            before = [lib.fake_launches(n) for n in names] + [lib.fake_graph_launches()]
+            ctx.decode_step([1], [5], logits=False)
+            after = [lib.fake_launches(n) for n in names] + [lib.fake_graph_launches()]
+            return [b - a for a, b in zip(before, after)], ctx.last_step_profile()[2]
+
+        stages = 4 * m.n_layers * m.max_loops
+        try:
+            good = {"first launch": 0, "capture": 1, "replay": 2}[refused]
+            for i in range(good):
+                assert step()[0] == [1, 0, i]  # a capture counts as a launch, and its graph is replayed
+            lib.fake_refuse_cooperative(1)
+            lib.fake_refuse_graph(int(refused == "replay"))
+            got, reported = step()
+            assert got[:2] == [0, stages] and reported > stages
+            lib.fake_refuse_graph(0)
+            for i in range(4):
+                got, reported = step()
+                assert got[0] == 0 and reported > stages
+            assert got == [0, 0, 1]  # replayed
+        finally:
+            lib.fake_refuse_cooperative(0)
+            lib.fake_refuse_graph(0)
+        assert ctx.cache_len(1, 1) == 10 + good + 5
