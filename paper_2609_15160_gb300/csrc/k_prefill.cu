@@ -334,7 +334,6 @@ __global__ void __launch_bounds__(PFT_THREADS) k_pf_attn_tc(ModelDims md, Prefil
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 5);
 
   pdl_wait();
-  pdl_trigger();
   const int S = p.S;
   const int* tbase = p.tile_base + r * (p.Smax + 1);
   const int tile = blockIdx.x, kvh = blockIdx.y;
@@ -369,6 +368,7 @@ __global__ void __launch_bounds__(PFT_THREADS) k_pf_attn_tc(ModelDims md, Prefil
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_trigger();  // a dependent CTA on this SM could otherwise take the columns that this one still waits for
   const uint32_t tmem = *tmem_slot;
   const uint32_t t_row = tmem + ((uint32_t)(quad * 32) << 16);  // this warp's 32 TMEM lanes
   constexpr uint32_t OCOL = 128;                                 // first TMEM column of O
@@ -722,7 +722,6 @@ __global__ void __launch_bounds__(PFA_THREADS, 1) k_pf_attn_pair(ModelDims md, P
     tmem_relinquish();
   }
   pdl_wait();
-  pdl_trigger();
   const int S = p.S;
   const int* tbase = p.tile_base + r * (p.Smax + 1);
   // 1-D grid, kv head fastest and query blocks in reverse order: the blocks with the most pages
@@ -747,6 +746,7 @@ __global__ void __launch_bounds__(PFA_THREADS, 1) k_pf_attn_pair(ModelDims md, P
   tc_fence_before();
   __syncthreads();  // barriers initialised, TMEM allocated
   tc_fence_after();
+  pdl_trigger();  // not before: a dependent CTA on this SM could take the columns that warp 9 still waits for
   const uint32_t tmem = *tmem_slot;
   // a bounded wait; once any role has given up, the others skip their waits and wind down
   auto wait = [&](uint32_t b, uint32_t parity) {
