@@ -613,8 +613,9 @@ __global__ void __launch_bounds__(PFT_THREADS) k_pf_attn_tc(ModelDims md, Prefil
 //                   precision), then K and V of every block through 3-D tensor maps into one ring;
 //   warp 9          MMA issuer: S = Qhi K^T + Qlo K^T, O += P V with V taken as an MN-major operand.
 // mbarriers connect the roles; every wait is bounded. A block past a sequence's last page loads its last
-// page twice: slots past the last query hold finite values (the pool is zeroed when created and only
-// ever holds finite entries), which the mask turns into P = 0.
+// page twice. Slots past the last query may hold anything (a released page keeps its entries), and P = 0 does not
+// cancel an infinity: the P V product of a tile ends with the group of 16 slots of its last query, and what lies behind
+// the block's last query in that group is zeroed in V.
 //
 // What bounds it: at head_dim 128 a block of a tile is 1536 cycles of MMAs (two S products for q's two terms, one P
 // V) against about 1024 of exponentials, so the tiles' softmaxes hide behind each other's MMAs; at head_dim 64 the
@@ -816,12 +817,14 @@ __global__ void __launch_bounds__(PFA_THREADS, 1) k_pf_attn_pair(ModelDims md, P
               tc_mma_f16(d, qd + pl * T_E + kc * COL_E + 2 * k, kd + kc * COL_E + 2 * k, IDS, (pl | kc | k) ? 1u : 0u);
         tc_commit(s_full(x));
       };
+      const int end0 = s0 + q0 + nq0, end1 = end0 + nq1;  // slots up to the tiles' last queries
       auto issue_pv = [&](int x, int kb) {
+        const int groups = ((x ? end1 : end0) - kb * 128 + 15) / 16;  // of 16 slots that the tile sees
         const uint64_t vd = dv + (uint64_t)((2 * kb + 1) % NST) * T_E;
         const uint32_t d = tmem + Sh::OCOL + (uint32_t)(HD * x), pa = tmem + Sh::PCOL + Sh::P_STEP * (uint32_t)x;
 #pragma unroll
         for (int k = 0; k < 8; ++k)  // K = 16 keys per MMA: 8 TMEM columns of P, +2048 B (16 rows) of V
-          tc_mma_f16_ts(d, pa + 8u * k, vd + V16_E * k, IDO, (kb > 0 || k > 0) ? 1u : 0u);
+          if (k < groups) tc_mma_f16_ts(d, pa + 8u * k, vd + V16_E * k, IDO, (kb > 0 || k > 0) ? 1u : 0u);
         tc_commit(o_done(x));
       };
       auto kfull = [&](int kb) { return wait(kv_full((2 * kb) % NST), (uint32_t)(2 * kb / NST) & 1u); };
@@ -853,6 +856,15 @@ __global__ void __launch_bounds__(PFA_THREADS, 1) k_pf_attn_pair(ModelDims md, P
           tc_commit(kv_empty((2 * kb + 2) % NST));
         }
         if (!vfull(kb)) break;
+        if (!next && end1 % 16) {
+          // V rows behind the last query, up to their group's end (a row of 128 bytes keeps its place in the swizzle)
+          uint8_t* v = sm + Sh::OFF_KV + (2 * kb + 1) % NST * Sh::T_BYTES;
+          for (int row = end1 - kb * 128; row % 16; ++row)
+            for (int a = 0; a < Sh::ATOMS; ++a)
+#pragma unroll
+              for (int c = 0; c < 8; ++c) *reinterpret_cast<uint4*>(v + a * Sh::COL + row * 128 + 16 * c) = make_uint4(0, 0, 0, 0);
+          fence_proxy_async_smem();
+        }
         for (int x = 0; x < 2 && ok; ++x) {
           if (kb < (x ? nb1 : nb0)) {
             ok = wait(p_full(x), (uint32_t)kb & 1u);

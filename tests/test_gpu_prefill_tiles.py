@@ -75,3 +75,30 @@ def test_pair_attention_blocks(tlf, hd, heads, kv):  # noqa: F811
                 np.testing.assert_array_equal(loops[b], oloops)
                 assert rel_err(lg[b], olog) < tol_for(m), (chunk, lens[b])
                 check_cache(ctx, ids[b], seqs[b], m)
+
+
+@pytest.mark.parametrize("hd,heads,kv", [(64, 4, 4), (64, 4, 1), (128, 4, 2)])
+@pytest.mark.parametrize("chunk", [8192, 256])
+def test_entries_of_released_pages_do_not_reach_a_prompt(tlf, hd, heads, kv, chunk):  # noqa: F811
+    """Prompts on pages that held infinities before: the slots behind a prompt's last token are masked, and what they
+    hold must not reach its result, bit for bit (0 x infinity is NaN)."""
+    m = _small(n_heads=heads, n_kv_heads=kv, head_dim=hd, d_model=128, max_loops=2, depth_probs=(0.4, 0.6))
+    w = synth.make_weights(m)
+    rng = np.random.default_rng(hd + kv)
+    lens = [1, 15, 66, 127, 130, 257, 390]
+    prompts = [rng.integers(0, m.vocab, size=n).astype(np.int32) for n in lens]
+    ids = list(range(1, 1 + len(lens)))
+    pages = 2 * sum((n + 63) // 64 + 1 for n in lens)
+    got = []
+    for dirty in (False, True):
+        with tlf.Context(m, w, max_seqs=8, max_batch=8, max_seq_len=64 * pages, kv_pool_pages=pages, prefill_chunk=chunk) as ctx:
+            if dirty:
+                n = 64 * (pages // 2) - 1  # every page of the pool
+                bad = np.full((n, m.n_layers, kv, hd), np.inf, np.float32)
+                ctx.load_cache(99, {"positions": [np.arange(n, dtype=np.int32)] * 2, "k": [bad] * 2, "v": [bad] * 2})
+                assert ctx.stats()[1] == 0
+                ctx.release(99)
+            lg, _ = ctx.prefill(ids, prompts)
+            assert np.isfinite(lg).all()
+            got.append(lg)
+    np.testing.assert_array_equal(got[0], got[1])
