@@ -201,19 +201,26 @@ __global__ void __launch_bounds__(AttnShape<T, HD, G>::THREADS, 2) k_attn_decode
       if (*flag) {
         // last contributor: merge the partials of CTAs c_first..c_last
         __threadfence();
-        for (int t = t0; t < G * HD; t += NT) {
+        // a thread's elements of a head go together: their loads are in flight at once, and the head's maximum and
+        // factors are read once. One at a time, the merging warp took four trips over the partials of a head of 128: one
+        // row of 3000 keys, 8 heads x 128, 22.4 us, now 16.2 (17.0 before there was a merging warp); 8 rows of 300-700
+        // keys 19.0, now 14.8 (16.0).
+        constexpr int E = HD > NT ? HD / NT : 1;
+        for (int t = t0; t < G * HD; t += NT * E) {
           const int gg = t / HD, e = t % HD;
           float mx = -INFINITY;
           for (int c = c_first; c <= c_last; ++c)
             mx = fmaxf(mx, __ldcg(part + (size_t)(item + c) * PSZ + gg * (HD + 2) + HD));
-          float o = 0.f, l = 0.f;
+          float o[E] = {}, l = 0.f;
           for (int c = c_first; c <= c_last; ++c) {
             const float* pp = part + (size_t)(item + c) * PSZ + gg * (HD + 2);
             const float f = exp2f(__ldcg(pp + HD) - mx);
-            o = fmaf(f, __ldcg(pp + e), o);
+#pragma unroll
+            for (int i = 0; i < E; ++i) o[i] = fmaf(f, __ldcg(pp + e + NT * i), o[i]);
             l = fmaf(f, __ldcg(pp + HD + 1), l);
           }
-          store_o(k, h * G + gg, e, o / l);
+#pragma unroll
+          for (int i = 0; i < E; ++i) store_o(k, h * G + gg, e + NT * i, o[i] / l);
         }
         if (t0 == 0) cnt[item] = 0;  // ready for the next launch
       }
