@@ -63,7 +63,6 @@ struct AttnShape {
   // item, 8 rows of 300-700 keys: 14.4 us, 15.5 with the one warp). With more query heads a kv head the tenth warp's
   // registers cost more than the barriers: 100 rows of 30-500 keys, 16 / 8 heads x 128, 40 -> 51 us.
   static constexpr bool MERGER = G == 1;
-  static constexpr int REDS = MERGER ? 4 : 1;
   static constexpr int THREADS = 32 * (ATT_WARPS + 1 + (MERGER ? 1 : 0));
   static constexpr int TEAM_WARPS = ATT_WARPS / TEAMS;
   static constexpr int KEYS_PER_WARP = ATT_PS / TEAM_WARPS;
@@ -72,13 +71,24 @@ struct AttnShape {
   static_assert(STEPS >= 1, "page too small for the warp split");
 };
 
-// MASKED (the dense-cache ablation): each stage also holds the page's 64 positions, -1 = masked slot.
+// Merge buffers. MASKED (the dense-cache ablation): each stage also holds the page's 64 positions, -1 = masked slot, and
+// heads of 128 give up a buffer for them, so that two CTAs still share an SM (16 rows of 2000 keys, 16 heads x 128: a
+// step of 872 us; 1079 with four buffers and one CTA an SM; 898 before there were several).
+template <typename T, int HD, int G, bool MASKED>
+constexpr int attn_reds() { return !AttnShape<T, HD, G>::MERGER ? 1 : MASKED && HD == 128 ? 3 : 4; }
 template <typename T, int HD, int G, bool MASKED>
 constexpr int attn_smem_bytes() {
   using S = AttnShape<T, HD, G>;
-  return 128 + S::NST * S::STAGE_BYTES + S::REDS * ATT_WARPS * G * (HD + 2) * 4 + (MASKED ? S::NST * ATT_PS * 4 : 0) +
-         2 * (S::NST + S::REDS) * 8 + 16;
+  constexpr int REDS = attn_reds<T, HD, G, MASKED>();
+  return 128 + S::NST * S::STAGE_BYTES + REDS * ATT_WARPS * G * (HD + 2) * 4 + (MASKED ? S::NST * ATT_PS * 4 : 0) +
+         2 * (S::NST + REDS) * 8 + 16;
 }
+// Whether the shared memory of two CTAs fits an SM (228 KB, 1 KB of it reserved for each CTA).
+template <typename T, int HD, int G, bool MASKED>
+constexpr bool attn_two_per_sm() { return 2 * (attn_smem_bytes<T, HD, G, MASKED>() + 1024) <= 233472; }
+static_assert(attn_two_per_sm<bf16, 128, 1, true>() && attn_two_per_sm<bf16, 64, 1, true>() &&
+                  attn_two_per_sm<bf16, 32, 1, true>() && attn_two_per_sm<bf16, 128, 1, false>(),
+              "the merge buffers cost the second CTA of an SM");
 
 __device__ __forceinline__ void consumer_sync() {
   asm volatile("bar.sync 1, %0;" ::"n"(32 * ATT_WARPS) : "memory");
@@ -91,6 +101,7 @@ __global__ void __launch_bounds__(AttnShape<T, HD, G>::THREADS, 2) k_attn_decode
                                                              const float* __restrict__ Q, float* __restrict__ part,
                                                              T* __restrict__ O, int* __restrict__ cnt, bool o_lo) {
   using S = AttnShape<T, HD, G>;
+  constexpr int REDS = attn_reds<T, HD, G, MASKED>();
   // output element (token k, query head hq, dim e); with o_lo also the lo plane of the
   // projection's two-term operand (bf16 of the rounding remainder, max_batch rows down)
   auto store_o = [&](int k, int hq, int e, float val) {
@@ -104,12 +115,12 @@ __global__ void __launch_bounds__(AttnShape<T, HD, G>::THREADS, 2) k_attn_decode
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
   uint8_t* ring = smem;                                                   // [NST][K seg | V seg]
   float* red = reinterpret_cast<float*>(ring + S::NST * S::STAGE_BYTES);  // [warps][G][HD + 2]
-  int* mring = reinterpret_cast<int*>(red + S::REDS * ATT_WARPS * PSZ);              // [NST][64] positions (MASKED)
+  int* mring = reinterpret_cast<int*>(red + REDS * ATT_WARPS * PSZ);       // [NST][64] positions (MASKED)
   uint64_t* full = reinterpret_cast<uint64_t*>(mring + (MASKED ? S::NST * ATT_PS : 0));
   uint64_t* empty = full + S::NST;
   uint64_t* red_full = empty + S::NST;       // [REDS] an item's parts of all warps are in its buffer (MERGER)
-  uint64_t* red_empty = red_full + S::REDS;  // [REDS] and merged
-  int* flags = reinterpret_cast<int*>(red_empty + S::REDS);  // last contributor: consumers, merging warp
+  uint64_t* red_empty = red_full + REDS;     // [REDS] and merged
+  int* flags = reinterpret_cast<int*>(red_empty + REDS);  // last contributor: consumers, merging warp
   volatile int* abort_flag = flags + 2;  // set when a bounded wait runs out: later waits are skipped
 
   pdl_wait();
@@ -131,7 +142,7 @@ __global__ void __launch_bounds__(AttnShape<T, HD, G>::THREADS, 2) k_attn_decode
       mbar_init(smem_u32(&full[i]), 1);
       mbar_init(smem_u32(&empty[i]), S::TEAM_WARPS);
     }
-    for (int i = 0; i < S::REDS; ++i) {
+    for (int i = 0; i < REDS; ++i) {
       mbar_init(smem_u32(&red_full[i]), ATT_WARPS);
       mbar_init(smem_u32(&red_empty[i]), 1);
     }
@@ -280,8 +291,8 @@ __global__ void __launch_bounds__(AttnShape<T, HD, G>::THREADS, 2) k_attn_decode
     int k, h, g;
     locate(p0, k, h, g);
     for (int p = p0, it = 0; (p += pages_of(k) - g) < p1; ++it) {  // the items before the CTA's last
-      const int b = it % S::REDS;
-      if (!*abort_flag && !mbar_wait(smem_u32(&red_full[b]), (it / S::REDS) & 1, s.err)) *abort_flag = 1;
+      const int b = it % REDS;
+      if (!*abort_flag && !mbar_wait(smem_u32(&red_full[b]), (it / REDS) & 1, s.err)) *abort_flag = 1;
       finish_item(red + b * ATT_WARPS * PSZ, flags + 1, k, h, lane, std::integral_constant<int, 32>{}, [] { __syncwarp(); });
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&red_empty[b]));
@@ -392,7 +403,7 @@ __global__ void __launch_bounds__(AttnShape<T, HD, G>::THREADS, 2) k_attn_decode
     const bool item_end = (g + 1 == pages_of(k));
     if (item_end || p + 1 == p1) {
       // ---- this CTA's part of item (k, h) is done: merge the lane groups, then the warps ----
-      const int b = it % S::REDS;
+      const int b = it % REDS;
       float* mred = red + b * ATT_WARPS * PSZ;
 #pragma unroll
       for (int gg = 0; gg < G; ++gg) {
@@ -403,8 +414,8 @@ __global__ void __launch_bounds__(AttnShape<T, HD, G>::THREADS, 2) k_attn_decode
           for (int e = 0; e < S::VEC; ++e) acc[gg][e] += __shfl_xor_sync(0xffffffffu, acc[gg][e], o);
         }
       }
-      if (S::MERGER && it >= S::REDS && !*abort_flag &&
-          !mbar_wait(smem_u32(&red_empty[b]), ((it / S::REDS) - 1) & 1, s.err))
+      if (S::MERGER && it >= REDS && !*abort_flag &&
+          !mbar_wait(smem_u32(&red_empty[b]), ((it / REDS) - 1) & 1, s.err))
         *abort_flag = 1;
       ++it;
       if (grp == 0) {

@@ -39,3 +39,14 @@ def test_items_of_a_cta(T, lens, heads, hd, dtype):  # noqa: F811
             assert np.max(np.abs(got[b] - want[b])) < tol * np.max(np.abs(want[b])), b
         first = got if first is None else first
         np.testing.assert_array_equal(got, first)
+
+
+@pytest.mark.parametrize("hd", [64, 128])
+def test_items_of_a_masked_cta(hd):
+    """Full-length caches (the dense-cache ablation) with more items a CTA than merge buffers: 250 rows of a page each over
+    8 kv heads leave a CTA seven."""
+    from paper_2609_15160_gb300 import build, tlf
+    from test_gpu_parity import _prefill_decode_compare, _small
+    build.build()
+    m = _small(n_heads=8, n_kv_heads=8, head_dim=hd, n_layers=1, max_loops=2, depth_probs=(0.5, 0.5))
+    _prefill_decode_compare(tlf, m, [1 + b % 3 for b in range(250)], steps=2, ablation="dense_cache")
