@@ -55,14 +55,16 @@ struct AttnShape {
   // Page teams: with one query head a kv head the warps' chain per page, not its instructions, is what a page costs, so
   // two teams of four warps take the pages in turn (a ring stage then always belongs to one team, so its depth is even).
   // With the registers of two CTAs an SM: 200 rows of 64-700 keys, 16 heads x 64, 80 -> 69 us; 32 rows of 128-8192 keys
-  // 98.5 -> 95 us.
-  static constexpr int TEAMS = G == 1 && NST % 2 == 0 ? 2 : 1;
+  // 98.5 -> 95 us. A ring of two stages is too short for two teams (float32 heads of 128: 32 rows of 128-8192 keys, 8
+  // heads, 178 us, 173 with one).
+  static constexpr int TEAMS = G == 1 && NST >= 4 && NST % 2 == 0 ? 2 : 1;
   // A warp of its own merges the parts of all items of a CTA but the last, out of REDS buffers, while the consumer warps
   // go on without a barrier: the 200 rows above 69 -> 62 us (5.1 TB/s), the 32 rows 95 -> 93 us (6.0 TB/s), 64 rows of
   // 500-1500 keys, 8 heads x 128, 50 us. The last item is the launch's tail, where all warps merge faster (one CTA an
   // item, 8 rows of 300-700 keys: 14.4 us, 15.5 with the one warp). With more query heads a kv head the tenth warp's
-  // registers cost more than the barriers: 100 rows of 30-500 keys, 16 / 8 heads x 128, 40 -> 51 us.
-  static constexpr bool MERGER = G == 1;
+  // registers cost more than the barriers: 100 rows of 30-500 keys, 16 / 8 heads x 128, 40 -> 51 us. Float32 heads of 128
+  // (one CTA an SM): 200 rows of 1-64 keys 31.4 us with the warp, 29.2 without.
+  static constexpr bool MERGER = G == 1 && HD * sizeof(T) <= 256;
   static constexpr int THREADS = 32 * (ATT_WARPS + 1 + (MERGER ? 1 : 0));
   static constexpr int TEAM_WARPS = ATT_WARPS / TEAMS;
   static constexpr int KEYS_PER_WARP = ATT_PS / TEAM_WARPS;
@@ -94,12 +96,18 @@ __device__ __forceinline__ void consumer_sync() {
   asm volatile("bar.sync 1, %0;" ::"n"(32 * ATT_WARPS) : "memory");
 }
 
-// Two CTAs an SM: the bound gives one query head the registers it can use (56 otherwise), and keeps four heads (131
-// otherwise, one CTA) at two: 36 rows of about 2950 keys, 32 / 8 heads x 128, 153 -> 141 us.
+// CTAs an SM that the registers are bounded for: two where the shared memory lets them, which gives one query head the
+// registers it can use (96; 56 otherwise). Four heads then spill (96 registers, 180 to 224 bytes), which still pays at
+// head_dim 64 (200 rows of 1-64 keys, 32 / 8 heads, 35.3 us, 38.6 with one CTA an SM; one row of 100 keys 13.0 and 12.8),
+// but not at 128, where one CTA an SM takes 168: one row of 3000 keys, 16 / 4 heads, 28.7 us (33.3 with two CTAs), 36
+// rows of about 2950 keys, 32 / 8 heads, 136 us (142), though 200 rows of 1-64 keys 47.7 us (45.5).
 template <typename T, int HD, int G, bool MASKED>
-__global__ void __launch_bounds__(AttnShape<T, HD, G>::THREADS, 2) k_attn_decode(ModelDims md, StepDev s, int r, int j,
-                                                             const float* __restrict__ Q, float* __restrict__ part,
-                                                             T* __restrict__ O, int* __restrict__ cnt, bool o_lo) {
+constexpr int attn_ctas_per_sm() { return attn_two_per_sm<T, HD, G, MASKED>() && !(HD == 128 && G == 4) ? 2 : 1; }
+
+template <typename T, int HD, int G, bool MASKED>
+__global__ void __launch_bounds__(AttnShape<T, HD, G>::THREADS, attn_ctas_per_sm<T, HD, G, MASKED>())
+    k_attn_decode(ModelDims md, StepDev s, int r, int j, const float* __restrict__ Q, float* __restrict__ part,
+                  T* __restrict__ O, int* __restrict__ cnt, bool o_lo) {
   using S = AttnShape<T, HD, G>;
   constexpr int REDS = attn_reds<T, HD, G, MASKED>();
   // output element (token k, query head hq, dim e); with o_lo also the lo plane of the
