@@ -40,6 +40,13 @@ using namespace tlf;
 namespace {
 thread_local std::string g_create_error = "no error";
 
+// How a step runs the shared block.
+enum class StepPath {
+  launches,  // a launch per stage
+  small,     // the persistent kernel (k_step.cu)
+  rows,      // one CTA per row (k_step_row.cu)
+};
+
 struct DeviceMat {
   void* ptr = nullptr;
   int N = 0, K = 0;
@@ -79,8 +86,8 @@ struct tlf_ctx {
   bool split_norm = false;      // pre-norms split across the neighbouring GEMMs (tcgen05 path)
   bool operand_lo = false;      // X, O, U carry a lo plane (two-term GEMM operands, tcgen05 path)
   bool pf_ws = true;            // prefill attention: the warp-specialised tensor-map kernel
-  bool step_row = false;        // float32 steps over short caches run the block one CTA per row
-  bool step_small = false;      // steps of up to 16 rows run the block in the persistent kernel
+  bool step_row = false;        // float32 steps may run the block one CTA per row (step_path)
+  bool step_small = false;      // steps of up to 16 rows may run the block in the persistent kernel (step_path)
   float* d_part_small = nullptr;  // its attention partials
   float* d_ss8 = nullptr;       // [16][d / 8] its sums of squares
   unsigned* d_gbar = nullptr;   // its grid barrier
@@ -167,7 +174,8 @@ struct tlf_ctx {
   // CUDA graphs of the step
   struct StepGraph {
     int B;
-    bool logits, rows;
+    bool logits;
+    StepPath path;
     cudaGraphExec_t exec;
     int launches;
   };
@@ -809,8 +817,7 @@ static CondArgs cond_args(const tlf_ctx* ctx, const int* m, int r, int j, int pa
   return c;
 }
 
-// rows: the block one CTA per row (float32 models; every cache of the step holds at most RowStep::MAX_KEYS entries).
-static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, bool rows, bool prof, cudaStream_t st) {
+static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, StepPath path, bool prof, cudaStream_t st) {
   const ModelDims& md = ctx->md;
   const int M = md.M, J = md.J, maxB = md.max_batch;
   CK(ctx, cudaMemcpyAsync(ctx->d_upload, ctx->h_upload, ctx->upload_ints * 4, cudaMemcpyHostToDevice, st));
@@ -860,11 +867,7 @@ static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, bool rows, bool p
   const int lo_rows = ctx->operand_lo ? maxB : 0;
   void* x_lo = ctx->operand_lo ? static_cast<void*>(reinterpret_cast<bf16*>(ctx->d_X) + (size_t)maxB * md.d) : nullptr;
   void* u_lo = ctx->operand_lo ? static_cast<void*>(reinterpret_cast<bf16*>(ctx->d_U) + (size_t)maxB * md.ff) : nullptr;
-  // Up to 16 rows: the whole block as one persistent kernel (a profiled step keeps a launch per stage, so
-  // that each can be timed; so does a context whose cooperative launch was refused, as for a stream that may use fewer
-  // SMs than the device has).
-  bool small = ctx->step_small && B <= SS_ROWS && !prof;
-  if (small) {
+  if (path == StepPath::small) {
     launch_norm_rows(md.dtype, ctx->d_H, md.d, ctx->d_idx, ctx->d_n, 0, B, ctx->d_attn_norm, md.d, md.eps, ctx->d_X, md.d,
                      st, cond_args(ctx, s.m, 0, 0, 2), ctx->d_ss, x_lo);
     SmallStep a{};
@@ -883,15 +886,16 @@ static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, bool rows, bool p
     a.rope = ctx->d_rope;
     a.cond = ctx->d_cond;
     a.gbar = ctx->d_gbar;
-    small = launch_step_small(a, ctx->num_sms, st) == cudaSuccess;
-    if (small) {
+    if (launch_step_small(a, ctx->num_sms, st) == cudaSuccess) {
       ctx->last_launches += 2;
     } else {
+      // refused, as on a stream that may use fewer SMs than the device has: this and later steps go by launches
       cudaGetLastError();
       ctx->step_small = false;
+      path = StepPath::launches;
     }
   }
-  if (rows) {
+  if (path == StepPath::rows) {
     RowStep a{};
     a.md = md;
     a.s = s;
@@ -906,7 +910,7 @@ static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, bool rows, bool p
     CK(ctx, launch_step_row(a, B, st));
     ctx->last_launches += 1;
   }
-  for (int r = 0; r < M && !small && !rows; ++r) {
+  for (int r = 0; r < M && path == StepPath::launches; ++r) {
     const int* n_dev = ctx->d_n + r;
     const int* idx_r = ctx->d_idx + (size_t)r * maxB;
     // rows that do not run loop r but are computed anyway (no-gather ablation) keep their residual
@@ -1040,7 +1044,7 @@ static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, bool rows, bool p
       ++ctx->last_launches;  // the attention (GEMMs counted in gemm(), norms where launched)
     }
   }
-  if (!rows) {
+  if (path != StepPath::rows) {
     launch_final(md, s, B, ctx->d_final_norm, ctx->d_Xf, st);
     mark(11);
     ++ctx->last_launches;
@@ -1061,11 +1065,35 @@ static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, bool rows, bool p
   return TLF_OK;
 }
 
-// The step as one CUDA graph per (batch size, logits on/off), built on first
+// The path of a step over the given sequences. A profiled step keeps a launch per stage, so that each can be timed.
+//
+// Persistent kernel: it saves a launch's fixed cost per stage, but its groups of warps stream pages slower than the CTAs
+// of k_attn_decode, and the more rows the sooner that shows: it takes steps whose first loop leaves a group of warps (two
+// a CTA) at most 112 pages, and at most 900 / rows. Mid-size model, launches against this kernel: 16 rows of 1000 / 8000
+// keys (14 / 106 pages a group) 1254 / 2060 and 1148 / 2154 us; 12 rows of 8000 (80) 1813 and 1800 us; 4 rows of 30000
+// (99) 1904 and 1797 us. Small model: 16 rows of 8000 / 20000 keys (53 / 132) 534 / 824 and 525 / 908 us. With head_dim
+// 32: 12 rows of 16000 (158) 1110 and 1143 us, 8 rows of 16000 (106) 891 and 853 us.
+static StepPath step_path(const tlf_ctx* ctx, int B, const int* slots, bool prof) {
+  const ModelDims& md = ctx->md;
+  if (prof) return StepPath::launches;
+  if (ctx->step_small && B <= SS_ROWS) {
+    long long pages = 0;
+    for (int b = 0; b < B; ++b) pages += (ctx->h_len[(size_t)slots[b] * md.M] + md.page_size) / md.page_size;
+    return pages * md.Hkv <= (long long)2 * ctx->num_sms * std::min(112, 900 / B) ? StepPath::small : StepPath::launches;
+  }
+  if (ctx->step_row) {
+    int keys = 0;
+    for (int b = 0; b < B; ++b) keys = std::max(keys, ctx->h_len[(size_t)slots[b] * md.M] + 1);
+    if (keys <= RowStep::MAX_KEYS) return StepPath::rows;
+  }
+  return StepPath::launches;
+}
+
+// The step as one CUDA graph per (batch size, logits on/off, path), built on first
 // use after the kernels have run once directly (their attributes are set).
-static cudaGraphExec_t step_graph(tlf_ctx* ctx, int B, bool need_logits, bool rows) {
+static cudaGraphExec_t step_graph(tlf_ctx* ctx, int B, bool need_logits, StepPath path) {
   for (auto& g : ctx->graphs)
-    if (g.B == B && g.logits == need_logits && g.rows == rows) {
+    if (g.B == B && g.logits == need_logits && g.path == path) {
       ctx->last_launches = g.launches;
       return g.exec;
     }
@@ -1078,7 +1106,7 @@ static cudaGraphExec_t step_graph(tlf_ctx* ctx, int B, bool need_logits, bool ro
     return nullptr;
   }
   const bool small = ctx->step_small;
-  const int rc = enqueue_step(ctx, B, need_logits, rows, false, ctx->cap_stream);
+  const int rc = enqueue_step(ctx, B, need_logits, path, false, ctx->cap_stream);
   const cudaError_t e1 = cudaStreamEndCapture(ctx->cap_stream, &graph);
   if (rc != TLF_OK || e1 != cudaSuccess || cudaGraphInstantiate(&exec, graph, 0) != cudaSuccess) {
     cudaGetLastError();
@@ -1088,7 +1116,7 @@ static cudaGraphExec_t step_graph(tlf_ctx* ctx, int B, bool need_logits, bool ro
     return nullptr;
   }
   cudaGraphDestroy(graph);
-  ctx->graphs.push_back({B, need_logits, rows, exec, ctx->last_launches});
+  ctx->graphs.push_back({B, need_logits, path, exec, ctx->last_launches});
   return exec;
 }
 
@@ -1109,27 +1137,22 @@ static int run_step(tlf_ctx* ctx, int B, const int* slots, const int* tokens, co
     h[1 + 2 * B + b] = slots[b];
   }
   memcpy(h + 1 + 3 * B, upd.data(), nu * sizeof(PageUpdate));
-  bool rows = ctx->step_row && !prof;
-  for (int b = 0; b < B && rows; ++b) rows = ctx->h_len[(size_t)slots[b] * M] + 1 <= RowStep::MAX_KEYS;
-  cudaGraphExec_t exec = prof ? nullptr : step_graph(ctx, B, need_logits, rows);
+  StepPath path = step_path(ctx, B, slots, prof);
+  cudaGraphExec_t exec = prof ? nullptr : step_graph(ctx, B, need_logits, path);
   if (exec) {
     const cudaError_t e = cudaGraphLaunch(exec, st);
-    if (e != cudaSuccess && ctx->step_small && B <= SS_ROWS) {
-      // the graph holds the persistent kernel: this and later steps run without it
+    if (e != cudaSuccess && path == StepPath::small) {
+      // the persistent kernel is refused: this and later steps run without it
       cudaGetLastError();
       ctx->step_small = false;
-      for (size_t i = ctx->graphs.size(); i-- > 0;)
-        if (ctx->graphs[i].B <= SS_ROWS) {
-          cudaGraphExecDestroy(ctx->graphs[i].exec);
-          ctx->graphs.erase(ctx->graphs.begin() + i);
-        }
+      path = StepPath::launches;
       exec = nullptr;
     } else {
       CK(ctx, e);
     }
   }
   if (!exec) {
-    const int rc = enqueue_step(ctx, B, need_logits, rows, prof, st);
+    const int rc = enqueue_step(ctx, B, need_logits, path, prof, st);
     if (rc) return rc;
     ctx->warmed = true;
   }

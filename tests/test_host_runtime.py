@@ -140,3 +140,27 @@ def test_a_refused_cooperative_launch_falls_back_to_a_launch_per_stage(lib, loop
             lib.fake_refuse_cooperative(0)
             lib.fake_refuse_graph(0)
         assert ctx.cache_len(1, 1) == 10 + good + 5
+
+
+def _kernel_of_step(lib, ctx, ids):
+    """Which kernel ran the block of a (directly launched) step."""
+    names = (b"k_step_small", b"k_step_row", b"k_attn_decode")
+    before = [lib.fake_launches(n) for n in names]
+    ctx.decode_step(ids, [5] * len(ids), logits=False)
+    ran = [n for n, b in zip(names, before) if lib.fake_launches(n) > b]
+    assert len(ran) == 1
+    return ran[0].decode()
+
+
+@pytest.mark.parametrize("rows,pages_a_group,want", [(1, 100, "k_step_small"), (1, 125, "k_attn_decode"),
+                                                     (8, 100, "k_step_small"), (16, 50, "k_step_small"),
+                                                     (16, 65, "k_attn_decode")])
+def test_the_persistent_step_leaves_long_caches_to_the_launches(lib, monkeypatch, rows, pages_a_group, want):
+    """The rule counts the pages of the first loop that each of the kernel's 2 x 152 groups of warps gets."""
+    monkeypatch.setenv("TLF_NO_GRAPH", "1")
+    m = _model(n_heads=8, n_kv_heads=8, head_dim=32, n_layers=1, max_loops=2)
+    keys = pages_a_group * 304 * 64 // (8 * rows)
+    with _context(m, max_seqs=rows, max_batch=rows, max_seq_len=keys + 10, kv_pool_pages=rows * 2 * (keys // 64 + 2)) as ctx:
+        for i in range(rows):
+            ctx.load_cache(i, {"positions": [np.arange(keys, dtype=np.int32), np.arange(0, dtype=np.int32)]})
+        assert _kernel_of_step(lib, ctx, list(range(rows))) == want
