@@ -284,12 +284,17 @@ __global__ void __launch_bounds__(SR_THREADS, 1) k_step_row(RowStep a) {
   if (tid < m) s.len[slot * M + tid] += 1;
 }
 
-// Whether a step of this model may run row by row: the widths its shared memory takes, and a layer small enough to be
-// read by one SM (1 MB, about 10 us at an SM's share of L2, against some 25 us for the layer's launches).
+// Whether a step of this model may run row by row: the widths its shared memory takes, and layers of up to 1 MB (which
+// steps do depends on their caches too).
 bool step_row_fits(const ModelDims& md) {
   if (md.dtype != 0 || md.J > SS_LAYERS || md.d % 4 || md.ff % 4) return false;
   const SrLayout l = sr_layout(md, RowStep::MAX_KEYS);
   return (long long)l.weights / md.J * 4 <= (1 << 20) && (long long)l.total_act * 4 <= SR_SMEM && md.d <= SR_THREADS;
+}
+
+long long step_row_weight_bytes(const ModelDims& md) {
+  const SrLayout l = sr_layout(md, RowStep::MAX_KEYS);
+  return (long long)(l.total_act + l.weights) * 4 <= SR_SMEM ? 0 : (long long)l.weights / md.J * 4;
 }
 
 cudaError_t launch_step_row(RowStep a, int B, cudaStream_t st) {

@@ -87,6 +87,7 @@ struct tlf_ctx {
   bool operand_lo = false;      // X, O, U carry a lo plane (two-term GEMM operands, tcgen05 path)
   bool pf_ws = true;            // prefill attention: the warp-specialised tensor-map kernel
   bool step_row = false;        // float32 steps may run the block one CTA per row (step_path)
+  long long row_bytes = 0;      // weights that a row's CTA then reads through L2 at every (loop, layer)
   bool step_small = false;      // steps of up to 16 rows may run the block in the persistent kernel (step_path)
   float* d_part_small = nullptr;  // its attention partials
   float* d_ss8 = nullptr;       // [16][d / 8] its sums of squares
@@ -645,6 +646,7 @@ static int create_impl(tlf_ctx* ctx, const tlf_weights* w) {
     ctx->split_norm = ctx->use_tc && !(e && e[0] == '1');
   }
   ctx->step_row = c.ablation == TLF_ABLATION_NONE && step_row_fits(md);
+  ctx->row_bytes = step_row_weight_bytes(md);
   ctx->step_small = ctx->split_norm && ctx->operand_lo && c.ablation == TLF_ABLATION_NONE &&
                     step_small_fits(md, ctx->num_sms);
   if (ctx->step_small) {
@@ -1073,6 +1075,13 @@ static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, StepPath path, bo
 // keys (14 / 106 pages a group) 1254 / 2060 and 1148 / 2154 us; 12 rows of 8000 (80) 1813 and 1800 us; 4 rows of 30000
 // (99) 1904 and 1797 us. Small model: 16 rows of 8000 / 20000 keys (53 / 132) 534 / 824 and 525 / 908 us. With head_dim
 // 32: 12 rows of 16000 (158) 1110 and 1143 us, 8 rows of 16000 (106) 891 and 853 us.
+//
+// One CTA per row: what one SM reads through L2 for the longest row at each (loop, layer), the layer's weights unless
+// they are staged and every head's K and V, takes it about 20 us a megabyte, and the stages' launches some 25 us, more
+// with many rows, which they run 32 at a time: up to 1 MB, from 128 rows on 1.75 MB. Two layers of width 192 (996 KB of weights) at
+// 32 / 300 keys (1.0 / 1.5 MB): one row 237 / 247 us by launches, 213 / 289 us so; 64 rows 423 / 468 and 306 / 489 us; 128
+// rows 647 / 674 and 374 / 547 us, and with 600 keys (1.9 MB) 730 and 708 us. Width 128, 393 KB of weights, 600 keys (1.0 MB), one row:
+// 129 and 127 us; 256 rows 612 and 477 us. The tiny model (staged) gains at every size: 1 / 256 rows 133 / 574 and 66 / 177 us.
 static StepPath step_path(const tlf_ctx* ctx, int B, const int* slots, bool prof) {
   const ModelDims& md = ctx->md;
   if (prof) return StepPath::launches;
@@ -1084,7 +1093,8 @@ static StepPath step_path(const tlf_ctx* ctx, int B, const int* slots, bool prof
   if (ctx->step_row) {
     int keys = 0;
     for (int b = 0; b < B; ++b) keys = std::max(keys, ctx->h_len[(size_t)slots[b] * md.M] + 1);
-    if (keys <= RowStep::MAX_KEYS) return StepPath::rows;
+    const long long bytes = ctx->row_bytes + 8LL * keys * md.q_dim;
+    if (keys <= RowStep::MAX_KEYS && bytes <= (B < 128 ? 1LL << 20 : 7LL << 18)) return StepPath::rows;
   }
   return StepPath::launches;
 }

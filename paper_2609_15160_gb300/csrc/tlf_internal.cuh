@@ -570,6 +570,7 @@ struct RowStep {
   int max_keys, weights_in_smem;  // set by the launcher
 };
 bool step_row_fits(const ModelDims& md);
+long long step_row_weight_bytes(const ModelDims& md);  // of a layer, read through L2 (0: all staged in shared memory)
 cudaError_t launch_step_row(RowStep a, int B, cudaStream_t st);
 
 bool step_small_fits(const ModelDims& md, int num_sms);

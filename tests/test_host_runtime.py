@@ -164,3 +164,25 @@ def test_the_persistent_step_leaves_long_caches_to_the_launches(lib, monkeypatch
         for i in range(rows):
             ctx.load_cache(i, {"positions": [np.arange(keys, dtype=np.int32), np.arange(0, dtype=np.int32)]})
         assert _kernel_of_step(lib, ctx, list(range(rows))) == want
+
+
+# layers of 996, 393 and 200 KB; the last is staged in shared memory
+ROW_MODELS = {"wide": dict(d_model=192, n_heads=3, n_kv_heads=3, head_dim=64, ffn_hidden=176),
+              "narrow": dict(d_model=128, n_heads=4, n_kv_heads=2, head_dim=32, n_layers=1, ffn_hidden=128),
+              "tiny": dict(d_model=64, n_heads=4, n_kv_heads=4, head_dim=16, n_layers=1, ffn_hidden=176)}
+
+
+@pytest.mark.parametrize("model,rows,keys,want", [
+    ("wide", 1, 30, "k_step_row"), ("wide", 1, 60, "k_attn_decode"), ("wide", 64, 300, "k_attn_decode"),
+    ("wide", 128, 300, "k_step_row"), ("wide", 256, 600, "k_attn_decode"), ("narrow", 1, 600, "k_step_row"),
+    ("narrow", 1, 700, "k_attn_decode"), ("tiny", 1, 1000, "k_step_row"), ("tiny", 256, 1000, "k_step_row"),
+    ("tiny", 1, 1024, "k_attn_decode")])
+def test_the_row_kernel_takes_what_one_sm_can_read(lib, monkeypatch, model, rows, keys, want):
+    """The rule counts a layer's weights, unless they are staged, and the K and V of the longest row's heads."""
+    monkeypatch.setenv("TLF_NO_GRAPH", "1")
+    m = _model("f32", **ROW_MODELS[model])
+    with _context(m, max_seqs=rows, max_batch=rows, max_seq_len=1100, kv_pool_pages=rows * 3 + 60) as ctx:
+        for i in range(rows):
+            n = keys if i == 0 else 3
+            ctx.load_cache(i, {"positions": [np.arange(n, dtype=np.int32)] + [np.arange(0, dtype=np.int32)] * 2})
+        assert _kernel_of_step(lib, ctx, list(range(rows))) == want
