@@ -1077,11 +1077,11 @@ static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, StepPath path, bo
 // 32: 12 rows of 16000 (158) 1110 and 1143 us, 8 rows of 16000 (106) 891 and 853 us.
 //
 // One CTA per row: what one SM reads through L2 for the longest row at each (loop, layer), the layer's weights unless
-// they are staged and every head's K and V, takes it about 20 us a megabyte, and the stages' launches some 25 us, more
-// with many rows, which they run 32 at a time: up to 1 MB, from 128 rows on 1.75 MB. Two layers of width 192 (996 KB of weights) at
-// 32 / 300 keys (1.0 / 1.5 MB): one row 237 / 247 us by launches, 213 / 289 us so; 64 rows 423 / 468 and 306 / 489 us; 128
-// rows 647 / 674 and 374 / 547 us, and with 600 keys (1.9 MB) 730 and 708 us. Width 128, 393 KB of weights, 600 keys (1.0 MB), one row:
-// 129 and 127 us; 256 rows 612 and 477 us. The tiny model (staged) gains at every size: 1 / 256 rows 133 / 574 and 66 / 177 us.
+// they are staged and every head's K and V, takes it some 20 us a megabyte; the stages' launches take some 25 us, more with
+// many rows, which they run 32 at a time. The lines cross at 1 MB for one row and at about 1.1 / 1.2 / 1.3 / 1.5 / 1.85 MB for
+// 16 / 32 / 64 / 96 / 128 rows. Two layers of width 192 (996 KB of weights) at 85 / 225 / 425 keys (1.1 / 1.3 / 1.6 MB): one row 209 /
+// 210 / 216 us by launches, 200 / 246 / 310 us so; 64 rows 360 / 389 / 408 and 254 / 312 / 455 us; 128 rows 539 / 562 / 594 and
+// 266 / 370 / 486 us. The tiny model (staged) gains at every size: at 985 keys, 1 / 256 rows, a fifth and a half.
 static StepPath step_path(const tlf_ctx* ctx, int B, const int* slots, bool prof) {
   const ModelDims& md = ctx->md;
   if (prof) return StepPath::launches;
@@ -1094,7 +1094,7 @@ static StepPath step_path(const tlf_ctx* ctx, int B, const int* slots, bool prof
     int keys = 0;
     for (int b = 0; b < B; ++b) keys = std::max(keys, ctx->h_len[(size_t)slots[b] * md.M] + 1);
     const long long bytes = ctx->row_bytes + 8LL * keys * md.q_dim;
-    if (keys <= RowStep::MAX_KEYS && bytes <= (B < 128 ? 1LL << 20 : 7LL << 18)) return StepPath::rows;
+    if (keys <= RowStep::MAX_KEYS && bytes <= std::min(200 + B, 370) * (1LL << 20) / 200) return StepPath::rows;
   }
   return StepPath::launches;
 }

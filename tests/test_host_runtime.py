@@ -173,8 +173,8 @@ ROW_MODELS = {"wide": dict(d_model=192, n_heads=3, n_kv_heads=3, head_dim=64, ff
 
 
 @pytest.mark.parametrize("model,rows,keys,want", [
-    ("wide", 1, 30, "k_step_row"), ("wide", 1, 60, "k_attn_decode"), ("wide", 64, 300, "k_attn_decode"),
-    ("wide", 128, 300, "k_step_row"), ("wide", 256, 600, "k_attn_decode"), ("narrow", 1, 600, "k_step_row"),
+    ("wide", 1, 15, "k_step_row"), ("wide", 1, 40, "k_attn_decode"), ("wide", 64, 200, "k_step_row"),
+    ("wide", 64, 300, "k_attn_decode"), ("wide", 256, 550, "k_step_row"), ("wide", 256, 650, "k_attn_decode"), ("narrow", 1, 600, "k_step_row"),
     ("narrow", 1, 700, "k_attn_decode"), ("tiny", 1, 1000, "k_step_row"), ("tiny", 256, 1000, "k_step_row"),
     ("tiny", 1, 1024, "k_attn_decode")])
 def test_the_row_kernel_takes_what_one_sm_can_read(lib, monkeypatch, model, rows, keys, want):
