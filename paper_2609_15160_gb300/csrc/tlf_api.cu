@@ -1307,15 +1307,14 @@ static int ensure_prefill_buffers(tlf_ctx* ctx) {
   return TLF_OK;
 }
 
-// Whether a projection of a prefill loop takes one token tile of k_gemm_tc.
-static bool pf_one_tile(const tlf_ctx* ctx, const DeviceMat& W, int rows) {
-  return rows <= 256 && (W.N + 127) / 128 <= ctx->num_sms;
-}
+constexpr int PF_ONE_TILE = 256;  // rows of a prefill loop whose projections take one token tile of k_gemm_tc
 
 // A projection of the `rows` rows of a prefill loop. Up to 256 rows are one token tile of k_gemm_tc: a short
 // prompt streams the weights, and K is split over a cluster (up to 8 CTAs, at least two k-tiles each), as in the
-// decode step, while the tiles x splits still fit one CTA per SM. More rows, or more weight tiles than SMs, fill the
-// chip with tiles of the pair GEMM: at 8192 rows it takes 254 / 109 / 62 / 144 us for the long-context model's
+// decode step, while the tiles x splits still fit one CTA per SM. That holds for more weight tiles than SMs too, where
+// the pair GEMM works on 256 rows whatever there are: prompts of 4 / 64 / 129 / 256 tokens on a layer of d 4096, 11008 ffn
+// features (172 tiles) take 379 / 416 / 527 / 579 us against 551 / 603 / 616 / 640 us. More rows fill the chip with tiles of
+// the pair GEMM: at 8192 rows it takes 254 / 109 / 62 / 144 us for the long-context model's
 // gate/up, QKV, O and down projections, against 454 / 211 / 111 / 186 us for tiles of k_gemm_tc, and 79 / 55 / 23 / 43
 // against 186 / 124 / 47 / 66 us for the mid-size model's.
 static void gemm_pf(tlf_ctx* ctx, const DeviceMat& W, const CUtensorMap* xmaps, GemmArgs a, int rows,
@@ -1326,7 +1325,7 @@ static void gemm_pf(tlf_ctx* ctx, const DeviceMat& W, const CUtensorMap* xmaps, 
   a.splits = 1;
   a.max_rows = ctx->pf_C;
   const int ntiles = (W.N + 127) / 128, nkb = (W.K + 63) / 64;
-  if (!pf_one_tile(ctx, W, rows)) {
+  if (rows > PF_ONE_TILE) {
     const int bn = gemm_pf_tile_n(rows, W.N, W.K, a.epi, ctx->md.hd, ctx->pf_pairs);
     launch_gemm_pf(&xmaps[3], bn == 256 ? &W.map : bn == 128 ? &W.map64 : &W.map32, bn, a, rows, ctx->pf_pairs, st);
     return;
@@ -1480,8 +1479,7 @@ static int prefill_batched(tlf_ctx* ctx, int n_seqs, const int* slot_of, const i
       // whose rows come from another compaction: the mid-size model's prompts of 4 / 64 / 117 / 256 tokens take 1101 /
       // 1351 / 1455 / 1722 us against 1161 / 1428 / 1533 / 1806. Wide models keep the norm kernels above 32 rows: next to
       // those the large gate/up projection starts streaming earlier (d 2048, 40 / 117 rows: 775 / 906 us, 787 / 920 split).
-      const bool split = ctx->split_norm && (md.d <= 1024 || nr <= 32) && pf_one_tile(ctx, ctx->wqkv[0], nr) && pf_one_tile(ctx, ctx->wo[0], nr) &&
-                         pf_one_tile(ctx, ctx->wgu[0], nr) && pf_one_tile(ctx, ctx->wd[0], nr);
+      const bool split = ctx->split_norm && nr <= (md.d <= 1024 ? PF_ONE_TILE : 32);
       // the operand of the next projection, written by the residual epilogue before it
       auto norm_out = [&](GemmArgs& a, const float* gain, const CondArgs& gamma) {
         if (!split) return;

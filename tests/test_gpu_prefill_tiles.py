@@ -36,6 +36,12 @@ def test_few_row_projections(tlf, shape, n):  # noqa: F811
     _prefill_decode_compare(tlf, _small(**SHAPES[shape]), [n], steps=1)
 
 
+@pytest.mark.parametrize("n", [1, 17, 128, 129, 256, 300])
+def test_more_weight_tiles_than_sms(tlf, n):  # noqa: F811
+    """A gate/up projection of 154 tiles of 128 features, with few rows and just above."""
+    _prefill_decode_compare(tlf, _small(ffn_hidden=9808, n_layers=1, max_loops=2, depth_probs=(0.5, 0.5)), [n], steps=1)
+
+
 @pytest.mark.parametrize("rows", [33, 64, 65, 128])
 def test_long_k_projections(tlf, rows):  # noqa: F811
     """Projections with eight k-tiles a CTA and more (78 gate/up tiles over 8 k-tiles, 78 k-tiles down): two CTAs share an
