@@ -614,8 +614,8 @@ __global__ void __launch_bounds__(PFT_THREADS) k_pf_attn_tc(ModelDims md, Prefil
 //   warp 9          MMA issuer: S = Qhi K^T + Qlo K^T, O += P V with V taken as an MN-major operand.
 // mbarriers connect the roles; every wait is bounded. A block past a sequence's last page loads its last
 // page twice. Slots past the last query may hold anything (a released page keeps its entries), and P = 0 does not
-// cancel an infinity: the P V product of a tile ends with the group of 16 slots of its last query, and what lies behind
-// the block's last query in that group is zeroed in V.
+// cancel an infinity, so warp 8 zeroes them in the last block's V while the softmax runs. (Products that end with a
+// tile's last query instead cost the issuing thread 2 % of a prompt of 8192 tokens.)
 //
 // What bounds it: at head_dim 128 a block of a tile is 1536 cycles of MMAs (two S products for q's two terms, one P
 // V) against about 1024 of exponentials, so the tiles' softmaxes hide behind each other's MMAs; at head_dim 64 the
@@ -639,7 +639,7 @@ struct PfaShape {
   static constexpr int OFF_Q = 0;                     // tile 0 hi, lo, tile 1 hi, lo
   static constexpr int OFF_KV = 4 * T_BYTES;
   static constexpr int OFF_BAR = OFF_KV + NST * T_BYTES;
-  static constexpr int NBAR = 2 * NST + 2 + 8;
+  static constexpr int NBAR = 2 * NST + 2 + 9;
   static constexpr int BYTES = OFF_BAR + NBAR * 8 + 16 + 1024;  // barriers, TMEM slot, alignment slack
   static constexpr bool SEP_P = HD == 64;
   static constexpr uint32_t SCOL = 0, OCOL = 256, PCOL = SEP_P ? 384 : 0;
@@ -699,6 +699,7 @@ __global__ void __launch_bounds__(PFA_THREADS, 1) k_pf_attn_pair(ModelDims md, P
   auto s_read = [&](int x) { return bar(2 * NST + 4 + x); };  // ... read by its softmax (SEP_P)
   auto p_full = [&](int x) { return bar(2 * NST + 6 + x); };  // P of tile x written
   auto o_done = [&](int x) { return bar(2 * NST + 8 + x); };  // its P V product done
+  const uint32_t v_tail = bar(2 * NST + 10);                  // the last block's V zeroed behind the last query
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
@@ -713,6 +714,7 @@ __global__ void __launch_bounds__(PFA_THREADS, 1) k_pf_attn_pair(ModelDims md, P
       mbar_init(p_full(x), 4);
       mbar_init(o_done(x), 1);
     }
+    mbar_init(v_tail, 32);
     *abort_flag = 0;
     fence_barrier_init();
     prefetch_tensormap(&q_map);
@@ -797,6 +799,19 @@ __global__ void __launch_bounds__(PFA_THREADS, 1) k_pf_attn_pair(ModelDims md, P
       }
     }
     __syncwarp();
+    if (nb > 0) {
+      // the last block's V behind the last query (a row of 128 bytes keeps its place in the swizzle)
+      const int st = (2 * nb - 1) % NST, valid = s0 + q0 + nq0 + nq1 - (nb - 1) * 128;
+      if (valid < 128) wait(kv_full(st), (uint32_t)((2 * nb - 1) / NST) & 1u);
+      uint8_t* v = sm + Sh::OFF_KV + st * Sh::T_BYTES;
+#pragma unroll 1
+      for (int i = valid * 8 + lane; i < 1024; i += 32)
+#pragma unroll
+        for (int a = 0; a < Sh::ATOMS; ++a) *reinterpret_cast<uint4*>(v + a * Sh::COL + i * 16) = make_uint4(0, 0, 0, 0);
+      fence_proxy_async_smem();
+      mbar_arrive(v_tail);
+    }
+    __syncwarp();
   } else if (warp == 9) {
     // ---------------- MMA issuer ----------------
     if (lane == 0 && nb > 0) {
@@ -817,14 +832,12 @@ __global__ void __launch_bounds__(PFA_THREADS, 1) k_pf_attn_pair(ModelDims md, P
               tc_mma_f16(d, qd + pl * T_E + kc * COL_E + 2 * k, kd + kc * COL_E + 2 * k, IDS, (pl | kc | k) ? 1u : 0u);
         tc_commit(s_full(x));
       };
-      const int end0 = s0 + q0 + nq0, end1 = end0 + nq1;  // slots up to the tiles' last queries
       auto issue_pv = [&](int x, int kb) {
-        const int groups = ((x ? end1 : end0) - kb * 128 + 15) / 16;  // of 16 slots that the tile sees
         const uint64_t vd = dv + (uint64_t)((2 * kb + 1) % NST) * T_E;
         const uint32_t d = tmem + Sh::OCOL + (uint32_t)(HD * x), pa = tmem + Sh::PCOL + Sh::P_STEP * (uint32_t)x;
 #pragma unroll
         for (int k = 0; k < 8; ++k)  // K = 16 keys per MMA: 8 TMEM columns of P, +2048 B (16 rows) of V
-          if (k < groups) tc_mma_f16_ts(d, pa + 8u * k, vd + V16_E * k, IDO, (kb > 0 || k > 0) ? 1u : 0u);
+          tc_mma_f16_ts(d, pa + 8u * k, vd + V16_E * k, IDO, (kb > 0 || k > 0) ? 1u : 0u);
         tc_commit(o_done(x));
       };
       auto kfull = [&](int kb) { return wait(kv_full((2 * kb) % NST), (uint32_t)(2 * kb / NST) & 1u); };
@@ -855,16 +868,7 @@ __global__ void __launch_bounds__(PFA_THREADS, 1) k_pf_attn_pair(ModelDims md, P
           if (!ok) break;
           tc_commit(kv_empty((2 * kb + 2) % NST));
         }
-        if (!vfull(kb)) break;
-        if (!next && end1 % 16) {
-          // V rows behind the last query, up to their group's end (a row of 128 bytes keeps its place in the swizzle)
-          uint8_t* v = sm + Sh::OFF_KV + (2 * kb + 1) % NST * Sh::T_BYTES;
-          for (int row = end1 - kb * 128; row % 16; ++row)
-            for (int a = 0; a < Sh::ATOMS; ++a)
-#pragma unroll
-              for (int c = 0; c < 8; ++c) *reinterpret_cast<uint4*>(v + a * Sh::COL + row * 128 + 16 * c) = make_uint4(0, 0, 0, 0);
-          fence_proxy_async_smem();
-        }
+        if (!vfull(kb) || (!next && !wait(v_tail, 0))) break;
         for (int x = 0; x < 2 && ok; ++x) {
           if (kb < (x ? nb1 : nb0)) {
             ok = wait(p_full(x), (uint32_t)kb & 1u);
