@@ -92,21 +92,19 @@ constexpr int tc_body_bytes(int nt, int stages, bool lo) {
 constexpr int tc_tmem_cols(int nt, bool lo) {
   return lo ? (2 * nt < 32 ? 32 : 2 * nt) : (nt < 32 ? 32 : nt);
 }
-// tcgen05.alloc blocks until columns are free, so the CTAs that shared memory lets
-// share an SM must fit in its 512 TMEM columns (otherwise clusters waiting for
-// partners could wait on each other): launches request at least this much.
-constexpr int SM_SMEM = 232448;  // shared memory per SM available to CTAs (227 KB + 1 KB per CTA)
-constexpr int tc_min_smem(int nt, bool lo) { return SM_SMEM / (512 / tc_tmem_cols(nt, lo) + 1) - 1024 + 1; }
+constexpr int SM_SMEM = 232448;  // most shared memory of one CTA (227 KB)
+constexpr int tc_used_smem(int nt, int stages, bool lo) {
+  return 1024 /*align slack*/ + tc_body_bytes(nt, stages, lo) + 256 /*barriers, tmem slot*/ + nt * (16 + 4 + 16);
+}
 constexpr int tc_smem_bytes(int nt, int stages, bool lo) {
-  const int raw = 1024 /*align slack*/ + tc_body_bytes(nt, stages, lo) + 256 /*barriers, tmem slot*/ +
-                  nt * (16 + 4 + 16);
-  return raw > tc_min_smem(nt, lo) ? raw : tc_min_smem(nt, lo);
+  return tc_used_smem(nt, stages, lo) > tmem_min_smem(tc_tmem_cols(nt, lo)) ? tc_used_smem(nt, stages, lo)
+                                                                            : tmem_min_smem(tc_tmem_cols(nt, lo));
 }
 // Deepest operand ring of a token tile: a 256-token two-term stage holds 80 KB, so two fit.
 constexpr int tc_max_stages(int nt, bool lo) { return (lo && nt >= 256) ? 2 : (!lo && nt == 128) ? 3 : TC_STAGES; }
 constexpr bool tmem_fits(int nt, bool lo) {
-  return (SM_SMEM / (tc_smem_bytes(nt, 1, lo) + 1024)) * tc_tmem_cols(nt, lo) <= 512 &&
-         tc_smem_bytes(nt, tc_max_stages(nt, lo), lo) <= SM_SMEM - 1024;
+  return tc_smem_bytes(nt, 1, lo) >= MIN_TMEM_SMEM && (SM_SHARED / (tc_smem_bytes(nt, 1, lo) + CTA_SHARED)) * tc_tmem_cols(nt, lo) <= 512 &&
+         tc_smem_bytes(nt, tc_max_stages(nt, lo), lo) <= SM_SMEM;
 }
 static_assert(tmem_fits(16, false) && tmem_fits(32, false) && tmem_fits(64, false) && tmem_fits(128, false) &&
                   tmem_fits(256, false) && tmem_fits(16, true) && tmem_fits(32, true) && tmem_fits(64, true) &&
@@ -633,7 +631,9 @@ int gemm_tc_stages(int K, int splits, int nt, bool lo, int cap) {
   return per_cta < 1 ? 1 : (per_cta > cap ? cap : per_cta);
 }
 
-int gemm_tc_per_sm(int nt, int stages, bool lo) { return std::min(16, SM_SMEM / (tc_smem_bytes(nt, stages, lo) + 1024)); }
+int gemm_tc_per_sm(int nt, int stages, bool lo) {
+  return std::min({16, 512 / tc_tmem_cols(nt, lo), SM_SMEM / (tc_used_smem(nt, stages, lo) + CTA_SHARED)});
+}
 
 template <int NT, bool LO>
 static void launch_tc_nt(const CUtensorMap* mapW, const CUtensorMap* mapX, GemmArgs a, cudaStream_t st) {

@@ -43,8 +43,9 @@ struct PgShape {
   static constexpr int OFF_STG = NS * ST_BYTES;
   static constexpr int OFF_BAR = OFF_STG + PG_EPI_WARPS * PG_STAGE_TILE;
   static constexpr int NBAR = 2 * NS + 4;
-  static constexpr int BYTES = OFF_BAR + NBAR * 8 + 16 + 1024;
   static constexpr uint32_t TMEM_COLS = 2 * BN;
+  static constexpr int USED = OFF_BAR + NBAR * 8 + 16 + 1024;
+  static constexpr int BYTES = USED > tmem_min_smem(TMEM_COLS) ? USED : tmem_min_smem(TMEM_COLS);
 };
 
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, int32_t c0, int32_t c1,

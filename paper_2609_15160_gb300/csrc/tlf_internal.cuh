@@ -234,6 +234,17 @@ __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
+// tcgen05.alloc blocks until an SM has the columns, and the CTAs of a cluster that holds some on one SM may wait for a
+// partner that is refused them on another: kernels on different streams could end up waiting for each other. So every
+// GEMM asks for shared memory in proportion to its columns (at least 32, a power of two), so much that CTAs which hold
+// all 512 between them leave less of an SM's 228 KB (1 KB of it reserved for each CTA) than the MIN_TMEM_SMEM that every
+// kernel with tensor memory asks for. CTAs that fit an SM together then always find their columns: more than 512, without
+// a CTA of 32 columns, would be at least 576 and need 234 KB; with one, the others' 512 leave it no room.
+constexpr int SM_SHARED = 233472, CTA_SHARED = 1024, MIN_TMEM_SMEM = 20000;
+constexpr int TMEM_COL_SMEM = (SM_SHARED - CTA_SHARED - MIN_TMEM_SMEM) / 512 + 1;  // of a column
+static_assert(512 * TMEM_COL_SMEM + CTA_SHARED + MIN_TMEM_SMEM > SM_SHARED && 576 * TMEM_COL_SMEM > SM_SHARED, "");
+constexpr int tmem_min_smem(int cols) { return cols * TMEM_COL_SMEM - CTA_SHARED; }
+
 // D(tmem) (+)= A(smem desc) * B(smem desc), kind::f16 (bf16 inputs, f32 accumulate).
 __device__ __forceinline__ void tc_mma_f16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                            uint32_t accumulate) {
