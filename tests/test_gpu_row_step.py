@@ -1,5 +1,5 @@
 """Small float32 models run a step's block one CTA per row: against the oracle around its edges, and against the
-launch-per-stage path (which profiled steps keep)."""
+launch-per-stage path (which profiled steps keep), with as many launches as each of them has."""
 import numpy as np
 import pytest
 
@@ -23,6 +23,11 @@ def test_row_steps_match_oracle(tlf, shape, lens):  # noqa: F811
     _prefill_decode_compare(tlf, _small("f32", **shape), lens, steps=2)
 
 
+def test_more_rows_than_sms(tlf):  # noqa: F811
+    """One CTA per row in more than one wave."""
+    _prefill_decode_compare(tlf, _small("f32", **SHAPES[0]), [1 + b % 3 for b in range(170)], steps=1)
+
+
 def test_long_caches_leave_the_row_kernel(tlf):  # noqa: F811
     """Steps across the longest cache that the row kernel takes (1024 entries) agree with profiled ones."""
     m = _small("f32", **SHAPES[0])
@@ -35,9 +40,11 @@ def test_long_caches_leave_the_row_kernel(tlf):  # noqa: F811
             snap = synth.make_cache_snapshot(m, n, seed=3 + i)
             a.load_cache(i, snap)
             b.load_cache(i, snap)
-        for _ in range(6):
+        for step in range(6):
             toks = rng.integers(0, m.vocab, size=2).astype(np.int32)
             la, ma, _ = a.decode_step([0, 1], toks)
             lb, mb, _ = b.decode_step([0, 1], toks)
             np.testing.assert_array_equal(ma, mb)
+            by_rows = a.last_step_profile()[2] == 4  # router, plan, block, LM head
+            assert by_rows == (1021 + step + 1 <= 1024)
             assert rel_err(la, lb) < 1e-5  # float32 sums in another order
