@@ -464,6 +464,7 @@ __global__ void __launch_bounds__(AttnShape<T, HD, G>::THREADS, attn_ctas_per_sm
       ++g;
     }
   }
+  if (*abort_flag) drain_copies();
 }
 
 template <typename T, int HD, int G, bool MASKED>

@@ -474,7 +474,10 @@ __global__ void __launch_bounds__(tc_threads(NT, LO)) k_gemm_tc(const __grid_con
     for (int i = pre; i < nk; ++i) {
       const int st = i % NS;
       const uint32_t ph = (uint32_t)(i / NS) & 1u;
-      if (!mbar_wait(empty(st), ph ^ 1u, a.err)) break;
+      if (!mbar_wait(empty(st), ph ^ 1u, a.err)) {
+        drain_copies();
+        break;
+      }
       mbar_arrive_expect_tx(full(st), A_BYTES + B_BYTES);
       const int kx = (kb0 + i) * TC_BK;
       tma_load_2d_hint(smem_u32(sA + st * A_BYTES), &mapW, kx, m0, full(st), w_policy);
@@ -529,7 +532,10 @@ __global__ void __launch_bounds__(tc_threads(NT, LO)) k_gemm_tc(const __grid_con
       for (int i = 0; i < nk; ++i) {
         const int st = i % NS;
         const uint32_t ph = (uint32_t)(i / NS) & 1u;
-        if (!mbar_wait(full(st), ph, a.err)) break;
+        if (!mbar_wait(full(st), ph, a.err)) {
+          drain_copies();
+          break;
+        }
         tc_fence_after();
         const uint64_t da = smem_desc_sw128(smem_u32(sA + st * A_BYTES));
         const uint64_t db = smem_desc_sw128(smem_u32(sB + st * B_BYTES));
@@ -574,6 +580,7 @@ __global__ void __launch_bounds__(tc_threads(NT, LO)) k_gemm_tc(const __grid_con
   bool ok = true;
   if (nk > 0) ok = mbar_wait(done, 0, a.err);
   ok = __all_sync(0xffffffffu, ok);  // tcgen05.ld is warp-collective
+  if (!ok) drain_copies();
   tc_fence_after();
   if (a.epi >= EPI_CL_RESID) {
     // Stage the partial tile in shared memory (the operand ring is free now),

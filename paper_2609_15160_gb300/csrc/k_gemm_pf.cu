@@ -469,6 +469,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
       if (lane == 0) mbar_arrive_cluster(dsmem_map(tempty(b), 0));
     }
   }
+  if (*abort_flag) drain_copies();
   tc_fence_before();
   __syncthreads();
   cluster_sync_all();  // neither CTA leaves while the pair's MMAs, copies or arrivals may touch it

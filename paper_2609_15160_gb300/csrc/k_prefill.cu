@@ -373,7 +373,14 @@ __global__ void __launch_bounds__(PFT_THREADS) k_pf_attn_tc(ModelDims md, Prefil
   const uint32_t t_row = tmem + ((uint32_t)(quad * 32) << 16);  // this warp's 32 TMEM lanes
   constexpr uint32_t OCOL = 128;                                 // first TMEM column of O
 
+  bool dead = false;  // a wait of this thread ran out: it waits for nothing more
+  auto wait = [&](uint32_t bar, uint32_t parity) {
+    if (dead || mbar_wait(bar, parity, s.err)) return;
+    dead = true;
+    drain_copies();
+  };
   auto stage_page = [&](int pg) {  // thread 0: K and V segments of page pg into staging buffer pg & 1
+    if (dead) return;
     const uint32_t bar = (pg & 1) ? stg1 : stg0;
     const int page = ptab[pg];
     if (page < 0 || page >= md.n_pages) {
@@ -391,7 +398,7 @@ __global__ void __launch_bounds__(PFT_THREADS) k_pf_attn_tc(ModelDims md, Prefil
   };
   // K tile of page pg (from its staging buffer) into K buffer pg & 1; rows = keys
   auto relayout_k = [&](int pg) {
-    mbar_wait((pg & 1) ? stg1 : stg0, (pg >> 1) & 1, s.err);
+    wait((pg & 1) ? stg1 : stg0, (pg >> 1) & 1);
     const uint8_t* raw = sm + Sh::OFF_RAW + (pg & 1) * Sh::RAW_BYTES;
     uint8_t* bk = sm + Sh::OFF_BK + (pg & 1) * Sh::BK_BYTES;
     const int valid = min(64, last + 1 - pg * 64);
@@ -490,7 +497,7 @@ __global__ void __launch_bounds__(PFT_THREADS) k_pf_attn_tc(ModelDims md, Prefil
     // operand tiles of page pg+1: its K buffer was last read by S of page pg-1 (complete), its V^T
     // buffer by P V of page pg-1, which also frees P and lets O be rescaled
     if (more) relayout_k(pg + 1);
-    if (pg > 0) mbar_wait(bar_o, (pg - 1) & 1, s.err);
+    if (pg > 0) wait(bar_o, (pg - 1) & 1);
     if (more) relayout_v(pg + 1);
     fence_proxy_async_smem();
     __syncthreads();
@@ -499,7 +506,7 @@ __global__ void __launch_bounds__(PFT_THREADS) k_pf_attn_tc(ModelDims md, Prefil
       issue_s(pg + 1);
     }
     __syncwarp();
-    mbar_wait((pg & 1) ? bar_s1 : bar_s0, (pg >> 1) & 1, s.err);
+    wait((pg & 1) ? bar_s1 : bar_s0, (pg >> 1) & 1);
     tc_fence_after();
 
     // this thread's 32 columns of the row
@@ -575,7 +582,7 @@ __global__ void __launch_bounds__(PFT_THREADS) k_pf_attn_tc(ModelDims md, Prefil
     }
     __syncwarp();
   }
-  mbar_wait(bar_o, (npages - 1) & 1, s.err);
+  wait(bar_o, (npages - 1) & 1);
   tc_fence_after();
   xch[half * 128 + row] = l_run;  // the two halves of each row sum
   __syncthreads();
@@ -989,6 +996,7 @@ __global__ void __launch_bounds__(PFA_THREADS, 1) k_pf_attn_pair(ModelDims md, P
       }
     }
   }
+  if (*abort_flag) drain_copies();
   tc_fence_before();
   __syncthreads();
   if (warp == 9) tmem_dealloc(tmem, 512);

@@ -492,7 +492,7 @@ __global__ void __launch_bounds__(SS_THREADS, 1) k_step_small(SmallStep a) {
         const int Kn = ph == 1 ? ff : ph == 3 ? q_dim : d;
         if (tid == 0 && Tn > 0) mbar_arrive_expect_tx(wide ? wbar1 : wbar2, (uint32_t)(Tn * 16 * Kn));
         __syncthreads();  // partial sums in, weights read
-        if (Tn > 0 && ph > 0) {
+        if (Tn > 0 && ph > 0 && !*abort_flag) {
           const SmallLayer& Ln = a.layer[ph == 1 ? j : jn];
           ss_fetch(ph == 2 ? 0 : 2, md, ph == 1 ? Ln.wd : ph == 2 ? Ln.wqkv : Ln.wo, Kn, ph == 2 ? uq : uo, Tn,
                    wide ? w1 : w2, wide ? wbar1 : wbar2, wi, lane);
@@ -560,7 +560,7 @@ __global__ void __launch_bounds__(SS_THREADS, 1) k_step_small(SmallStep a) {
 
         // ---- attention: the group's share of the pages, after the QKV projection ----
         grid_sync(true);
-        ss_fetch(1, md, a.layer[j].wgu, d, ug, tg, w1, wbar1, wi, lane);  // (its space held the partial sums till now)
+        if (!*abort_flag) ss_fetch(1, md, a.layer[j].wgu, d, ug, tg, w1, wbar1, wi, lane);  // (its space held the partial sums till now)
         if (p0 >= total) continue;
         int k = k0, h = h0, g = g0;
         if (w8 == 0) {
@@ -728,6 +728,7 @@ __global__ void __launch_bounds__(SS_THREADS, 1) k_step_small(SmallStep a) {
     }
     __syncthreads();  // rowmeta is rewritten for the next loop
   }
+  if (*abort_flag) drain_copies();
 }
 
 // Shared memory of the kernel's parts for a model on a grid of `ctas` CTAs: fills the byte counts and ring depth of

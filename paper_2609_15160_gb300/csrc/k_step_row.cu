@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(SR_THREADS, 1) k_step_row(RowStep a) {
     }
   }
   __syncthreads();
-  if (a.weights_in_smem) mbar_wait(smem_u32(&wbar), 0, s.err);
+  if (a.weights_in_smem && !mbar_wait(smem_u32(&wbar), 0, s.err)) drain_copies();
 
   // every warp takes the row's RMSNorm factor for itself
   auto norm_factor = [&]() {

@@ -146,6 +146,12 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_
   }
 }
 
+// For a kernel one of whose waits ran out: time (2 ms, some thousand times a copy's) for the copies and MMAs it has in
+// flight to land before it reuses or leaves its shared memory, where they would hit the next CTA's.
+__device__ __forceinline__ void drain_copies() {
+  for (const uint64_t t0 = globaltimer_ns(); globaltimer_ns() - t0 < 2000000ull;) __nanosleep(1000);
+}
+
 // 1-D bulk copy global -> shared (TMA engine), completing tx bytes on `bar`.
 // dst, src and bytes must be multiples of 16.
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {

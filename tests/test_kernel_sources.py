@@ -32,3 +32,12 @@ def test_dependents_start_only_once_tensor_memory_is_allocated(name):
     alloc = re.search(r"tmem_alloc\w*\(", body).start()
     published = body.index("__syncthreads();", alloc)
     assert published < body.index("pdl_trigger();")
+
+
+COPYING_KERNELS = {name: body for name, body in _kernels() if re.search(r"bulk_g2s|tma_load|ss_fetch", body)}
+
+
+@pytest.mark.parametrize("name", sorted(COPYING_KERNELS))
+def test_a_kernel_whose_wait_ran_out_waits_for_its_copies(name):
+    """Copies in flight when a CTA leaves would land in the next CTA's shared memory."""
+    assert "drain_copies()" in COPYING_KERNELS[name]
