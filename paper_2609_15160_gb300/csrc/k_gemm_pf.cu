@@ -108,22 +108,7 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
   }
 }
 
-__device__ __forceinline__ void tmem_ld_32_issue(uint32_t taddr, uint32_t* r) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,"
-      "%29,%30,%31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-}
 
-__device__ __forceinline__ uint32_t pack2(float a, float b) {  // one packed conversion
-  const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
-  return *reinterpret_cast<const uint32_t*>(&v);
-}
 
 }  // namespace
 
@@ -347,7 +332,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
                 const float gq = __uint_as_float(g[i + 2 * e + h]);
                 y[h] = gq / (1.f + expf(-gq)) * __uint_as_float(w[i + 2 * e + h]);
               }
-              p[e] = pack2(y[0], y[1]);
+              p[e] = pack_bf16(y[0], y[1]);
             }
             *reinterpret_cast<uint4*>(sw + i / 2) = make_uint4(p[0], p[1], p[2], p[3]);
           }
@@ -402,8 +387,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
 #pragma unroll
                 for (int i = 0; i < 16; i += 2) {
                   const float a0 = __bfloat162float(__float2bfloat16_rn(v[i])), a1 = __bfloat162float(__float2bfloat16_rn(v[i + 1]));
-                  sw[at + i / 2] = pack2(a0, a1);
-                  sw[16 + at + i / 2] = pack2(v[i] - a0, v[i + 1] - a1);
+                  sw[at + i / 2] = pack_bf16(a0, a1);
+                  sw[16 + at + i / 2] = pack_bf16(v[i] - a0, v[i + 1] - a1);
                 }
               };
               split(r0, 0);
@@ -439,11 +424,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
               uint32_t* sw = reinterpret_cast<uint32_t*>(srow);
 #pragma unroll
               for (int i = 0; i < 16; i += 8) {
-                *reinterpret_cast<uint4*>(sw + i / 2) = make_uint4(pack2(r0[i], r0[i + 1]), pack2(r0[i + 2], r0[i + 3]),
-                                                                  pack2(r0[i + 4], r0[i + 5]), pack2(r0[i + 6], r0[i + 7]));
+                *reinterpret_cast<uint4*>(sw + i / 2) = make_uint4(pack_bf16(r0[i], r0[i + 1]), pack_bf16(r0[i + 2], r0[i + 3]),
+                                                                  pack_bf16(r0[i + 4], r0[i + 5]), pack_bf16(r0[i + 6], r0[i + 7]));
                 *reinterpret_cast<uint4*>(sw + 8 + i / 2) =
-                    make_uint4(pack2(r1[i], r1[i + 1]), pack2(r1[i + 2], r1[i + 3]), pack2(r1[i + 4], r1[i + 5]),
-                               pack2(r1[i + 6], r1[i + 7]));
+                    make_uint4(pack_bf16(r1[i], r1[i + 1]), pack_bf16(r1[i + 2], r1[i + 3]), pack_bf16(r1[i + 4], r1[i + 5]),
+                               pack_bf16(r1[i + 6], r1[i + 7]));
               }
               __syncwarp();
               const int c = (lane & 3) * 8;

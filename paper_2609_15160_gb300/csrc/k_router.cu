@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(256) k_plan(ModelDims md, StepDev s, int B) {
   // attention merge tickets start at zero every step
   if (blockIdx.x == 0)
     for (int i = b; i < maxB * md.Hkv; i += blockDim.x) s.cnt[i] = 0;
-  if (blockIdx.x == 0 && b < 8 && s.gbar) s.gbar[32 * b] = 0;
+  if (blockIdx.x == 0 && b == 0 && s.gbar) *s.gbar = 0;
   // without the gather (an ablation), every row of the step is listed at every loop that runs
   const bool all_rows = md.ablation == TLF_ABLATION_NO_GATHER;
   const bool dense = md.ablation == TLF_ABLATION_DENSE_CACHE;

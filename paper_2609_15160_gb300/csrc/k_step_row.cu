@@ -27,13 +27,12 @@ static __host__ __device__ int sr_outputs(const ModelDims& md) {
   const int n = md.qkv_dim > 2 * md.ff ? md.qkv_dim : 2 * md.ff;
   return n > md.d ? n : md.d;
 }
-static __host__ __device__ SrLayout sr_layout(const ModelDims& md, int max_keys) {
+static __host__ __device__ SrLayout sr_layout(const ModelDims& md) {
   SrLayout l;
   // h, a projection's outputs, o, u; partial value sums; score rows
   const int part = SR_THREADS > md.q_dim ? SR_THREADS : md.q_dim;
   l.scores = (md.d + sr_outputs(md) + md.q_dim + md.ff + part + md.Hq + 3) / 4 * 4;
-  l.total_act = l.scores + md.Hq * max_keys;
-  l.total_act = (l.total_act + 3) / 4 * 4;
+  l.total_act = l.scores + md.Hq * RowStep::MAX_KEYS;
   l.weights = md.J * (md.qkv_dim * md.d + md.d * md.q_dim + 3 * md.ff * md.d + 2 * md.d);  // matrices, norm gains
   return l;
 }
@@ -83,14 +82,14 @@ __global__ void __launch_bounds__(SR_THREADS, 1) k_step_row(RowStep a) {
   const StepDev& s = a.s;
   const int d = md.d, hd = md.hd, q_dim = md.q_dim, qkv_dim = md.qkv_dim, ff = md.ff, M = md.M, J = md.J, Hq = md.Hq;
   const int G = Hq / md.Hkv, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const SrLayout lay = sr_layout(md, a.max_keys);
+  const SrLayout lay = sr_layout(md);
   float* h = smf;                 // [d] residual stream of the row
   float* y = h + d;               // a projection's outputs; QKV's become the rotated q (scaled)
   float* o = y + sr_outputs(md);  // [q_dim] attention output
   float* u = o + q_dim;           // [ff]
   float* part = u + ff;           // partial value sums
   float* lsum = part + (SR_THREADS > q_dim ? SR_THREADS : q_dim);  // [Hq] softmax sums
-  float* sc = smf + lay.scores;   // [Hq][max_keys]
+  float* sc = smf + lay.scores;   // [Hq][MAX_KEYS]
   float* wsm = smf + lay.total_act;
   const size_t per_layer = (size_t)lay.weights / J;
   const size_t nq = (size_t)qkv_dim * d, no = (size_t)d * q_dim, ng = (size_t)2 * ff * d, nd = (size_t)d * ff;
@@ -119,7 +118,7 @@ __global__ void __launch_bounds__(SR_THREADS, 1) k_step_row(RowStep a) {
   if (tid < m) {
     const int k = s.col[tid * md.max_batch + b];  // the row's place in A_r
     info_s[tid] = s.rowinfo[tid * md.max_batch + k];
-    keys_s[tid] = min(s.nch[tid * md.max_batch + k], a.max_keys);
+    keys_s[tid] = min(s.nch[tid * md.max_batch + k], RowStep::MAX_KEYS);
   }
   for (int i = tid; i < m * (RowStep::MAX_KEYS / 64); i += SR_THREADS) {
     const int r = i / (RowStep::MAX_KEYS / 64), p = i % (RowStep::MAX_KEYS / 64);
@@ -216,11 +215,11 @@ __global__ void __launch_bounds__(SR_THREADS, 1) k_step_row(RowStep a) {
           const float4 x = kp[c], y = qp[c];
           acc = fmaf(x.x, y.x, fmaf(x.y, y.y, fmaf(x.z, y.z, fmaf(x.w, y.w, acc))));
         }
-        sc[hh * a.max_keys + key] = acc;
+        sc[hh * RowStep::MAX_KEYS + key] = acc;
       }
       __syncthreads();
       for (int hh = warp; hh < Hq; hh += SR_THREADS / 32) {
-        float* row = sc + hh * a.max_keys;
+        float* row = sc + hh * RowStep::MAX_KEYS;
         float mx = -INFINITY;
         for (int i = lane; i < L; i += 32) mx = fmaxf(mx, row[i]);
         mx = warp_max(mx);
@@ -236,7 +235,7 @@ __global__ void __launch_bounds__(SR_THREADS, 1) k_step_row(RowStep a) {
       __syncthreads();
       for (int t = tid; t < splits * q_dim; t += SR_THREADS) {
         const int sp = t / q_dim, f = t - sp * q_dim, hh = f / hd;
-        const float* row = sc + hh * a.max_keys;
+        const float* row = sc + hh * RowStep::MAX_KEYS;
         const float* vb = pool + ((size_t)(j * 2 + 1) * md.Hkv + hh / G) * 64 * hd + f % hd;
         float acc = 0.f;
         int key = sp;
@@ -288,28 +287,18 @@ __global__ void __launch_bounds__(SR_THREADS, 1) k_step_row(RowStep a) {
 // steps do depends on their caches too).
 bool step_row_fits(const ModelDims& md) {
   if (md.dtype != 0 || md.J > SS_LAYERS || md.d % 4 || md.ff % 4) return false;
-  const SrLayout l = sr_layout(md, RowStep::MAX_KEYS);
+  const SrLayout l = sr_layout(md);
   return (long long)l.weights / md.J * 4 <= (1 << 20) && (long long)l.total_act * 4 <= SR_SMEM && md.d <= SR_THREADS;
 }
 
 long long step_row_weight_bytes(const ModelDims& md) {
-  const SrLayout l = sr_layout(md, RowStep::MAX_KEYS);
+  const SrLayout l = sr_layout(md);
   return (long long)(l.total_act + l.weights) * 4 <= SR_SMEM ? 0 : (long long)l.weights / md.J * 4;
 }
 
 cudaError_t launch_step_row(RowStep a, int B, cudaStream_t st) {
-  a.max_keys = RowStep::MAX_KEYS;
-  SrLayout l = sr_layout(a.md, a.max_keys);
-  // shorter score rows where that lets the weights in
-  for (int keys = a.max_keys; keys >= a.keys; keys /= 2) {
-    const SrLayout t = sr_layout(a.md, keys);
-    if ((long long)(t.total_act + t.weights) * 4 <= SR_SMEM) {
-      a.max_keys = keys;
-      l = t;
-      a.weights_in_smem = 1;
-      break;
-    }
-  }
+  const SrLayout l = sr_layout(a.md);
+  a.weights_in_smem = (long long)(l.total_act + l.weights) * 4 <= SR_SMEM;
   const int smem = (l.total_act + (a.weights_in_smem ? l.weights : 0)) * 4;
   (void)ensure_kernel_attrs((const void*)k_step_row, SR_SMEM);  // a failure shows at launch
   return launch_k(k_step_row, dim3(B), dim3(SR_THREADS), smem, st, a);

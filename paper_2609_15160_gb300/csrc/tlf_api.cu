@@ -653,8 +653,8 @@ static int create_impl(tlf_ctx* ctx, const tlf_weights* w) {
     if ((rc = dev_alloc(ctx, &ctx->d_part_small, step_small_part_floats(md, ctx->num_sms) * 4, "attention partials")))
       return rc;
     if ((rc = dev_alloc(ctx, &ctx->d_ss8, (size_t)16 * (d / 8) * 4, "norm partial sums"))) return rc;
-    if ((rc = dev_alloc(ctx, &ctx->d_gbar, 8 * 128, "grid barrier"))) return rc;
-    CK(ctx, cudaMemset(ctx->d_gbar, 0, 8 * 128));
+    if ((rc = dev_alloc(ctx, &ctx->d_gbar, sizeof(unsigned), "grid barrier"))) return rc;
+    CK(ctx, cudaMemset(ctx->d_gbar, 0, sizeof(unsigned)));
   }
   CK(ctx, cudaMemset(ctx->d_attn_cnt, 0, (size_t)B * md.Hkv * 4));
   if ((rc = dev_alloc(ctx, &ctx->d_logits, (size_t)B * V * 4, "logits"))) return rc;
@@ -908,7 +908,6 @@ static int enqueue_step(tlf_ctx* ctx, int B, bool need_logits, StepPath path, bo
     a.cond = ctx->d_cond;
     a.final_norm = ctx->d_final_norm;
     a.Xf = reinterpret_cast<float*>(ctx->d_Xf);
-    a.keys = RowStep::MAX_KEYS;
     CK(ctx, launch_step_row(a, B, st));
     ctx->last_launches += 1;
   }

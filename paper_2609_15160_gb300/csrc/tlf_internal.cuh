@@ -67,6 +67,11 @@ template <typename T> __device__ __forceinline__ T from_f32(float x);
 template <> __device__ __forceinline__ float from_f32<float>(float x) { return x; }
 template <> __device__ __forceinline__ bf16 from_f32<bf16>(float x) { return __float2bfloat16_rn(x); }
 
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {  // one packed conversion
+  const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+
 // 16 bytes of T widened to float: 4 floats or 8 bf16.
 template <typename T> struct Vec16;
 template <> struct Vec16<float> {
@@ -167,11 +172,6 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t
 __device__ __forceinline__ uint64_t l2_policy_evict_first() {
   uint64_t p;
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
-__device__ __forceinline__ uint64_t l2_policy_evict_normal() {
-  uint64_t p;
-  asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
   return p;
 }
 
@@ -355,9 +355,9 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
 // The same with B MN-major (bit 16).
 __host__ __device__ constexpr uint32_t idesc_bf16_f32_bmn(int M, int N) { return idesc_bf16_f32(M, N) | (1u << 16); }
 
-// 32 lanes x 32-bit, 32 consecutive columns per thread (one wait).
-__device__ __forceinline__ void tmem_ld_32(uint32_t taddr, float* v) {
-  uint32_t r[32];
+
+// 32 lanes x 32-bit, 32 consecutive columns per thread; the registers may be read after tmem_ld_wait().
+__device__ __forceinline__ void tmem_ld_32_issue(uint32_t taddr, uint32_t* r) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
       "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,"
@@ -367,7 +367,11 @@ __device__ __forceinline__ void tmem_ld_32(uint32_t taddr, float* v) {
         "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
         "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_ld_32(uint32_t taddr, float* v) {
+  uint32_t r[32];
+  tmem_ld_32_issue(taddr, r);
+  tmem_ld_wait();
 #pragma unroll
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
@@ -458,7 +462,7 @@ struct StepDev {
   int* pos_table;      // [n_pages][page_size]
   void* pool;          // KV pages
   uint32_t* err;
-  unsigned* gbar;      // grid-barrier counters of the persistent step kernel, 8 x 128 bytes (zeroed by the plan kernel; NULL: none)
+  unsigned* gbar;      // grid-barrier counter of the persistent step kernel (zeroed by the plan kernel; NULL: none)
 };
 
 struct ModelDims {
@@ -583,8 +587,7 @@ struct RowStep {
   const float* cond;        // conditioning table (NULL: none)
   const float* final_norm;
   float* Xf;                // [B][d] the LM head's operand
-  int keys;                 // at least the longest cache of the step, the new entry included
-  int max_keys, weights_in_smem;  // set by the launcher
+  int weights_in_smem;      // set by the launcher
 };
 bool step_row_fits(const ModelDims& md);
 long long step_row_weight_bytes(const ModelDims& md);  // of a layer, read through L2 (0: all staged in shared memory)
