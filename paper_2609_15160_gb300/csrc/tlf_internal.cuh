@@ -152,8 +152,9 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_
 }
 
 // For a kernel one of whose waits ran out: time (2 ms, some thousand times a copy's) for the copies and MMAs it has in
-// flight to land before it reuses or leaves its shared memory, where they would hit the next CTA's.
-__device__ __forceinline__ void drain_copies() {
+// flight to land before it reuses or leaves its shared memory, where they would hit the next CTA's. Not inlined: its code
+// in the way of k_gemm_tc's roles cost 1 to 3 % of a step (128 rows of the mid-size model: 1696 us, and 1643 us so).
+static __device__ __noinline__ void drain_copies() {
   for (const uint64_t t0 = globaltimer_ns(); globaltimer_ns() - t0 < 2000000ull;) __nanosleep(1000);
 }
 
