@@ -86,3 +86,36 @@ def test_many_pages_a_group(tlf, rows, keys):  # noqa: F811
     items lie over several groups (16 kv heads, 304 groups: 34, 65 and 28 pages of the first loop each)."""
     m = _small(head_dim=32, n_heads=16, n_kv_heads=16, n_layers=1, max_loops=2, depth_probs=(0.3, 0.7))
     _pair(tlf, m, [synth.make_cache_positions(m, keys - i, seed=i) for i in range(rows)], steps=2)
+
+
+def test_contexts_step_at_the_same_time(tlf):  # noqa: F811
+    """Two threads, each with a context and a stream of its own, step at once: one through the persistent kernel, which
+    needs every SM, one through it or through the launches. Every step gives what it gives alone."""
+    import threading
+
+    import torch
+    m = _small()
+    w = synth.make_weights(m)
+    steps = 60
+
+    def run(rows, stream, out):
+        toks = np.random.default_rng(rows).integers(0, m.vocab, size=(steps, rows)).astype(np.int32)
+        with tlf.Context(m, w, max_seqs=rows, max_batch=rows, max_seq_len=700) as ctx:
+            for i in range(rows):
+                ctx.load_cache(i, synth.make_cache_snapshot(m, 30 + 29 * (i % 20), seed=i))
+            for t in toks:
+                out.append(ctx.decode_step(list(range(rows)), t, stream=stream)[0].copy())
+
+    for pair in ((4, 16), (4, 40)):
+        alone, both = [[], []], [[], []]
+        for rows, out in zip(pair, alone):
+            run(rows, None, out)
+        streams = [torch.cuda.Stream() for _ in pair]
+        threads = [threading.Thread(target=run, args=(rows, s.cuda_stream, out)) for rows, s, out in zip(pair, streams, both)]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+        for a, b in zip(alone, both):
+            assert len(b) == steps
+            np.testing.assert_array_equal(np.stack(a), np.stack(b))
