@@ -377,11 +377,12 @@ def measure(T, wl, args, rank: int, ws: int, local: int, steps: int, warmup: int
 
     # --- kernel-level pass: attention kernel time and algorithmic KV bytes ---
     ctx.set_profiling(True)
-    att_ms, att_bytes, att_launches = 0.0, 0.0, 0
+    att_ms, att_bytes, att_launches, att_timed = 0.0, 0.0, 0, True
     kernel_ms = {}
     for s in range(steps):
         ctx.decode_step(ids, toks[2 * n_steps + s], forced=forced, logits=logits_dev, stream=stream)
-        ms, by, _ = ctx.last_step_profile()
+        ms, by, nl = ctx.last_step_profile()
+        att_timed = nl * steps == launches  # the timed steps launched the same kernels
         att_ms += ms
         att_bytes += by
         att_launches += m.n_layers * m.max_loops
@@ -398,7 +399,7 @@ def measure(T, wl, args, rank: int, ws: int, local: int, steps: int, warmup: int
     step_bytes = [int(lp.max()) * w_loop + m.vocab * m.d_model * eb + int(lp.sum()) * kv_entry for lp in loops_seen]
     alg_bytes = float(np.mean(step_bytes)) + att_bytes / steps
     r = dict(total_ms=total_ms, e2e_ms=e2e_ms, step_ms=step_ms, att_ms=att_ms, att_bytes=att_bytes,
-             launches=launches, att_launches=att_launches, kernel_ms=kernel_ms, alg_bytes=alg_bytes,
+             launches=launches, att_launches=att_launches, att_timed=att_timed, kernel_ms=kernel_ms, alg_bytes=alg_bytes,
              loops=np.concatenate(loops_seen), margins=np.concatenate(margins), how=how, l2_note=l2_note,
              setup_s=setup_s, clocks=clk,
              prefill=({"tokens": ctx.prefill_tokens, "seconds": ctx.prefill_seconds,
@@ -424,6 +425,8 @@ def summarize(wl, r, steps: int, ws: int, total_ms: float, e2e_ms: float, peak: 
         "step_floor_ms": r["alg_bytes"] / (peak * 1e9) * 1e3,
         "attention_gbs": att_gbs,
         "attention_frac": (att_gbs / peak) if att_gbs else None,
+        "attention_of": "k_attn_decode in a profiled pass, a launch per stage" + (
+            "" if r["att_timed"] else "; the timed steps attend inside one kernel for the block"),
         "mean_loops": float(r["loops"].mean()),
         "depth_histogram": np.bincount(r["loops"], minlength=m.max_loops + 1)[1:].tolist(),
         "near_tie_tokens": near,

@@ -288,7 +288,9 @@ int tlf_load_cache(tlf_ctx* ctx, uint64_t seq_id, const int32_t* lens, const int
  * holds only valid entries, so no mask is needed): for row b and query head
  * h, out[b][h] = softmax(q[b][h] . K_b^T / sqrt(hd)) V_b over the first
  * lens[b] entries of the cache addressed by page_table[b], kv head
- * h / (n_heads / n_kv_heads). The same split-K kernels serve tlf_decode_step.
+ * h / (n_heads / n_kv_heads). tlf_decode_step uses the same kernel where it
+ * launches every stage; steps of up to 16 bf16 rows and of small float32
+ * models attend inside the one kernel that runs their block.
  * All pointers are device pointers. Page layout, in the dtype:
  * [n_pages][n_layers][2 (K, V)][n_kv_heads][page_size][head_dim]; entry e of
  * row b sits in page page_table[b * max_pages + e / page_size] at offset

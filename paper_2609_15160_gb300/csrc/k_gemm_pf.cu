@@ -15,11 +15,12 @@
 // Epilogues: residual add + scatter (vector reductions, one writer per element), RoPE + q out + K/V
 // append, SwiGLU.
 //
-// Tile and split: what bounds a dense projection is operand delivery to the tensor cores. A pair on a 256 x
-// 256 tile reads each operand byte from shared memory half as often as a single-CTA 128 x 256 tile, and
-// with the tokens as M no partial tile is staged for another warp. Measured at 8192 rows, K 2048, 11008
-// features with SwiGLU: 254 us, 1450 TFLOP/s, 0.76 of the measured bf16 rate (454 us with single-CTA tiles of
-// k_gemm_tc, whose epilogue ran between the MMAs); what remains is the last wave and the pipeline's ends.
+// Tile and split: a pair on a 256 x 256 tile reads each operand byte from shared memory half as often as a
+// single-CTA 128 x 256 tile, and with the tokens as M no partial tile is staged for another warp. Measured at 8192
+// rows, K 2048, 11008 features with SwiGLU: 254 us, 1450 TFLOP/s, 0.74 of the measured bf16 rate (454 us with
+// single-CTA tiles of k_gemm_tc, whose epilogue ran between the MMAs). Part of the rest is the last wave (1376 tiles
+// over 76 pairs, 18.1 waves run as 19; 384 tiles, 5.05 waves run as 6, for the mid-size model's QKV) and the pipeline's
+// ends; what holds the full waves is not measured (at the full MMA rate an SM would take 64 bytes a cycle from L2).
 #include <type_traits>
 
 #include "tlf_internal.cuh"

@@ -3,10 +3,11 @@
 // The rows of a step are independent between the router and the LM head, and the block of a small model is a few
 // hundred kilobytes: as launches of their own its stages (norm, QKV, rotary and append, attention, O, norm, gate/up,
 // SwiGLU, down per loop and layer) were all launch latency, 112 us a step for four loops of one layer of width 64; as one
-// launch the step is 62 us (host, router, plan and LM head included). Here a CTA takes its row through every loop the row runs, with the residual and every activation in shared memory and only block
-// barriers between stages, so an exited row costs nothing and no stage of another row is waited for. Weights that fit
-// are staged in shared memory by bulk copies while the router and the plan run; larger ones are read through L2, which
-// pays as long as a layer's weights cross one SM's port in less than its launches took.
+// launch the step is 62 us (host, router, plan and LM head included). Here a CTA takes its row through every loop the row
+// runs, with the residual and every activation in shared memory and only block barriers between stages, so an exited row
+// costs nothing and no stage of another row is waited for. Weights that fit are staged in shared memory by bulk copies
+// while the router and the plan run; larger ones, and K and V, are read through L2, which pays as long as they cross one
+// SM's port in less time than the launches take (step_path in tlf_api.cu).
 //
 // A projection gives each output to a group of lanes (16 for a reduction of up to 64, else a warp), float4 loads and a
 // shuffle reduction; the pre-norm's factor is applied to the sum. Attention: a thread per (head, key) for the scores, a
