@@ -83,6 +83,14 @@ class ClockSampler:
                                           "-lms", "20"], stdout=self.f, stderr=subprocess.DEVNULL)
         except (OSError, FileNotFoundError):
             self.proc = None
+        # nvidia-smi's own start can hold up the driver for a few hundred milliseconds, longer than a short warm-up: a
+        # step of 290 ms among those of 2.9 ms was seen in its way. So it has to be sampling before anything is timed.
+        limit = time.monotonic() + 10
+        while self.proc is not None and self.proc.poll() is None and time.monotonic() < limit:
+            with open(self.path) as f:
+                if len(f.read().splitlines()) > 3:
+                    break
+            time.sleep(0.02)
 
     def stop(self):
         if self.proc is None:
